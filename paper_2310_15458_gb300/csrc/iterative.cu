@@ -307,14 +307,16 @@ __global__ void k_dot_final(const double2* __restrict__ part, int np, double2* _
   if (threadIdx.x == 0) *out = double2{sr[0], si[0]};
 }
 
-// y = alpha x + beta y
+// y = alpha x + beta y; beta = 0 does not read y (scratch that was never written)
 template <typename T>
 __global__ void k_axpby(T* __restrict__ y, const T* __restrict__ x, double ar, double ai, double br, double bi, int64_t n) {
+  const bool set = br == 0.0 && bi == 0.0;
   for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
     if constexpr (sizeof(T) == sizeof(double)) {
-      y[i] = ar * x[i] + br * y[i];
+      y[i] = set ? ar * x[i] : ar * x[i] + br * y[i];
     } else {
-      y[i] = zd{ar, ai} * x[i] + zd{br, bi} * y[i];
+      const zd v = zd{ar, ai} * x[i];
+      y[i] = set ? v : v + zd{br, bi} * y[i];
     }
   }
 }
