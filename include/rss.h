@@ -96,11 +96,15 @@ typedef struct {
                                      Schur update on warp-level MMAs (mma.sync), the same
                                      integer arithmetic and, for real factors, the same
                                      result */
-  int id_cluster;                 /* colour classes with fewer boxes than the GPU has room for:
-                                     0 spreads each box's ID over a thread-block cluster of
-                                     up to 8 CTAs, > 0 sets the largest cluster size (1: one
-                                     CTA per box; at most 16, above 8 a non-portable cluster
-                                     size), -1 is the same as 1 */
+  int id_cluster;                 /* 0: the ID of a real stack (real symmetric kernels; Helmholtz and
+                                     Lippmann-Schwinger, which are complex symmetric; id_rows 0)
+                                     comes from its exact Gram matrix when eps >= 1e-9 and no box of
+                                     the level holds more than 186 points, else from Householder
+                                     reflectors, a box spread over a thread-block cluster of up to 8
+                                     CTAs where its colour class cannot fill the GPU; > 0: reflectors
+                                     with that largest cluster size (1: one CTA per box; at most 16,
+                                     above 8 a non-portable cluster size), -1 is the same as 1.  The
+                                     same pivot rule and stop test either way */
   double bump_cx, bump_cy, bump_a;/* RSS_HELMHOLTZ_LS: b(x) = exp(-bump_a |x - c|^2); bump_a
                                      <= 0 selects the paper's (0.5, 0.5) and 32 */
   int diag_rule;                  /* 0: the diagonal is diag_re + i diag_im; 1: the paper's

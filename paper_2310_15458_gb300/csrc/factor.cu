@@ -2566,6 +2566,8 @@ __global__ void __launch_bounds__(NT) k_schur_oz_c(LevelDev<zd> L, const BoxRec<
     }
 }
 
+#include "id_gram.cuh"
+
 // ------------------------------------------------------------------ merge (Section 2.4)
 template <typename T> __global__ void __launch_bounds__(NT) k_merge_pts(LevelDev<T> C, LevelDev<T> P) {
   const int Pb = blockIdx.x, gp = P.g, px = Pb % gp, py = Pb / gp;
@@ -3232,8 +3234,70 @@ rss_status factor_impl(const rss_tree* tree, const rss_params* prm, cudaStream_t
         }
         return RSS_OK;
       };
+      // the ID from the exact Gram matrix of a real stack: where its fixed-point
+      // error is below the reflectors' (eps >= IDG_EPS) and G fits on chip; a
+      // cluster policy asks for the reflector kernels
+      const bool gram = (half || split) && f->params.eps >= IDG_EPS && prm->id_cluster == 0 && mmax < 65536 &&
+                        idg_chol_bytes(nmax) <= GI_CHOL_SM && idg_tsolve_bytes(nmax) <= GI_CHOL_SM;
+      auto run_gram = [&]() -> rss_status {
+        auto up = [](size_t b) { return (b + 255) & ~size_t(255); };
+        GramWs w;
+        w.nch = (mmax + GI_K - 1) / GI_K;
+        w.ch = ((mmax + w.nch - 1) / w.nch + GI_B - 1) / GI_B * GI_B;
+        w.J = (nmax + GI_B - 1) / GI_B;
+        w.o_part = (size_t)w.nch * (w.ch / GI_B) * OZ_S * w.J * GI_BLK;
+        w.o_R = w.o_part + (size_t)w.nch * w.J * w.J * GI_B * GI_B * sizeof(uint4);
+        w.o_ex = w.o_R + up(sizeof(double) * (nn + nmax));
+        w.o_m = w.o_ex + up(sizeof(int) * (size_t)w.nch * w.J * GI_B);
+        w.slot = w.o_m + 256;
+        const int cap = (int)std::max<size_t>(1, std::min<size_t>({(size_t)nb, (size_t(2) << 30) / w.slot, size_t(32768)}));
+        const int nchunks = (nb + cap - 1) / cap;
+        const int chunk = (nb + nchunks - 1) / nchunks;
+        if (!gb_Y.ensure(w.slot * chunk)) {
+          rss_set_error("rss_factor: device workspace allocation failed");
+          return RSS_ENOMEM;
+        }
+        w.p = static_cast<unsigned char*>(gb_Y.p);
+        f->peak_transient = std::max(f->peak_transient, transient + w.slot * chunk);
+        const size_t smc = idg_chol_bytes(nmax), smt = idg_tsolve_bytes(nmax);
+        RSS_CUDA(cudaFuncSetAttribute(k_idg_gram, cudaFuncAttributeMaxDynamicSharedMemorySize, GI_ST));
+        RSS_CUDA(cudaFuncSetAttribute(k_idg_chol<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smc));
+        RSS_CUDA(cudaFuncSetAttribute(k_idg_tsolve<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smt));
+        IdArgs<double, T> a{};
+        a.L = cur.d;
+        a.boxes = d_cls + seg0;
+        a.half = half;
+        a.k_out = d_k;
+        a.perm_out = d_perm;
+        a.T_ws = d_Tws;
+        a.ixy = d_ixy;
+        a.kp = f->kp;
+        a.geo = f->geo;
+        a.eps = f->params.eps;
+        a.P = P;
+        a.rho = ratio * Lbox;
+        a.Lbox = Lbox;
+        a.ptab = d_ptab;
+        a.lsz = lsz;
+        for (int c0 = 0; c0 < nb; c0 += chunk) {
+          const int cnt = std::min(chunk, nb - c0);
+          a.base = c0;
+          const int ntc = cnt <= 152 ? (nmax > 64 ? 1024 : 512) : nmax > 72 ? 512 : nmax > 32 ? 256 : 128;
+          k_idg_split<T><<<dim3(w.J * (GI_B / 8), w.nch, cnt), 256, 0, st>>>(a, w);
+          RSS_LAUNCHED();
+          k_idg_gram<<<dim3(idg_items(w.J), w.nch, cnt), 256, GI_ST, st>>>(cur.d.n, d_cls + seg0 + c0, w, d_err);
+          RSS_LAUNCHED();
+          k_idg_chol<T><<<cnt, ntc, smc, st>>>(a, w);
+          RSS_LAUNCHED();
+          k_idg_tsolve<T><<<dim3((nmax + 31) / 32, cnt), 128, smt, st>>>(a, w);
+          RSS_LAUNCHED();
+          f->launches += 4;
+          f->n_id += 4;
+        }
+        return RSS_OK;
+      };
       {
-        const rss_status s_id = split ? run_id(double{}) : run_id(T{});
+        const rss_status s_id = gram ? run_gram() : split ? run_id(double{}) : run_id(T{});
         if (s_id != RSS_OK) return s_id;
       }
       evs.back().second->stop(st);
@@ -3518,7 +3582,7 @@ rss_status factor_impl(const rss_tree* tree, const rss_params* prm, cudaStream_t
     int herr = 0;
     RSS_CUDA(cudaMemcpy(&herr, d_err, sizeof(int), cudaMemcpyDeviceToHost));
     if (herr == RSS_ETIMEOUT) {
-      rss_set_error("rss_factor: a tensor-core barrier wait of the Schur update ran out");
+      rss_set_error("rss_factor: a tensor-core barrier wait of the ID or of the Schur update ran out");
       return RSS_ETIMEOUT;
     }
     if (herr) { rss_set_error("rss_factor: zero pivot in the LU of a redundant block"); return RSS_ENUMERIC; }
