@@ -1251,154 +1251,14 @@ template <typename T> __global__ void __launch_bounds__(NT, 4) k_elim_lu(ElimArg
   if (tid == 0) L.nact[B] = k;
 }
 
+#include "elim_split.cuh"
+
 // One panel of 16 MA rows of C.  The rows of A(u, B) (columns of B in pivot
 // order) sit in shared memory as [column][row]; X_CR overwrites the R columns in
 // place, then E = X_CR U^{-1} goes to global memory; the same buffer then takes
 // the columns of A(B, u) for X_RC and F^T = (L^{-1} P_R X_RC)^T.  The right
 // operands (T, U^{-1}, L^{-1}) are staged from global memory in chunks, so any
 // rank fits.
-// On-chip k_elim_lu for boxes whose blocks fit in shared memory (and whose E
-// and F come from the panel kernels): the permuted diagonal block A_BB is
-// staged by cp.async, and X_SR, X_RR, the LU and both triangular inverses stay
-// on chip.  Every phase spreads its work over the whole CTA; U^{-1} and L^{-1}
-// are built by row sweeps (after row i is final it is subtracted from the
-// rows it feeds, one rank-1 update per row).
-template <typename T> __host__ __device__ inline size_t elim_lu_sm_bytes(int k, int r) {
-  const size_t n = (size_t)k + r;
-  const size_t ints = ((n + 2 * (size_t)r) * sizeof(int) + 15) & ~size_t(15);
-  const size_t kr = (size_t)k * r, rr = (size_t)r * r;
-  return ints + sizeof(T) * (n * n + kr + (kr > rr ? kr : rr) + rr + r);
-}
-
-template <typename T> __global__ void __launch_bounds__(NT, 2) k_elim_lu_sm(ElimArgs<T> a) {
-  extern __shared__ __align__(16) unsigned char smraw[];
-  const LevelDev<T>& L = a.L;
-  const BoxRec<T> R = a.recs[blockIdx.x];
-  const int nmax = L.nmax, g = L.g, B = R.box, k = R.k, r = R.r, c = R.c, n = k + r;
-  const size_t nn = (size_t)nmax * nmax;
-  const int* perm_g = a.perm_in + (size_t)a.cls_idx[blockIdx.x] * nmax;
-  const T* Tw = a.T_ws + (size_t)a.cls_idx[blockIdx.x] * nn;
-  const int tid = threadIdx.x, bs = blockDim.x;
-  int* sp = reinterpret_cast<int*>(smraw);   // n: B's points in pivot order
-  int* sperm = sp + n;                      // 2 r: exchange order and its inverse
-  T* Ap = reinterpret_cast<T*>(smraw + (((size_t)(n + 2 * r) * sizeof(int) + 15) & ~size_t(15)));   // n x n
-  T* Ts = Ap + (size_t)n * n;                       // k x r
-  T* Xs = Ts + (size_t)k * r;                       // k x r: X_SR; later U^{-1} (r x r)
-  T* LU = Xs + (size_t)max(k * r, r * r);           // r x r, then r reciprocals of U's diagonal
-  T* Ui = Xs;
-  T* Li = Ap;                                       // r x r, once A_BB is no longer needed
-  __shared__ int nb[9], coff[10], ord[9];
-  if (tid == 0) {
-    const int o9[9] = {4, 0, 1, 2, 3, 5, 6, 7, 8};
-    int off = 0;
-    for (int q = 0; q < 9; ++q) {
-      const int s = o9[q];
-      ord[q] = s;
-      nb[s] = nbr_box(B, g, s % 3 - 1, s / 3 - 1);
-      coff[q] = off;
-      off += s == 4 ? k : (nb[s] >= 0 ? L.nact[nb[s]] : 0);
-    }
-    coff[9] = off;
-  }
-  for (int i = tid; i < n; i += bs) sp[i] = perm_g[i];
-  __syncthreads();
-  const T* Abb = L.blk + ((size_t)B * 25 + 12) * nn;
-  for (int e = tid; e < n * n; e += bs) cp_async_el(Ap + e, Abb + (size_t)sp[e / n] * nmax + sp[e % n]);
-  for (int e = tid; e < k * r; e += bs) cp_async_el(Ts + e, Tw + (size_t)(e / k) * nmax + e % k);
-  for (int i = tid; i < c; i += bs) {
-    int q = 0;
-    while (coff[q + 1] <= i) ++q;
-    const int s = ord[q], ii = i - coff[q], u = nb[s];
-    const int pos = s == 4 ? sp[ii] : L.act[u * nmax + ii];
-    R.cmap[i] = (s << 16) | pos;
-    R.idxC[i] = L.pts[u * nmax + pos];
-  }
-  for (int j = tid; j < r; j += bs) R.idxR[j] = L.pts[B * nmax + sp[k + j]];
-  cp_async_wait_all();
-  __syncthreads();
-  for (int e = tid; e < k * r; e += bs) R.Tm[e] = Ts[e];
-  // X_SR = A_SR - A_SS T
-  for (int e = tid; e < k * r; e += bs) {
-    const int si = e % k, j = e / k;
-    T x = Ap[si + (size_t)(k + j) * n];
-    for (int q = 0; q < k; ++q) x = msb(x, Ap[si + (size_t)q * n], Ts[q + (size_t)j * k]);
-    Xs[e] = x;
-  }
-  __syncthreads();
-  // X_RR = A_RR - A_RS T - T^* X_SR
-  for (int e = tid; e < r * r; e += bs) {
-    const int ai = e % r, bj = e / r;
-    T x = Ap[(k + ai) + (size_t)(k + bj) * n];
-    for (int q = 0; q < k; ++q) x = msb(x, Ap[(k + ai) + (size_t)q * n], Ts[q + (size_t)bj * k]);
-    for (int q = 0; q < k; ++q) x = msbc(x, Ts[q + (size_t)ai * k], Xs[q + (size_t)bj * k]);
-    LU[e] = x;
-  }
-  __syncthreads();
-  if (!lu_pp_block(LU, r, R.piv, a.err)) return;
-  // U^{-1}: rows from the bottom
-  for (int e = tid; e < r * r; e += bs) Ui[e] = (e % r == e / r) ? from_re<T>(1.0) : zero<T>();
-  for (int e = tid; e < r * r; e += bs) Li[e] = (e % r == e / r) ? from_re<T>(1.0) : zero<T>();
-  T* Dr = LU + (size_t)r * r;   // r reciprocals of the diagonal of U, one division each
-  for (int i = tid; i < r; i += bs) Dr[i] = dv(from_re<T>(1.0), LU[i + (size_t)i * r]);
-  __syncthreads();
-  for (int i = r - 1; i >= 0; --i) {
-    const T d = Dr[i];
-    for (int j = i + tid; j < r; j += bs) Ui[i + (size_t)j * r] = Ui[i + (size_t)j * r] * d;
-    __syncthreads();
-    const int w = r - i;
-    for (int e = tid; e < i * w; e += bs) {
-      const int l = e % i, j = i + e / i;
-      Ui[l + (size_t)j * r] = msb(Ui[l + (size_t)j * r], LU[l + (size_t)i * r], Ui[i + (size_t)j * r]);
-    }
-    __syncthreads();
-  }
-  // L^{-1} (unit lower): rows from the top
-  for (int i = 0; i < r - 1; ++i) {
-    const int below = r - 1 - i;
-    for (int e = tid; e < below * (i + 1); e += bs) {
-      const int l = i + 1 + e % below, j = e / below;
-      Li[l + (size_t)j * r] = msb(Li[l + (size_t)j * r], LU[l + (size_t)i * r], Li[i + (size_t)j * r]);
-    }
-    __syncthreads();
-  }
-  if (tid == 0) {   // exchange order sig (P v = v[sig]) and its inverse
-    for (int i = 0; i < r; ++i) sperm[i] = i;
-    for (int i = 0; i < r; ++i) {
-      const int p = R.piv[i], t = sperm[i];
-      sperm[i] = sperm[p];
-      sperm[p] = t;
-    }
-    for (int i = 0; i < r; ++i) sperm[r + sperm[i]] = i;
-  }
-  __syncthreads();
-  for (int e = tid; e < r * r; e += bs) {
-    R.LU[e] = LU[e];
-    R.Ui[e] = Ui[e];
-    R.Li[e] = Li[e];
-    R.LiP[e] = Li[e % r + (size_t)sperm[r + e / r] * r];
-  }
-  if (R.ozp) {   // W_E and W_F, as in k_elim_lu
-    for (int e = tid; e < n * r; e += bs) {
-      const int l = e % n, j = e / n;
-      T we, wf;
-      if (l < k) {
-        we = zero<T>();
-        for (int m = 0; m <= j; ++m) we = msb(we, Ts[l + (size_t)m * k], Ui[m + (size_t)j * r]);
-        wf = zero<T>();
-        for (int m = 0; m < r; ++m) wf = msb(wf, Li[j + (size_t)sperm[r + m] * r], cj(Ts[l + (size_t)m * k]));
-      } else {
-        we = l - k <= j ? Ui[(l - k) + (size_t)j * r] : zero<T>();
-        wf = Li[j + (size_t)sperm[r + l - k] * r];
-      }
-      R.We[e] = we;
-      R.Wf[e] = wf;
-    }
-  }
-  // B keeps only its skeleton
-  for (int q = tid; q < k; q += bs) L.act[B * nmax + q] = sp[q];
-  if (tid == 0) L.nact[B] = k;
-}
-
 template <typename T, int MA, int NBMAX>
 __device__ void elim_panel_body(const ElimArgs<T>& a, const BoxRec<T>& R, unsigned char* smraw, int p0, int rows) {
   constexpr int EPR = 16 * MA;
@@ -1494,18 +1354,17 @@ template <typename T, int MA> __global__ void __launch_bounds__(NT, 2) k_elim_pa
 
 
 // Real factors: the columns of W_E and W_F cut into digit slices once per box
-// (every panel CTA of the box reads them).  One CTA per box, eight threads per
+// (every panel CTA of the box reads them).  32 columns per CTA, eight threads per
 // column.
 __global__ void __launch_bounds__(NT) k_w_split(ElimArgs<double> a) {
   const BoxRec<double> R = a.recs[blockIdx.x];
   if (!R.ozp) return;
   const int r = R.r, n = R.k + r, np = (n + 15) & ~15, rp = (r + 31) & ~31;
-  for (int c0 = 0; c0 < 2 * rp; c0 += NT / 8) {
-    const int col = c0 + (int)threadIdx.x / 8, pass = col / rp, j = col % rp;
-    const double* w = (pass ? R.Wf : R.We) + (size_t)j * n;
-    oz_split_vec<8>([&](int l) { return w[l]; }, j < r ? n : 0, np, R.Wsl + (size_t)col * OZ_S * np, np,
-                    &R.Wexp[col], true);
-  }
+  if ((int)blockIdx.y * (NT / 8) >= 2 * rp) return;
+  const int col = (int)blockIdx.y * (NT / 8) + (int)threadIdx.x / 8, pass = col / rp, j = col % rp;
+  const double* w = (pass ? R.Wf : R.We) + (size_t)j * n;
+  oz_split_vec<8>([&](int l) { return w[l]; }, j < r ? n : 0, np, R.Wsl + (size_t)col * OZ_S * np, np, &R.Wexp[col],
+                  true);
 }
 
 // Real factors: E = A_CB W_E and F^T = A_BC^T W_F for one 64-row panel of C,
@@ -3332,6 +3191,7 @@ rss_status factor_impl(const rss_tree* tree, const rss_params* prm, cudaStream_t
         R.Tm = static_cast<T*>(f->arena.get(sizeof(T) * (size_t)k * r));
         R.LU = static_cast<T*>(f->arena.get(sizeof(T) * (size_t)r * r));
         R.piv = static_cast<int*>(f->arena.get(sizeof(int) * r));
+        R.pos = static_cast<int*>(f->arena.get(sizeof(int) * r));
         R.LiP = static_cast<T*>(f->arena.get(sizeof(T) * (size_t)r * r));
         R.Ui = static_cast<T*>(f->arena.get(sizeof(T) * (size_t)r * r));
         R.Li = static_cast<T*>(f->arena.get(sizeof(T) * (size_t)r * r));
@@ -3340,7 +3200,7 @@ rss_status factor_impl(const rss_tree* tree, const rss_params* prm, cudaStream_t
         R.idxR = static_cast<int*>(f->arena.get(sizeof(int) * r));
         R.idxC = static_cast<int*>(f->arena.get(sizeof(int) * c));
         R.cmap = static_cast<int*>(f->arena.get(sizeof(int) * c));
-        if (!R.Tm || !R.LU || !R.piv || !R.LiP || !R.Ui || !R.Li || !R.E || !R.Ft || !R.idxR || !R.idxC ||
+        if (!R.Tm || !R.LU || !R.piv || !R.pos || !R.LiP || !R.Ui || !R.Li || !R.E || !R.Ft || !R.idxR || !R.idxC ||
             !R.cmap) {
           rss_set_error("rss_factor: device arena allocation failed");
           return RSS_ENOMEM;
@@ -3469,19 +3329,41 @@ rss_status factor_impl(const rss_tree* tree, const rss_params* prm, cudaStream_t
           sizeof(T) * ((size_t)max_r * max_r + std::max((size_t)max_k * max_r, (size_t)max_r * max_r)) + ints;
       const size_t ecap = std::min<size_t>(want, 200 * 1024);
       ea.smem_cap = (int)((ecap - ints) / sizeof(T));
-      // the on-chip kernel when every box fits and takes E and F from the panel kernels
-      size_t sm_lu = 0;
-      bool lu_sm = true;
-      for (const BoxRec<T>& R : recs) {
-        sm_lu = std::max(sm_lu, elim_lu_sm_bytes<T>(R.k, R.r));
-        lu_sm = lu_sm && (R.panels || R.ozp);
-      }
-      lu_sm = lu_sm && sm_lu <= 200 * 1024;
       evs.emplace_back(1, std::make_unique<Ev>());
       evs.back().second->start(st);
-      if (lu_sm) {
-        RSS_CUDA(cudaFuncSetAttribute(k_elim_lu_sm<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm_lu));
-        k_elim_lu_sm<T><<<nrec, NT, sm_lu, st>>>(ea);
+      int max_n = 0;
+      bool ef_later = true;   // every box takes E and F from the panel kernels
+      for (const BoxRec<T>& R : recs) {
+        max_n = std::max(max_n, R.k + R.r);
+        ef_later = ef_later && (R.panels || R.ozp);
+      }
+      const size_t xb = std::max(elim_x_bytes<T>(8, max_k, max_n), elim_inv_bytes<T>(16, max_r));
+      if (ef_later && xb <= 200 * 1024) {
+        // columns per CTA: as many as still give every SM two CTAs
+        auto launch_x = [&](auto kern, int jc, size_t smem) -> cudaError_t {
+          cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+          if (e != cudaSuccess) return e;
+          kern<<<dim3((max_r + jc - 1) / jc, nrec), 256, smem, st>>>(ea);
+          return cudaGetLastError();
+        };
+        auto launch_inv = [&](auto kern, int nbc) -> cudaError_t {
+          const size_t smem = elim_inv_bytes<T>(nbc, max_r);
+          cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+          if (e != cudaSuccess) return e;
+          kern<<<dim3((max_r + nbc - 1) / nbc, 2, nrec), 16 * nbc, smem, st>>>(ea);
+          return cudaGetLastError();
+        };
+        const long long groups = (long long)nrec * ((max_r + 15) / 16);
+        RSS_CUDA(groups < 2 * 152 ? launch_x(k_elim_x<T, 2>, 4, elim_x_bytes<T>(2, max_k, max_n))
+                                  : launch_x(k_elim_x<T, 8>, 16, elim_x_bytes<T>(8, max_k, max_n)));
+        const size_t lub = std::min<size_t>(sizeof(T) * (size_t)max_r * (max_r | 1), 224 * 1024) + sizeof(int) * (size_t)max_r;
+        const size_t lus = std::min<size_t>(lub, 224 * 1024);
+        ea.smem_cap = (int)(lus / sizeof(T));
+        RSS_CUDA(cudaFuncSetAttribute(k_elim_lu2<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)lus));
+        k_elim_lu2<T><<<nrec, 256, lus, st>>>(ea);
+        RSS_LAUNCHED();
+        RSS_CUDA(2 * groups < 2 * 152 ? launch_inv(k_elim_inv<T, 8>, 8) : launch_inv(k_elim_inv<T, 16>, 16));
+        f->launches += 2;
       } else {
         RSS_CUDA(cudaFuncSetAttribute(k_elim_lu<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ecap));
         k_elim_lu<T><<<nrec, NT, ecap, st>>>(ea);
@@ -3502,7 +3384,7 @@ rss_status factor_impl(const rss_tree* tree, const rss_params* prm, cudaStream_t
       }
       if constexpr (sizeof(T) == sizeof(double)) {
         if (ozp_np > 0) {
-          k_w_split<<<nrec, NT, 0, st>>>(ea);
+          k_w_split<<<dim3(nrec, 2 * ((max_r + 31) / 32)), NT, 0, st>>>(ea);
           RSS_LAUNCHED();
           const int smem = (64 + OZ_NCH) * (OZ_S * ozp_np + 8) * (int)sizeof(uint16_t);
           RSS_CUDA(cudaFuncSetAttribute(k_elim_oz, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));

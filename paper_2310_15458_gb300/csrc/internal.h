@@ -34,6 +34,7 @@ template <typename T> struct BoxRec {
   T* Tm;        // k x r, ld k
   T* LU;        // r x r packed LU of X_RR, ld r
   int* piv;     // r getrf pivots (0-based)
+  int* pos;     // r: P e_m = e_pos[m] for the exchanges of piv (factor time only)
   T* LiP;       // r x r, ld r: L_R^{-1} P_R (the solve applies it as one product)
   T* Ui;        // r x r, ld r: U_R^{-1}
   T* Li;        // r x r, ld r: L_R^{-1} (unit lower), factor time only
