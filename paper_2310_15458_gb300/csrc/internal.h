@@ -139,8 +139,6 @@ struct rss_factorization {
   std::vector<LevelInfo> levels;
   // top dense block
   int ntop = 0;
-  void* d_top_lu = nullptr;            // ntop x ntop
-  int* d_top_piv = nullptr;
   int* d_top_idx = nullptr;            // tree indices
   void* d_top_inv = nullptr;           // ntop x ntop: A_top^{-1}, applied by the solve
   // slices of E and F for the tensor-core sweeps (real factors), built by the
@@ -166,7 +164,6 @@ template <typename T> rss_status factor_impl(const rss_tree* tree, const rss_par
                                              cudaStream_t st, rss_factorization* f);
 template <typename T> rss_status solve_impl(const rss_factorization* f, T* b_dev, int64_t nrhs,
                                             int64_t ldb, cudaStream_t st);
-template <typename T> rss_status top_inverse(const T* LU, const int* piv, int n, T* Ainv, cudaStream_t st);
 // device bytes one solve of nrhs columns allocates (working copy plus sweep
 // workspace), beside the caller's b
 size_t solve_device_bytes(const rss_factorization* f, int64_t nrhs);

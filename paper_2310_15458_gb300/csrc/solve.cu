@@ -1262,90 +1262,6 @@ __global__ void __launch_bounds__(SW_NT) k_top_gemv(const T* __restrict__ Ainv, 
     if (q < nq) x[idx[i] + (int64_t)(q0 + q) * N] = acc[q];
 }
 
-// Dense top solve, blocked by 32: one warp solves each diagonal block (no
-// block-wide barrier per row), then all threads update the rows below (above).
-template <typename T, int RC>
-__global__ void __launch_bounds__(1024) k_top_solve(const T* __restrict__ LU, const int* __restrict__ piv,
-                                                    const int* __restrict__ idx, int n, T* __restrict__ x,
-                                                    int64_t N, int nrhs) {
-  extern __shared__ __align__(16) unsigned char smraw[];
-  T* z = reinterpret_cast<T*>(smraw);   // n x RC
-  const int q0 = blockIdx.x * RC, nq = min(RC, nrhs - q0);
-  const int tid = threadIdx.x, bs = blockDim.x, lane = tid & 31, warp = tid >> 5;
-  T* xq = x + (int64_t)q0 * N;
-  for (int e = tid; e < n * RC; e += bs) {
-    const int i = e / RC, q = e % RC;
-    z[e] = q < nq ? xq[idx[i] + (int64_t)q * N] : zero<T>();
-  }
-  __syncthreads();
-  if (tid < RC)
-    for (int j = 0; j < n; ++j) {
-      const int p = piv[j];
-      if (p != j) {
-        const T t = z[j * RC + tid];
-        z[j * RC + tid] = z[p * RC + tid];
-        z[p * RC + tid] = t;
-      }
-    }
-  __syncthreads();
-  // forward: unit lower L
-  for (int jb = 0; jb < n; jb += 32) {
-    const int je = min(n, jb + 32);
-    if (warp == 0) {
-      for (int j = jb; j < je; ++j) {
-        const int l = jb + lane;
-        if (l > j && l < je)
-          for (int q = 0; q < RC; ++q) z[l * RC + q] = msb(z[l * RC + q], LU[l + (size_t)j * n], z[j * RC + q]);
-        __syncwarp();
-      }
-    }
-    __syncthreads();
-    for (int e = tid; e < (n - je) * RC; e += bs) {
-      const int l = je + e / RC, q = e % RC;
-      T acc = z[l * RC + q];
-      for (int j = jb; j < je; ++j) acc = msb(acc, LU[l + (size_t)j * n], z[j * RC + q]);
-      z[l * RC + q] = acc;
-    }
-    __syncthreads();
-  }
-  // backward: upper U
-  for (int je = n; je > 0; je -= 32) {
-    const int jb = max(0, je - 32);
-    if (warp == 0) {
-      for (int j = je - 1; j >= jb; --j) {
-        if (lane == 0)
-          for (int q = 0; q < RC; ++q) z[j * RC + q] = dv(z[j * RC + q], LU[j + (size_t)j * n]);
-        __syncwarp();
-        const int l = jb + lane;
-        if (l < j)
-          for (int q = 0; q < RC; ++q) z[l * RC + q] = msb(z[l * RC + q], LU[l + (size_t)j * n], z[j * RC + q]);
-        __syncwarp();
-      }
-    }
-    __syncthreads();
-    for (int e = tid; e < jb * RC; e += bs) {
-      const int l = e / RC, q = e % RC;
-      T acc = z[l * RC + q];
-      for (int j = jb; j < je; ++j) acc = msb(acc, LU[l + (size_t)j * n], z[j * RC + q]);
-      z[l * RC + q] = acc;
-    }
-    __syncthreads();
-  }
-  for (int e = tid; e < n * RC; e += bs) {
-    const int i = e / RC, q = e % RC;
-    if (q < nq) xq[idx[i] + (int64_t)q * N] = z[e];
-  }
-}
-
-__global__ void k_iota(int* v, int n) {
-  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) v[i] = i;
-}
-template <typename T> __global__ void k_identity(T* A, int n) {
-  const long long tot = (long long)n * n;
-  for (long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x; e < tot; e += (long long)gridDim.x * blockDim.x)
-    A[e] = (e % n == e / n) ? from_re<T>(1.0) : zero<T>();
-}
-
 // Workspace of the sweeps for nrhs right-hand sides in chunks of rc columns:
 // the downward sweep's partial sums, one counter per box, the gathered top block.
 // (The persistent sweeps use the same partial-sum region, with 64-row chunks,
@@ -1737,32 +1653,6 @@ rss_status run_sweeps(const rss_factorization* f, T* x, int64_t N, int64_t nrhs,
 }
 
 }  // namespace
-
-// A_top^{-1}, column by column from the LU (identity right-hand sides).
-template <typename T> rss_status top_inverse(const T* LU, const int* piv, int n, T* Ainv, cudaStream_t st) {
-  constexpr int RT = 4;
-  const size_t tsm = sizeof(T) * (size_t)n * RT;
-  if (tsm > 200 * 1024) {
-    rss_set_error("rss_factor: top block too large for the on-chip solve");
-    return RSS_EINVAL;
-  }
-  int* iota = nullptr;
-  RSS_CUDA(pool_malloc(reinterpret_cast<void**>(&iota), sizeof(int) * (size_t)n, st));
-  k_iota<<<cdiv(n, 256), 256, 0, st>>>(iota, n);
-  k_identity<T><<<std::min<long long>(cdiv((long long)n * n, 256), 152LL * 8), 256, 0, st>>>(Ainv, n);
-  RSS_CUDA(cudaFuncSetAttribute(k_top_solve<T, RT>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024));
-  k_top_solve<T, RT><<<cdiv(n, RT), 1024, tsm, st>>>(LU, piv, iota, n, Ainv, n, n);
-  const cudaError_t e = cudaGetLastError();
-  pool_free(iota, st);
-  if (e != cudaSuccess) {
-    rss_set_error(std::string("rss_factor: top inverse launch failed: ") + cudaGetErrorString(e));
-    return RSS_ECUDA;
-  }
-  return RSS_OK;
-}
-
-template rss_status top_inverse<double>(const double*, const int*, int, double*, cudaStream_t);
-template rss_status top_inverse<zd>(const zd*, const int*, int, zd*, cudaStream_t);
 
 template <typename T>
 rss_status solve_impl(const rss_factorization* f, T* b, int64_t nrhs, int64_t ldb, cudaStream_t st) {
