@@ -26,8 +26,8 @@
 // The reflector kernels do 4 m n k FP64 flops a box (two FMAs per clock and SM) and
 // read the stack once per pivot; here the m n^2 part runs on the tensor cores, the
 // rest in 32-bit integer arithmetic, and the stack is read once.  ID phase of a
-// factorization, reflectors before, this after: Laplace 1024^2 132.0 -> 46.9 ms,
-// 256^2 31.3 -> 10.1, 64^2 (eps 1e-8) 15.7 -> 5.3, Helmholtz 256^2 54.6 -> 13.4.
+// factorization, reflectors before, this after: Laplace 1024^2 132.0 -> 42.1 ms,
+// 256^2 31.3 -> 8.1, 64^2 (eps 1e-8) 15.7 -> 4.0, Helmholtz 256^2 54.6 -> 11.1.
 
 constexpr int GI_K = 512;                    // rows of a part
 constexpr int GI_B = 32;                     // rows and columns of a block of digits
@@ -363,14 +363,6 @@ __device__ __forceinline__ U96 u96_shl(U96 a, int s) {   // s >= 0
   return U96{a.x << s, __funnelshift_l(a.x, a.y, s), __funnelshift_l(a.y, a.z, s)};
 }
 __device__ __forceinline__ int u96_clz(U96 a) { return a.z ? __clz(a.z) : a.y ? 32 + __clz(a.y) : 64 + __clz(a.x); }
-// the fraction a / 2^96 to 64 bits, in FP64
-__device__ __forceinline__ double u96_double(U96 a) {
-  const int lz = u96_clz(a);
-  if (lz >= 96) return 0.0;
-  const U96 b = u96_shl(a, lz);
-  const double d = __ull2double_rn(((unsigned long long)b.z << 32) | b.y);   // in [2^63, 2^64]
-  return __longlong_as_double(__double_as_longlong(d) - ((long long)(64 + lz) << 52));
-}
 __device__ __forceinline__ U96 s96_abs(uint32_t x, uint32_t y, uint32_t z, uint32_t* neg) {
   const uint32_t s = (uint32_t)((int)z >> 31);
   x ^= s; y ^= s; z ^= s;
@@ -378,6 +370,47 @@ __device__ __forceinline__ U96 s96_abs(uint32_t x, uint32_t y, uint32_t z, uint3
   const uint32_t xx = x + c0, c1 = xx < c0, yy = y + c1, c2 = yy < c1;
   *neg = s;
   return U96{xx, yy, z + c2};
+}
+
+// g -= v / 2, or g += v / 2 where neg is all ones (g signed, 95 fraction bits)
+__device__ __forceinline__ void s96_sub_half(uint32_t& x, uint32_t& y, uint32_t& z, U96 v, uint32_t neg) {
+  const uint32_t s = ~neg;   // all ones: subtract
+  const uint32_t a0 = __funnelshift_r(v.x, v.y, 1) ^ s, a1 = __funnelshift_r(v.y, v.z, 1) ^ s, a2 = (v.z >> 1) ^ s;
+  asm("{\n.reg .u32 c;\nadd.cc.u32 c, %6, %6;\naddc.cc.u32 %0, %0, %3;\naddc.cc.u32 %1, %1, %4;\naddc.u32 %2, %2, %5;\n}\n"
+      : "+r"(x), "+r"(y), "+r"(z)
+      : "r"(a0), "r"(a1), "r"(a2), "r"(s & 0x80000000u));
+}
+// a / 2^96 2^e2 as the bits of a double, truncated (0 when it would not be normal):
+// integer instructions only, and non-negative doubles order like their bits
+__device__ __forceinline__ unsigned long long u96_dbits(U96 a, int e2) {
+  const int lz = u96_clz(a), f = 1022 - lz + e2;
+  if (lz >= 96 || f <= 0) return 0ull;
+  const U96 b = u96_shl(a, lz);
+  return ((unsigned long long)f << 52) + (((((unsigned long long)b.z << 32) | b.y) << 1) >> 12);
+}
+// 1 / (2 sqrt(v)) in (1/2, 1] as a 96-bit fraction, v a fraction in [1/4, 1): a 22-bit
+// seed, one Newton step in 64 bits (about 43 bits), one third-order step in 96;
+// relative error below 2^-91.  Integer instructions but for the seed: a chain of FP64
+// instructions here costs several times as long, and every pivot waits for it.
+__device__ __forceinline__ U96 u96_rsqrt_half(U96 v) {
+  const float r0 = rsqrtf((float)v.z * 0x1p-32f);
+  const uint32_t R0 = (uint32_t)fminf(r0 * 0x1p31f, 4294967040.0f);
+  const unsigned long long vh = ((unsigned long long)v.z << 32) | v.y;
+  const long long e0 = (1ll << 62) - (long long)__umul64hi(vh, (unsigned long long)R0 * R0);   // (1 - 4 v r^2) 2^62
+  const long long d0 = ((long long)R0 * (e0 >> 12)) >> 19;
+  unsigned long long r1 = ((unsigned long long)R0 << 32) + (unsigned long long)d0;
+  if (d0 > 0 && r1 < (unsigned long long)d0) r1 = ~0ull;
+  const unsigned long long sh = __umul64hi(r1, r1), sl = r1 * r1;
+  const U96 t = u96_mulhi(v, U96{(uint32_t)(sl >> 32), (uint32_t)sh, (uint32_t)(sh >> 32)});
+  // (1 - 4 v r^2) 2^94: t is near 2^94, their difference fits 64 bits
+  const unsigned long long tl = ((unsigned long long)t.y << 32) | t.x;
+  const long long e1 = (long long)(0ull - tl);
+  const long long q = e1 >> 24;
+  const long long x = e1 + (long long)(((unsigned long long)(q * q) * 3ull) >> 48);
+  const __int128 d = ((__int128)(unsigned __int128)r1 * x) >> 63;
+  __int128 r = ((__int128)(unsigned __int128)r1 << 32) + d;
+  if (r >> 96) r = ((__int128)1 << 96) - 1;
+  return U96{(uint32_t)r, (uint32_t)(r >> 32), (uint32_t)(r >> 64)};
 }
 
 // shared memory of k_idg_chol: G (upper triangle, three limb planes), the new
@@ -403,9 +436,8 @@ template <typename S> __global__ void __launch_bounds__(1024, 1) k_idg_chol(IdAr
   int* rem = ex + nmax;              // remaining columns, ascending; two lists
   int* perm = rem + 2 * nmax;
   int* pos = perm + nmax;
-  __shared__ int s_q, s_shift, s_emax;
+  __shared__ int s_q, s_stop, s_shift, s_emax;
   __shared__ U96 s_rinv;
-  __shared__ double s_rkk;
   unsigned char* slot = w.p + (size_t)box * w.slot;
   const int m = *reinterpret_cast<const int*>(slot + w.o_m), nparts = (m + w.ch - 1) / w.ch;
   const int* pex = reinterpret_cast<const int*>(slot + w.o_ex);
@@ -429,13 +461,10 @@ template <typename S> __global__ void __launch_bounds__(1024, 1) k_idg_chol(IdAr
   const int emax = s_emax;
   const int shift = 16 + (m > 1 ? 32 - __clz(m - 1) : 0);   // |G| <= m 2^110 -> |g| <= 1/2 with 95 fraction bits
   auto tidx = [n](int i, int j) { return i * n - i * (i - 1) / 2 - i + j; };   // i <= j
+  // remaining squared norm of column j in the true scale, relative to the largest column's
   auto norm_of = [&](int j, uint32_t x, uint32_t y, uint32_t z) {
-    uint32_t neg;
-    const U96 v = s96_abs(x, y, z, &neg);
-    const double d = u96_double(v);
-    const int e2 = max(2 * (ex[j] - emax), -1000);   // true scale, relative to the largest column's
-    const double t = d * __longlong_as_double((long long)(1023 + e2) << 52);
-    return neg ? -t : t;
+    const int e2 = max(2 * (ex[j] - emax), -2000);
+    return (int)z < 0 ? 0.0 : __longlong_as_double((long long)u96_dbits(U96{x, y, z}, e2));
   };
   // G: the parts under the columns' common scales
   for (int i = warp; i < n; i += nw) {
@@ -461,16 +490,17 @@ template <typename S> __global__ void __launch_bounds__(1024, 1) k_idg_chol(IdAr
     }
   }
   __syncthreads();
-  double thresh = 0.0, y2max = 0.0;   // warp 0
-  if (warp == 0) {
+  // warp 0 picks the pivots, warp 1 runs the stop test
+  double thresh = 0.0;
+  float y2max = 0.0f;
+  if (warp < 2) {
     double s = 0.0, mx = 0.0;
     for (int c = lane; c < n; c += 32) {
       s += norms[c];
       mx = fmax(mx, norms[c]);
     }
-    s = warp_sum(s);
-    y2max = warp_max(mx);
-    thresh = a.eps * a.eps * s;
+    thresh = a.eps * a.eps * warp_sum(s);
+    y2max = (float)warp_max(mx);
   }
   int k = 0;
   const int kmax = emax >= GI_NAN ? 0 : min(m, n);
@@ -478,57 +508,47 @@ template <typename S> __global__ void __launch_bounds__(1024, 1) k_idg_chol(IdAr
     const int nr = n - k;
     const int* rm = rem + (k & 1) * nmax;
     int* rn = rem + ((k + 1) & 1) * nmax;
-    if (warp == 0) {   // stop test and pivot: largest remaining norm, lowest column among ties
-      double s = 0.0, mx = -1.0;
-      for (int b = lane; b < nr; b += 32) {
-        const double v = norms[rm[b]];
-        s += v;
-        mx = fmax(mx, v);
-      }
-      s = warp_sum(s);
-      mx = warp_max(mx);
-      const double thr = mx - (TIE_REL * mx + TIE_ABS * sqrt(mx * y2max));
+    if (warp == 0) {   // pivot: largest remaining norm, lowest column among ties
+      unsigned long long mk = 0;
+      for (int b = lane; b < nr; b += 32) mk = max(mk, (unsigned long long)__double_as_longlong(norms[rm[b]]));
+      const uint32_t hi = __reduce_max_sync(0xffffffffu, (uint32_t)(mk >> 32));
+      const uint32_t lo = __reduce_max_sync(0xffffffffu, (uint32_t)(mk >> 32) == hi ? (uint32_t)mk : 0u);
+      mk = ((unsigned long long)hi << 32) | lo;
+      const double mx = __longlong_as_double((long long)mk);
+      const float mf = (float)mx;
+      // (the window to 24 bits: it is a small part of mx)
+      const double thr = mx - (double)((float)TIE_REL * mf + (float)TIE_ABS * sqrtf(mf * y2max));
+      const unsigned long long tk = thr > 0.0 ? (unsigned long long)__double_as_longlong(thr) : 0ull;
       int q = INT_MAX;
       for (int b = lane; b < nr; b += 32) {
         const int c = rm[b];
-        if (norms[c] >= thr) {
+        if ((unsigned long long)__double_as_longlong(norms[c]) >= tk) {
           q = c;
           break;
         }
       }
-      q = __reduce_min_sync(0xffffffffu, q);
-      const bool stop = s <= thresh || !(mx > 0.0) || q == INT_MAX;
-      if (!stop) {
-        // 1 / sqrt(g_qq): g 2^(2s) in [1/4, 1), FP64 seed, one correction in double-double
+      q = (int)__reduce_min_sync(0xffffffffu, (uint32_t)q);
+      if (mk == 0) q = -1;
+      if (q >= 0) {
         const int t = tidx(q, q);
         const U96 g{g0[t], g1[t], g2[t]};
-        const int sft = (u96_clz(g) - 1) & ~1;
-        const U96 v = u96_shl(g, sft);   // 95 fraction bits
-        const double d2 = (double)v.z * 0x1p-31, d1 = (double)v.y * 0x1p-63, d0 = (double)v.x * 0x1p-95;
-        const double hi = d2 + d1, lo = (d1 - (hi - d2)) + d0;
-        const double r0 = rsqrt(hi);
-        const double p = r0 * r0, pe = fma(r0, r0, -p);
-        const double h = hi * p, he = fma(hi, p, -h) + (hi * pe + lo * p);
-        const double rl = 0.5 * r0 * ((1.0 - h) - he);
-        // r / 2 as a 96-bit fraction
-        __int128 x = ((__int128)(unsigned long long)(r0 * 0x1p52) << 43) + __double2ll_rn(rl * 0x1p95);
-        if (x >> 96) x = ((__int128)1 << 96) - 1;
+        const int sft = (u96_clz(g) - 1) & ~1;   // g 2^sft in [1/4, 1), 95 fraction bits
+        const U96 ri = u96_rsqrt_half(u96_shl(g, sft + 1));
         if (lane == 0) {
-          s_rinv = U96{(uint32_t)x, (uint32_t)(x >> 32), (uint32_t)(x >> 64)};
+          s_rinv = ri;
           s_shift = sft / 2;
-          const int pq = pos[q], ck = perm[k];
-          perm[k] = q;
-          perm[pq] = ck;
-          pos[ck] = pq;
-          pos[q] = k;
-          s_rkk = r0;
         }
       }
-      if (lane == 0) s_q = stop ? -1 : q;
+      if (lane == 0) s_q = q;
+    } else if (warp == 1) {
+      double s = 0.0;
+      for (int b = lane; b < nr; b += 32) s += norms[rm[b]];
+      s = warp_sum(s);
+      if (lane == 0) s_stop = s <= thresh;
     }
     __syncthreads();
     const int q = s_q;
-    if (q < 0) break;
+    if (s_stop || q < 0) break;
     const U96 ri = s_rinv;
     const int sft = s_shift;
     // row k of R: g_qc / sqrt(g_qq) for the remaining columns
@@ -540,12 +560,16 @@ template <typename S> __global__ void __launch_bounds__(1024, 1) k_idg_chol(IdAr
         const U96 v = u96_mulhi(u96_shl(s96_abs(g0[t], g1[t], g2[t], &neg), sft + 1), ri);
         const U96 l = u96_shl(v, 1);
         row[c] = make_uint4(l.x, l.y, l.z, neg);
-        const double d = u96_double(l);
+        const double d = __longlong_as_double((long long)u96_dbits(l, 0));
         R[(size_t)c * nmax + k] = neg ? -d : d;
         rn[b - (c > q)] = c;
       } else {
-        // 1 / R_kk in the units of R (g has 95 fraction bits: its value is r^2, r < 1)
-        rinv[k] = s_rkk * __longlong_as_double((long long)(1023 + sft) << 52);
+        rinv[k] = __longlong_as_double((long long)u96_dbits(ri, sft + 1));   // 1 / R_kk in the units of R
+        const int pq = pos[q], ck = perm[k];
+        perm[k] = q;
+        perm[pq] = ck;
+        pos[ck] = pq;
+        pos[q] = k;
       }
     }
     __syncthreads();
@@ -554,20 +578,21 @@ template <typename S> __global__ void __launch_bounds__(1024, 1) k_idg_chol(IdAr
       const int i = rn[x];
       const uint4 li = row[i];
       const int rs = tidx(i, 0);
-      for (int b = x + lane; b < nr - 1; b += 32) {
-        const int j = rn[b], t = rs + j;
-        const uint4 lj = row[j];
-        const U96 v = u96_mulhi(U96{li.x, li.y, li.z}, U96{lj.x, lj.y, lj.z});
-        // g -= +-(v / 2)
-        const uint32_t s = ~(li.w ^ lj.w);   // all ones: subtract
-        const uint32_t a0 = __funnelshift_r(v.x, v.y, 1) ^ s, a1 = __funnelshift_r(v.y, v.z, 1) ^ s, a2 = (v.z >> 1) ^ s;
-        uint32_t x0, x1, x2;
-        asm("{\n.reg .u32 c;\nadd.cc.u32 c, %9, %9;\naddc.cc.u32 %0, %3, %6;\naddc.cc.u32 %1, %4, %7;\naddc.u32 %2, %5, %8;\n}\n"
-            : "=&r"(x0), "=&r"(x1), "=&r"(x2)
-            : "r"(g0[t]), "r"(g1[t]), "r"(g2[t]), "r"(a0), "r"(a1), "r"(a2), "r"(s & 0x80000000u));
+      for (int b = x + lane; b < nr - 1; b += 64) {   // two columns in flight
+        const bool two = b + 32 < nr - 1;
+        const int j = rn[b], t = rs + j, j2 = two ? rn[b + 32] : j, t2 = rs + j2;
+        const uint4 lj = row[j], lk = row[j2];
+        uint32_t x0 = g0[t], x1 = g1[t], x2 = g2[t], y0 = g0[t2], y1 = g1[t2], y2 = g2[t2];
+        s96_sub_half(x0, x1, x2, u96_mulhi(U96{li.x, li.y, li.z}, U96{lj.x, lj.y, lj.z}), li.w ^ lj.w);
+        s96_sub_half(y0, y1, y2, u96_mulhi(U96{li.x, li.y, li.z}, U96{lk.x, lk.y, lk.z}), li.w ^ lk.w);
         g0[t] = x0;
         g1[t] = x1;
         g2[t] = x2;
+        if (two) {
+          g0[t2] = y0;
+          g1[t2] = y1;
+          g2[t2] = y2;
+        }
         if (i == j) norms[i] = norm_of(i, x0, x1, x2);
       }
     }
