@@ -186,15 +186,15 @@ rss_status rss_solve_noalloc(const rss_factorization* f, void* b, int64_t nrhs, 
 /* Autotuner of the solve's launch form.  The FP64 sweeps (fewer than 32
  * right-hand sides) run in one of three forms, which add the same products in
  * the same order, so results are bitwise the same under any of them:
- *  - "per_class": kernels per colour class (two or three launches each);
+ *  - "per_class": one launch per colour class and sweep (a thread-block cluster
+ *    per box where the class cannot fill the GPU);
  *  - "persistent": two cooperative launches that walk all colour classes of the
- *    factorization, meeting at grid barriers; a class with few boxes is split
- *    across CTAs by rows of C (one more barrier);
+ *    factorization, one box per CTA, meeting at grid barriers;
  *  - "hybrid": per-class kernels for the fine levels and persistent launches for
  *    the tail of colour classes with fewer than "tail_boxes" boxes each (the
  *    coarse levels, where per-class launches are bound by latency).
- * The persistent part has two knobs: "spread", the target number of work items
- * per CTA and class, and "ctas_per_sm" (0: as many as fit).  rss_tune_solve
+ * The persistent part has a knob, "ctas_per_sm" (0: as many as fit); "spread" is
+ * read and written for tables from earlier builds and has no effect.  rss_tune_solve
  * times the solve of nrhs zero right-hand sides under eleven candidates (the
  * per-class form, four persistent and six hybrid schedules; median of three
  * after one untimed run, CUDA events on stream), keeps the fastest for the

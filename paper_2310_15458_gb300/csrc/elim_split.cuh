@@ -282,42 +282,38 @@ template <typename T, int NBC> __global__ void __launch_bounds__(16 * NBC) k_eli
     for (int e = tid; e < r * cw; e += NTH) {
       const int i = e % r, j = e / r;
       const T x = i < rows ? X[i * NBC + j] : zero<T>();
-      R.Ui[i + (size_t)(c0 + j) * r] = x;
-      if (R.ozp) R.We[(size_t)(c0 + j) * n + k + i] = x;
+      if (R.Ui) R.Ui[i + (size_t)(c0 + j) * r] = x;
+      R.We[(size_t)(c0 + j) * n + k + i] = x;
     }
-    if (R.ozp)   // W_E = [-T U^{-1}; U^{-1}]
-      for (int e = tid; e < k * cw; e += NTH) {
-        const int l = e % k, j = e / k;
-        T x = zero<T>();
+    for (int e = tid; e < k * cw; e += NTH) {   // W_E = [-T U^{-1}; U^{-1}]
+      const int l = e % k, j = e / k;
+      T x = zero<T>();
 #pragma unroll 4
-        for (int m = 0; m < rows; ++m) x = msb(x, R.Tm[l + (size_t)m * k], X[m * NBC + j]);
-        R.We[(size_t)(c0 + j) * n + l] = x;
-      }
+      for (int m = 0; m < rows; ++m) x = msb(x, R.Tm[l + (size_t)m * k], X[m * NBC + j]);
+      R.We[(size_t)(c0 + j) * n + l] = x;
+    }
   } else {
     // row c0 + j of L^{-1} P: entry m is entry pos(m) of the row of L^{-1}
     const int* pos = R.pos;
-    for (int e = tid; e < r * NBC; e += NTH) {
-      const int j = e % NBC, m = e / NBC;
-      if (j >= cw) continue;
-      const int pm = pos[m];
-      R.LiP[(c0 + j) + (size_t)m * r] = pm < rows ? X[pm * NBC + j] : zero<T>();
-      if (R.panels && !R.ozp) R.Li[(c0 + j) + (size_t)m * r] = m < rows ? X[m * NBC + j] : zero<T>();
+    if (R.Li)
+      for (int e = tid; e < r * NBC; e += NTH) {
+        const int j = e % NBC, m = e / NBC;
+        if (j < cw) R.Li[(c0 + j) + (size_t)m * r] = m < rows ? X[m * NBC + j] : zero<T>();
+      }
+    // W_F = [-(L^{-1} P T^*)^T; (L^{-1} P)^T]
+    for (int e = tid; e < r * cw; e += NTH) {
+      const int m = e % r, j = e / r, pm = pos[m];
+      R.Wf[(size_t)(c0 + j) * n + k + m] = pm < rows ? X[pm * NBC + j] : zero<T>();
     }
-    if (R.ozp) {   // W_F = [-(L^{-1} P T^*)^T; (L^{-1} P)^T]
-      for (int e = tid; e < r * cw; e += NTH) {
-        const int m = e % r, j = e / r, pm = pos[m];
-        R.Wf[(size_t)(c0 + j) * n + k + m] = pm < rows ? X[pm * NBC + j] : zero<T>();
-      }
-      for (int e = tid; e < k * cw; e += NTH) {
-        const int l = e % k, j = e / k;
-        T x = zero<T>();
+    for (int e = tid; e < k * cw; e += NTH) {
+      const int l = e % k, j = e / k;
+      T x = zero<T>();
 #pragma unroll 4
-        for (int m = 0; m < r; ++m) {
-          const int pm = pos[m];
-          if (pm < rows) x = msb(x, X[pm * NBC + j], cj(R.Tm[l + (size_t)m * k]));
-        }
-        R.Wf[(size_t)(c0 + j) * n + l] = x;
+      for (int m = 0; m < r; ++m) {
+        const int pm = pos[m];
+        if (pm < rows) x = msb(x, X[pm * NBC + j], cj(R.Tm[l + (size_t)m * k]));
       }
+      R.Wf[(size_t)(c0 + j) * n + l] = x;
     }
   }
 }

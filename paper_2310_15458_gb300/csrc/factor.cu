@@ -1174,7 +1174,7 @@ template <typename T> __global__ void __launch_bounds__(NT, 4) k_elim_lu(ElimArg
   if (onchip)
     for (int e = tid; e < r * r; e += bs) R.LU[e] = LU[e];
   __syncthreads();
-  if (R.ozp) {
+  {
     // W_E = [-T U^{-1}; U^{-1}] and W_F = [-(L^{-1} P T^*)^T; (L^{-1} P)^T], n x r, ld n:
     // E = X_CR U^{-1} = A_CB W_E and F^T = (L^{-1} P X_RC)^T = A_BC^T W_F (Eqs. 7, 8)
     const int n = k + r;
@@ -2732,7 +2732,7 @@ rss_status factor_impl(const rss_tree* tree, const rss_params* prm, cudaStream_t
   f->launches += 1;
 
   // workspaces reused across colour classes and levels
-  GrowBuf gb_cls(st), gb_k(st), gb_perm(st), gb_clsidx(st), gb_Tws(st), gb_Y(st), gb_oz(st), gb_w(st);
+  GrowBuf gb_cls(st), gb_k(st), gb_perm(st), gb_clsidx(st), gb_Tws(st), gb_Y(st), gb_oz(st), gb_w(st), gb_inv(st);
   // leaf level
   size_t transient = 0;
   HostLevel<T> cur;
@@ -3061,15 +3061,14 @@ rss_status factor_impl(const rss_tree* tree, const rss_params* prm, cudaStream_t
         R.LU = static_cast<T*>(f->arena.get(sizeof(T) * (size_t)r * r));
         R.piv = static_cast<int*>(f->arena.get(sizeof(int) * r));
         R.pos = static_cast<int*>(f->arena.get(sizeof(int) * r));
-        R.LiP = static_cast<T*>(f->arena.get(sizeof(T) * (size_t)r * r));
-        R.Ui = static_cast<T*>(f->arena.get(sizeof(T) * (size_t)r * r));
-        R.Li = static_cast<T*>(f->arena.get(sizeof(T) * (size_t)r * r));
+        R.We = static_cast<T*>(f->arena.get(sizeof(T) * (size_t)n * r));
+        R.Wf = static_cast<T*>(f->arena.get(sizeof(T) * (size_t)n * r));
         R.E = static_cast<T*>(f->arena.get(sizeof(T) * (size_t)c * r));
         R.Ft = static_cast<T*>(f->arena.get(sizeof(T) * (size_t)c * r));
         R.idxR = static_cast<int*>(f->arena.get(sizeof(int) * r));
         R.idxC = static_cast<int*>(f->arena.get(sizeof(int) * c));
         R.cmap = static_cast<int*>(f->arena.get(sizeof(int) * c));
-        if (!R.Tm || !R.LU || !R.piv || !R.pos || !R.LiP || !R.Ui || !R.Li || !R.E || !R.Ft || !R.idxR || !R.idxC ||
+        if (!R.Tm || !R.LU || !R.piv || !R.pos || !R.We || !R.Wf || !R.E || !R.Ft || !R.idxR || !R.idxC ||
             !R.cmap) {
           rss_set_error("rss_factor: device arena allocation failed");
           return RSS_ENOMEM;
@@ -3121,9 +3120,8 @@ rss_status factor_impl(const rss_tree* tree, const rss_params* prm, cudaStream_t
       if (prm->schur_path == 0 || prm->schur_path == 2) {
         size_t bytes = 0;
         for (const BoxRec<T>& R : recs)
-          if (R.k + R.r <= ozp_nmax)
-            bytes += 2 * (((size_t)(R.k + R.r) * R.r * sizeof(T) + 255) & ~size_t(255)) + wsl_bytes(R);
-        if (bytes > 0) {
+          if (R.k + R.r <= ozp_nmax) bytes += wsl_bytes(R);
+        {
           if (!gb_w.ensure(bytes)) {
             rss_set_error("rss_factor: device workspace allocation failed");
             return RSS_ENOMEM;
@@ -3131,10 +3129,6 @@ rss_status factor_impl(const rss_tree* tree, const rss_params* prm, cudaStream_t
           char* p = static_cast<char*>(gb_w.p);
           for (BoxRec<T>& R : recs) {
             if (R.k + R.r > ozp_nmax) continue;
-            const size_t b = ((size_t)(R.k + R.r) * R.r * sizeof(T) + 255) & ~size_t(255);
-            R.We = reinterpret_cast<T*>(p);
-            R.Wf = reinterpret_cast<T*>(p + b);
-            p += 2 * b;
             if (sizeof(T) == sizeof(double)) {
               const size_t np = (R.k + R.r + 15) & ~15, rp = (R.r + 31) & ~31;
               const size_t bs = (2 * rp * OZ_S * np * sizeof(uint16_t) + 255) & ~size_t(255);
@@ -3180,6 +3174,35 @@ rss_status factor_impl(const rss_tree* tree, const rss_params* prm, cudaStream_t
         }
         f->peak_transient = std::max(f->peak_transient, transient + bytes);
       }
+      // the column-group kernels, for boxes that fit them and take E and F from the
+      // panel kernels; the FP64 panels read U^{-1} and L^{-1}, k_elim_lu also L^{-1} P
+      int max_n = 0;
+      bool ef_later = true;
+      for (const BoxRec<T>& R : recs) {
+        max_n = std::max(max_n, R.k + R.r);
+        ef_later = ef_later && (R.panels || R.ozp);
+      }
+      const bool elim_cols =
+          ef_later && std::max(elim_x_bytes<T>(8, max_k, max_n), elim_inv_bytes<T>(16, max_r)) <= 200 * 1024;
+      {
+        auto rr = [](const BoxRec<T>& R) { return ((size_t)R.r * R.r * sizeof(T) + 255) & ~size_t(255); };
+        size_t bytes = 0;
+        for (const BoxRec<T>& R : recs)
+          if (!elim_cols || !R.ozp) bytes += 3 * rr(R);
+        if (!gb_inv.ensure(bytes)) {
+          rss_set_error("rss_factor: device workspace allocation failed");
+          return RSS_ENOMEM;
+        }
+        f->peak_transient = std::max(f->peak_transient, transient + bytes);
+        char* p = static_cast<char*>(gb_inv.p);
+        for (BoxRec<T>& R : recs) {
+          if (elim_cols && R.ozp) continue;
+          R.Ui = reinterpret_cast<T*>(p);
+          R.Li = reinterpret_cast<T*>(p + rr(R));
+          R.LiP = reinterpret_cast<T*>(p + 2 * rr(R));
+          p += 3 * rr(R);
+        }
+      }
       BoxRec<T>* d_recs = static_cast<BoxRec<T>*>(f->arena.get(sizeof(BoxRec<T>) * nrec));
       if (!d_recs) { rss_set_error("rss_factor: device arena allocation failed"); return RSS_ENOMEM; }
       RSS_CUDA(cudaMemcpyAsync(d_recs, recs.data(), sizeof(BoxRec<T>) * nrec, cudaMemcpyHostToDevice, st));
@@ -3200,14 +3223,7 @@ rss_status factor_impl(const rss_tree* tree, const rss_params* prm, cudaStream_t
       ea.smem_cap = (int)((ecap - ints) / sizeof(T));
       evs.emplace_back(1, std::make_unique<Ev>());
       evs.back().second->start(st);
-      int max_n = 0;
-      bool ef_later = true;   // every box takes E and F from the panel kernels
-      for (const BoxRec<T>& R : recs) {
-        max_n = std::max(max_n, R.k + R.r);
-        ef_later = ef_later && (R.panels || R.ozp);
-      }
-      const size_t xb = std::max(elim_x_bytes<T>(8, max_k, max_n), elim_inv_bytes<T>(16, max_r));
-      if (ef_later && xb <= 200 * 1024) {
+      if (elim_cols) {
         // columns per CTA: as many as still give every SM two CTAs
         auto launch_x = [&](auto kern, int jc, size_t smem) -> cudaError_t {
           cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
@@ -3312,7 +3328,7 @@ rss_status factor_impl(const rss_tree* tree, const rss_params* prm, cudaStream_t
       }
       RSS_LAUNCHED();
       evs.back().second->stop(st);
-      for (BoxRec<T>& R : recs) R.Esl = R.Fsl = nullptr, R.Eexp = R.Fexp = nullptr;
+      for (BoxRec<T>& R : recs) R.Esl = R.Fsl = nullptr, R.Eexp = R.Fexp = nullptr, R.Ui = R.Li = R.LiP = nullptr;
       f->launches += 2;
       f->n_elim += 1;
       f->n_schur += 1;
@@ -3321,7 +3337,7 @@ rss_status factor_impl(const rss_tree* tree, const rss_params* prm, cudaStream_t
       std::memcpy(hcopy, recs.data(), sizeof(BoxRec<T>) * nrec);
       f->rec_host.push_back(hcopy);
       const int colour = (boxes[0] % g) % 3 + 3 * ((boxes[0] / g) % 3);
-      f->batches.push_back(Batch{g, colour, nrec, d_recs, max_k, max_r, max_c});
+      f->batches.push_back(Batch{g, colour, nrec, d_recs, max_k, max_r, max_c, max_n});
     }
     RSS_CUDA(cudaStreamSynchronize(st));
     for (auto& pe : evs) {

@@ -9,7 +9,7 @@
 
 #include "common.cuh"
 
-constexpr int SWP_SPREAD_DEFAULT = 4;   // persistent sweeps: target work items per CTA and class
+constexpr int SWP_SPREAD_DEFAULT = 4;   // reported for tables that carry a spread; no launch form uses it
 
 enum : uint32_t { RSS_TAG_TREE = 0x52545245u, RSS_TAG_FACTOR = 0x52464143u, RSS_TAG_SERVER = 0x52535256u };
 
@@ -35,9 +35,10 @@ template <typename T> struct BoxRec {
   T* LU;        // r x r packed LU of X_RR, ld r
   int* piv;     // r getrf pivots (0-based)
   int* pos;     // r: P e_m = e_pos[m] for the exchanges of piv (factor time only)
-  T* LiP;       // r x r, ld r: L_R^{-1} P_R (the solve applies it as one product)
-  T* Ui;        // r x r, ld r: U_R^{-1}
-  T* Li;        // r x r, ld r: L_R^{-1} (unit lower), factor time only
+  // factor time only, where a kernel of the class needs them (else null), ld r
+  T* LiP;       // r x r: L_R^{-1} P_R
+  T* Ui;        // r x r: U_R^{-1}
+  T* Li;        // r x r: L_R^{-1} (unit lower)
   int panels;   // 1: E and F^T are formed by the panel kernel
   T* E;         // c x r, ld c:  X_CR U_R^{-1}
   T* Ft;        // c x r, ld c:  (L_R^{-1} P_R X_RC)^T (plain transpose)
@@ -51,11 +52,12 @@ template <typename T> struct BoxRec {
   int* Eexp;      // c row exponents
   int* Fexp;
   int kp;         // r rounded up to a multiple of 16
-  // factor-time only, tensor-core panel path (ozp = 1): with the columns of B
-  // in pivot order, E = A_CB W_E and F^T = A_BC^T W_F (n x r each, ld n), where
-  // W_E = [-T U^{-1}; U^{-1}] and W_F = [-(L^{-1} P T^*)^T; (L^{-1} P)^T]
+  // with the columns of B in pivot order, E = A_CB W_E and F^T = A_BC^T W_F (n x r
+  // each, ld n), where W_E = [-T U^{-1}; U^{-1}] and W_F = [-(L^{-1} P T^*)^T;
+  // (L^{-1} P)^T]; the solve applies W_F^T and W_E to the points of B
   T* We;
   T* Wf;
+  // factor-time only, tensor-core panel path (ozp = 1) of real factors:
   // the columns of W_E then W_F (2 rp columns, rp = r rounded up to 32, the
   // padding columns zero), each cut into OZ_S bf16 digit slices of np = n
   // rounded up to 16 entries: column j at Wsl + j * OZ_S * np, slice p at
@@ -83,7 +85,7 @@ struct Batch {
   int colour;
   int nrec;
   void* d_recs;   // BoxRec<T>[nrec] on the device
-  int max_k, max_r, max_c;
+  int max_k, max_r, max_c, max_n;   // (max_n: of k + r)
 };
 
 struct LevelInfo {
@@ -130,8 +132,8 @@ struct rss_factorization {
   Arena arena;
   std::vector<Batch> batches;          // factor order
   void* d_swp = nullptr;               // the batches as the persistent sweeps read them (arena)
-  int swp_spread = 0;                  // their schedule's knobs (0: the defaults; rss_tune_solve sets them):
-  int swp_ctas = 0;                    // work items per CTA and class, CTAs per SM (0: as many as fit),
+  int swp_spread = 0;                  // a knob of earlier schedules, kept in the tables (no effect),
+  int swp_ctas = 0;                    // CTAs per SM of the persistent sweeps (0: as many as fit),
   int swp_launch = 0;                  // the launch form (0, 1: per-class kernels; 2: persistent;
                                        // 3: per-class, then persistent for the coarse tail),
   int swp_tail_boxes = 0;              // and the tail: the classes with fewer boxes than this
