@@ -183,7 +183,7 @@ rss_status rss_solve(const rss_factorization* f, void* b, int64_t nrhs, int64_t 
 rss_status rss_solve_noalloc(const rss_factorization* f, void* b, int64_t nrhs, int64_t ldb,
                              void* stream);
 
-/* Autotuner of the solve's launch form.  The FP64 sweeps (fewer than 32
+/* Autotuner of the solve's launch form.  The FP64 sweeps (fewer than 16
  * right-hand sides) run in one of three forms, which add the same products in
  * the same order, so results are bitwise the same under any of them:
  *  - "per_class": one launch per colour class and sweep (a thread-block cluster
@@ -201,9 +201,9 @@ rss_status rss_solve_noalloc(const rss_factorization* f, void* b, int64_t nrhs, 
  * later solves of f, and writes the table to json (may be NULL) as {"nrhs": ..,
  * "path": .., "candidates": [..], "launch": .., "spread": .., "ctas_per_sm":
  * .., "tail_boxes": .., "ms": ..}; passing that text back as
- * rss_params.tune_table applies it without measuring.  With 32 or more
- * right-hand sides (tensor-core sweeps) there is nothing to tune and the table
- * says so.  The paper has no counterpart.  Synchronises stream; allocates
+ * rss_params.tune_table applies it without measuring.  With 16 to 31
+ * right-hand sides it times the FP64 sweeps of that many columns; with 32 or more
+ * (tensor-core sweeps) there is nothing to tune and the table says so.  The paper has no counterpart.  Synchronises stream; allocates
  * n * nrhs scalars for the duration of the call; solves that run meanwhile on
  * other streams may take either form. */
 rss_status rss_tune_solve(rss_factorization* f, int64_t nrhs, void* stream, char* json, size_t len);
@@ -215,8 +215,11 @@ rss_status rss_tune_solve(rss_factorization* f, int64_t nrhs, void* stream, char
  * device-memory budget allows) into one right-hand-side panel and solves it
  * with one rss_solve; requests arriving meanwhile join the next panel, and
  * panels of different factorizations run concurrently on their own streams.
- * Every column goes through the same operations whatever it is batched with,
- * so a result equals the one rss_solve gives for the request alone.  This is
+ * A panel takes the tensor-core sweeps when all of its requests would by
+ * themselves (16 or more columns), and with a real factor from 32 columns on; the
+ * others take the FP64 sweeps, where every column goes through the same
+ * operations whatever it is batched with, so a result equals the one rss_solve
+ * gives for the request alone (between the two kinds of sweeps: to rounding).  This is
  * the serving pattern the workloads ask for (requests of 1-64 right-hand sides
  * against several resident factorizations); the paper has no counterpart. */
 

@@ -147,6 +147,33 @@ __device__ __forceinline__ void umma_bf16(uint32_t tmem_d, uint64_t adesc, uint6
       "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(tmem_d),
       "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate));
 }
+// The same for a warp that runs the issuing loop together, one lane (`lead`) issuing:
+// without a divergent branch the operands stay in uniform registers, and an issue
+// costs a few cycles instead of about 85.  Descriptors by their low words (start
+// address >> 4, LBO); UMMA_HI: SBO 512, version 1.
+constexpr uint32_t UMMA_HI = (512u >> 4) | (1u << 14);
+__device__ __forceinline__ uint32_t umma_lo(uint32_t saddr) { return ((saddr >> 4) & 0x3FFF) | ((128u >> 4) << 16); }
+__device__ __forceinline__ void umma_bf16_w(uint32_t tmem_d, uint32_t alo, uint32_t blo, uint32_t idesc,
+                                            uint32_t accumulate, uint32_t lead) {
+  asm volatile(
+      "{\n.reg .pred p, q;\n.reg .b64 da, db;\nmov.b64 da, {%1, %6};\nmov.b64 db, {%2, %6};\n"
+      "setp.ne.b32 p, %4, 0;\nsetp.ne.b32 q, %5, 0;\n"
+      "@q tcgen05.mma.cta_group::1.kind::f16 [%0], da, db, %3, p;\n}\n" ::"r"(tmem_d),
+      "r"(alo), "r"(blo), "r"(idesc), "r"(accumulate), "r"(lead), "r"(UMMA_HI));
+}
+__device__ __forceinline__ void umma_commit_w(uint64_t* mbar, uint32_t lead) {
+  asm volatile(
+      "{\n.reg .pred q;\nsetp.ne.b32 q, %1, 0;\n"
+      "@q tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n}\n" ::"r"(smem_u32(mbar)),
+      "r"(lead)
+      : "memory");
+}
+// one lane of a converged warp
+__device__ __forceinline__ uint32_t elect_one() {
+  uint32_t e;
+  asm volatile("{\n.reg .pred p;\nelect.sync _|p, 0xffffffff;\nselp.u32 %0, 1, 0, p;\n}\n" : "=r"(e));
+  return e;
+}
 // the mbarrier receives one arrival when every tcgen05.mma issued so far by this thread is done
 __device__ __forceinline__ void umma_commit(uint64_t* mbar) {
   asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n" ::"r"(smem_u32(mbar))
@@ -224,31 +251,51 @@ __device__ __forceinline__ long long oz_scaled_int(double x, int emax_b) {
   else X = 0;
   return (b >> 63) ? -X : X;
 }
-// bf16 bit pattern of a small integer d, |d| <= 128 (exact: conversion instructions)
-__device__ __forceinline__ unsigned oz_bf16_int(int d) {
-  return (unsigned)__bfloat16_as_ushort(__float2bfloat16_rn((float)d));
-}
-// the eight digits of X (|X| < 2^56), most significant first, packed for two
-// adjacent entries: out[p] = bf16(d_p(X0)) | bf16(d_p(X1)) << 16
+// the eight digits of X (|X| <= 2^56), most significant first, packed for two
+// adjacent entries: out[p] = bf16(d_p(X0)) | bf16(d_p(X1)) << 16.  With 64 added to
+// each of the digits 1 .. 7 they are plain 7-bit fields of X; a field becomes an FP32
+// integer by one OR and one addition, whose upper half is its bf16 (exact).  (About
+// 45 instructions an entry with the scaling, none of them integer-to-float
+// conversions, which run at an eighth of the rate.)
 __device__ __forceinline__ void oz_digits2(long long X0, long long X1, uint32_t* out) {
-  int d0[8], d1[8];
+  constexpr long long BIAS = 64ll * (1 + (1ll << 7) + (1ll << 14) + (1ll << 21) + (1ll << 28) + (1ll << 35) + (1ll << 42));
+  const unsigned long long Y0 = (unsigned long long)(X0 + BIAS), Y1 = (unsigned long long)(X1 + BIAS);
+  const uint32_t l0 = (uint32_t)Y0, h0 = (uint32_t)(Y0 >> 32), l1 = (uint32_t)Y1, h1 = (uint32_t)(Y1 >> 32);
 #pragma unroll
-  for (int p = 7; p >= 1; --p) {
-    d0[p] = (int)(((X0 + 64) & 127) - 64);
-    X0 = (X0 - d0[p]) >> 7;
-    d1[p] = (int)(((X1 + 64) & 127) - 64);
-    X1 = (X1 - d1[p]) >> 7;
+  for (int p = 1; p < 8; ++p) {
+    const int sh = 7 * (7 - p);
+    const uint32_t w0 = sh < 32 ? __funnelshift_r(l0, h0, sh) : h0 >> (sh - 32);
+    const uint32_t w1 = sh < 32 ? __funnelshift_r(l1, h1, sh) : h1 >> (sh - 32);
+    const float f0 = __uint_as_float((w0 & 127u) | 0x4B000000u) - 8388672.0f;   // 2^23 + field - (2^23 + 64)
+    const float f1 = __uint_as_float((w1 & 127u) | 0x4B000000u) - 8388672.0f;
+    out[p] = __byte_perm(__float_as_uint(f0), __float_as_uint(f1), 0x7632);
   }
-  d0[0] = (int)X0;
-  d1[0] = (int)X1;
-#pragma unroll
-  for (int p = 0; p < 8; ++p) out[p] = oz_bf16_int(d0[p]) | (oz_bf16_int(d1[p]) << 16);
+  const float f0 = __int_as_float(0x4B400000 + ((int)h0 >> 17)) - 12582912.0f;
+  const float f1 = __int_as_float(0x4B400000 + ((int)h1 >> 17)) - 12582912.0f;
+  out[0] = __byte_perm(__float_as_uint(f0), __float_as_uint(f1), 0x7632);
 }
 // An FP32 value holding an integer |g| < 2^22 as an int32, by adding 1.5 2^23 and
 // reading the mantissa (one FP32 add and one integer add)
 __device__ __forceinline__ int oz_fint(float g) {
   return __float_as_int(g + 12582912.0f) - 0x4B400000;
 }
+
+// Eight group sums G_u (g(u), integers in FP32) as W = sum_u G_u 2^(39-7u), the pairs
+// (G_u 2^7 + G_{u+1}) 2^(32-7u) exact in 32 bits, the last one rounded to weight 1.
+// WIDE: for |G_u| up to 2^24 instead of 2^22 (a conversion in place of an addition).
+template <bool WIDE = false, class G> __device__ __forceinline__ long long oz_join(G g) {
+  int v[4];
+#pragma unroll
+  for (int u = 0; u < 4; ++u) {
+    const float f0 = g(2 * u), f1 = g(2 * u + 1);
+    v[u] = WIDE ? __float2int_rn(f0) * 128 + __float2int_rn(f1) : oz_fint(f0) * 128 + oz_fint(f1);
+  }
+  long long w = ((long long)v[0] << 32) + ((v[3] + 512) >> 10);
+  asm("mad.wide.s32 %0, %1, 262144, %0;\n" : "+l"(w) : "r"(v[1]));
+  asm("mad.wide.s32 %0, %1, 16, %0;\n" : "+l"(w) : "r"(v[2]));
+  return w;
+}
+static_assert(OZ_S == 8 && OZ_BITS == 7, "");
 
 // ------------------------------------------------------------------ E and F on the tensor cores
 // One vector x_0..x_{len-1} (x_l = val(l)) shared by G consecutive lanes, cut

@@ -29,6 +29,7 @@
 
 #include "internal.h"
 #include "tc_gemm.cuh"
+#include "tw_common.cuh"
 
 namespace {
 
@@ -1466,14 +1467,7 @@ __global__ void __launch_bounds__(NT, 2) k_elim_oz(ElimArgs<double> a) {
       for (int ni = 0; ni < 2; ++ni)
 #pragma unroll
         for (int e = 0; e < 4; ++e) {
-          long long w = 0;
-#pragma unroll
-          for (int u = 0; u < OZ_S; u += 2) {
-            const long long gv = (long long)(oz_fint(acc[u][ni][e]) * 128 + oz_fint(acc[u + 1][ni][e]));
-            const int sh = 32 - OZ_BITS * u;
-            w += sh >= 0 ? (gv << sh) : ((gv + (1LL << (-sh - 1))) >> (-sh));
-          }
-          W[ni][e] = w;
+          W[ni][e] = oz_join([&](int u) { return acc[u][ni][e]; });
         }
       double* out = cc < rp ? R.E : R.Ft;
 #pragma unroll
@@ -1713,15 +1707,9 @@ __global__ void __launch_bounds__(NT, 2) k_schur_oz(LevelDev<double> L, const Bo
     for (int ni = 0; ni < 2; ++ni)
 #pragma unroll
       for (int e = 0; e < 4; ++e) {
-        long long w = W[ni][e];
+        W[ni][e] += oz_join([&](int u) { return acc[u][ni][e]; });
 #pragma unroll
-        for (int u = 0; u < OZ_S; u += 2) {
-          const long long gv = (long long)(oz_fint(acc[u][ni][e]) * 128 + oz_fint(acc[u + 1][ni][e]));
-          const int sh = 32 - OZ_BITS * u;
-          w += sh >= 0 ? (gv << sh) : ((gv + (1LL << (-sh - 1))) >> (-sh));
-          acc[u][ni][e] = acc[u + 1][ni][e] = 0.f;
-        }
-        W[ni][e] = w;
+        for (int u = 0; u < OZ_S; ++u) acc[u][ni][e] = 0.f;
       }
   };
   const int nch = (kp + SRK - 1) / SRK;
@@ -1911,14 +1899,7 @@ __global__ void __launch_bounds__(ST_NT, 2) k_schur_tc(LevelDev<double> L, const
       tmem_ld_wait();
 #pragma unroll
       for (int jj = 0; jj < 8; ++jj) {
-        long long w = 0;
-#pragma unroll
-        for (int u = 0; u < OZ_S; u += 2) {
-          const long long gv = (long long)(oz_fint(__uint_as_float(gr[u][jj])) * 128 +
-                                           oz_fint(__uint_as_float(gr[u + 1][jj])));
-          const int sh = 32 - OZ_BITS * u;
-          w += sh >= 0 ? (gv << sh) : ((gv + (1LL << (-sh - 1))) >> (-sh));
-        }
+        const long long w = oz_join([&](int u) { return __uint_as_float(gr[u][jj]); });
         const int j = CH * half + c0 + jj;
         if (i < c && j0 + j < c) L.blk[rowb + colb[j]] = cv[c0 + jj] - oz_ldexp_int(w, rexp + cexp[j] - 53);
       }
@@ -2087,14 +2068,7 @@ __global__ void __launch_bounds__(SRW_NT, 1) k_schur_tc_rows(LevelDev<double> L,
           tmem_ld_wait();
 #pragma unroll
           for (int jj = 0; jj < 8; ++jj) {
-            long long w = 0;
-#pragma unroll
-            for (int u = 0; u < OZ_S; u += 2) {
-              const long long gv = (long long)(oz_fint(__uint_as_float(gr[u][jj])) * 128 +
-                                               oz_fint(__uint_as_float(gr[u + 1][jj])));
-              const int sh = 32 - OZ_BITS * u;
-              w += sh >= 0 ? (gv << sh) : ((gv + (1LL << (-sh - 1))) >> (-sh));
-            }
+            const long long w = oz_join([&](int u) { return __uint_as_float(gr[u][jj]); });
             const int j = CH * half + c0 + jj;
             if (i < c && j0 + j < c) L.blk[rowb + colb[cb3][j]] = cv[c0 + jj] - oz_ldexp_int(w, rexp + cexp[cb3][j] - 53);
           }
@@ -2260,14 +2234,7 @@ __global__ void __launch_bounds__(ST_NT, 1) k_schur_tc_c(LevelDev<zd> L, const B
         tmem_ld_wait();
 #pragma unroll
         for (int jj = 0; jj < 8; ++jj) {
-          long long acc = 0;
-#pragma unroll
-          for (int u = 0; u < OZ_S; u += 2) {
-            const long long gv = (long long)(oz_fint(__uint_as_float(gr[u][jj])) * 128 +
-                                             oz_fint(__uint_as_float(gr[u + 1][jj])));
-            const int sh = 32 - OZ_BITS * u;
-            acc += sh >= 0 ? (gv << sh) : ((gv + (1LL << (-sh - 1))) >> (-sh));
-          }
+          const long long acc = oz_join([&](int u) { return __uint_as_float(gr[u][jj]); });
           w[part][jj] = acc;
         }
       }

@@ -161,18 +161,6 @@ template <typename S> __global__ void __launch_bounds__(256) k_idg_split(IdArgs<
   }
 }
 
-// Bulk copy global -> shared memory (both 16-byte aligned, a multiple of 16 bytes),
-// counted on the mbarrier.
-__device__ __forceinline__ void bulk_g2s(void* smem, const void* gmem, uint32_t bytes, uint64_t* mbar) {
-  asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];\n" ::"r"(
-                   smem_u32(smem)),
-               "l"(gmem), "r"(bytes), "r"(smem_u32(mbar))
-               : "memory");
-}
-__device__ __forceinline__ void mbar_expect_tx(uint64_t* mbar, uint32_t bytes) {
-  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n" ::"r"(smem_u32(mbar)), "r"(bytes) : "memory");
-}
-
 __host__ __device__ inline int idg_items(int J) {   // column blocks c and row tiles of 128 with a row <= the columns
   int s = 0;
   for (int t = 0; 4 * t < J; ++t) s += J - 4 * t;

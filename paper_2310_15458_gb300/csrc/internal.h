@@ -68,16 +68,13 @@ template <typename T> struct BoxRec {
 };
 
 
-// Digit slices of the two large blocks of a real box record, for the
-// tensor-core sweeps with many right-hand sides (built on first use): the rows
-// of E (c rows, K = r) and the rows of F = (F^T)^T (r rows, K = c), each row cut
-// into OZ_S bf16 digit slices under one power-of-two scale over its K entries.
+// Digits of the four matrices of a real box that the tensor-core sweeps apply (built
+// on first use), in the order up W_F^T, E, down F, W_E: every row cut into OZ_S signed
+// 7-bit digits under one power-of-two scale, in the layout of the sweeps' stages
+// (sweep_tc.cuh), and the rows' biased exponents.
 struct SliceRec {
-  uint16_t* Esl;   // c x OZ_S x kp: row i at Esl + i * OZ_S * kp, slice p at + p * kp
-  int* Eexp;       // c row scales
-  uint16_t* Fsl;   // r x OZ_S x cp
-  int* Fexp;       // r row scales
-  int kp, cp;      // r and c rounded up to 16 (zero padding)
+  unsigned char* dig[4];
+  int* eb[4];
 };
 
 struct Batch {
@@ -165,7 +162,11 @@ struct rss_factorization {
 template <typename T> rss_status factor_impl(const rss_tree* tree, const rss_params* p,
                                              cudaStream_t st, rss_factorization* f);
 template <typename T> rss_status solve_impl(const rss_factorization* f, T* b_dev, int64_t nrhs,
-                                            int64_t ldb, cudaStream_t st);
+                                            int64_t ldb, cudaStream_t st, bool fp64 = false);
+// whether a panel of `cols` columns, packed from requests of at least `smallest`
+// columns, takes the FP64 sweeps whatever its width, so that each request's result is
+// the one of its own solve
+bool panel_in_fp64(const rss_factorization* f, int64_t cols, int64_t smallest);
 // device bytes one solve of nrhs columns allocates (working copy plus sweep
 // workspace), beside the caller's b
 size_t solve_device_bytes(const rss_factorization* f, int64_t nrhs);

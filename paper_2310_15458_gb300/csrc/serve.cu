@@ -139,16 +139,18 @@ bool launch_panel(rss_server* S, Slot& s) {
     }
     s.h_cap = bytes;
   }
-  int64_t col = 0;
+  int64_t col = 0, smallest = cols;
   for (Request* r : batch) {
+    smallest = std::min<int64_t>(smallest, r->nrhs);
     std::memcpy(static_cast<char*>(s.h_panel) + esz * n * col, r->b, esz * n * r->nrhs);
     col += r->nrhs;
   }
   cudaError_t e = cudaMemcpyAsync(s.d_panel, s.h_panel, bytes, cudaMemcpyHostToDevice, s.stream);
   rss_status st = RSS_OK;
+  const bool fp64 = panel_in_fp64(s.f, cols, smallest);
   if (e == cudaSuccess)
-    st = s.f->is_complex ? solve_impl<zd>(s.f, static_cast<zd*>(s.d_panel), cols, n, s.stream)
-                         : solve_impl<double>(s.f, static_cast<double*>(s.d_panel), cols, n, s.stream);
+    st = s.f->is_complex ? solve_impl<zd>(s.f, static_cast<zd*>(s.d_panel), cols, n, s.stream, fp64)
+                         : solve_impl<double>(s.f, static_cast<double*>(s.d_panel), cols, n, s.stream, fp64);
   if (e == cudaSuccess && st == RSS_OK)
     e = cudaMemcpyAsync(s.h_panel, s.d_panel, bytes, cudaMemcpyDeviceToHost, s.stream);
   if (e == cudaSuccess && st == RSS_OK) e = cudaEventRecord(s.done, s.stream);

@@ -46,18 +46,20 @@ template <int W, typename T> __device__ __forceinline__ T part_sum(T v) {
   return v;
 }
 
+// (entry (g, q) of the right-hand sides at x[g * ldx + q]: the columns of a point
+// side by side)
 // x_g(i) = [keep(i)] x_g(i) + sgn sum_j M(i, j) w_j for the rows i < rows of M (ld
 // scalars between columns) and the columns j >= lo(i) (M is zero before), w in shared
 // memory (RC scalars per j): four lanes per row, or, for one column when the rows fill
 // half the CTA, one thread per row (no shuffles); the same sums either way.
 template <typename T, int RC, typename LO, typename GI, typename KP>
 __device__ __forceinline__ void row_products(int rows, int r, int nq, int tid, int nt, const T* w, const T* M, size_t ld,
-                                             LO lo, GI gidx, KP keep, double sgn, T* xq, int64_t N) {
+                                             LO lo, GI gidx, KP keep, double sgn, T* xq, int64_t ldx) {
   const int L4 = (r + SW_PE - 1) / SW_PE;
   if constexpr (RC == 1) {
     if (rows * 2 >= nt) {
       for (int i = tid; i < rows; i += nt) {
-        T* g = xq + gidx(i);
+        T* g = xq + gidx(i) * ldx;
         const int a = lo(i);
         const T* m = M + i;
         T acc[SW_PE];
@@ -87,7 +89,7 @@ __device__ __forceinline__ void row_products(int rows, int r, int nq, int tid, i
       const bool kp = keep(i);
 #pragma unroll
       for (int q = 0; q < RC; q += SW_PE)
-        if (p + q < nq) old[q / SW_PE] = kp ? ld_l2(xq + gi + (int64_t)(p + q) * N) : zero<T>();
+        if (p + q < nq) old[q / SW_PE] = kp ? ld_l2(xq + gi * ldx + p + q) : zero<T>();
       const int j1 = min(r, (p + 1) * L4);
       const T* m = M + i;
 #pragma unroll 4
@@ -102,7 +104,7 @@ __device__ __forceinline__ void row_products(int rows, int r, int nq, int tid, i
     if (i < rows) {
 #pragma unroll
       for (int q = 0; q < RC; ++q)
-        if (q % SW_PE == p && q < nq) xq[gi + (int64_t)q * N] = old[q / SW_PE] + scl(sgn, acc[q]);
+        if (q % SW_PE == p && q < nq) xq[gi * ldx + q] = old[q / SW_PE] + scl(sgn, acc[q]);
     }
   }
 }
@@ -124,7 +126,7 @@ struct ClusterCta {
 // CTA `rank` of Q on one box; peer(p, q): the address of shared scalar p in CTA q.
 // Every thread calls it.
 template <typename T, int RC, typename CL>
-__device__ void up_box(const BoxRec<T>& R, T* xq, int64_t N, int nq, T* sm, size_t sm_cap, int rank, int Q,
+__device__ void up_box(const BoxRec<T>& R, T* xq, int64_t ldx, int nq, T* sm, size_t sm_cap, int rank, int Q,
                        bool wait_prev, CL cl) {
   cl.arrive();   // this CTA runs: its peers may write its y
   const int k = R.k, r = R.r, c = R.c, n = k + r, tid = threadIdx.x, nt = blockDim.x;
@@ -150,7 +152,7 @@ __device__ void up_box(const BoxRec<T>& R, T* xq, int64_t N, int nq, T* sm, size
   if (wait_prev) pdl_wait();
   for (int e = tid; e < n * RC; e += nt) {
     const int l = e / RC, q = e % RC;
-    v[e] = q < nq ? ld_l2(xq + (l < k ? R.idxC[l] : R.idxR[l - k]) + (int64_t)q * N) : zero<T>();
+    v[e] = q < nq ? ld_l2(xq + (l < k ? R.idxC[l] : R.idxR[l - k]) * ldx + q) : zero<T>();
   }
   cp_async_wait_group<1>();
   __syncthreads();
@@ -184,14 +186,14 @@ __device__ void up_box(const BoxRec<T>& R, T* xq, int64_t N, int nq, T* sm, size
   cl.wait();   // y is complete, and every CTA has read its copy of v
   for (int e = tid; e < (j1 - j0) * RC; e += nt) {
     const int j = j0 + e / RC, q = e % RC;
-    if (q < nq) xq[R.idxR[j] + (int64_t)q * N] = y[j * RC + q];
+    if (q < nq) xq[R.idxR[j] * ldx + q] = y[j * RC + q];
   }
   row_products<T, RC>(rows, r, nq, tid, nt, y, ste ? Es : R.E + i0, ste ? lde : c, [](int) { return 0; },
-                      [&](int i) { return (int64_t)R.idxC[i0 + i]; }, [](int) { return true; }, -1.0, xq, N);
+                      [&](int i) { return (int64_t)R.idxC[i0 + i]; }, [](int) { return true; }, -1.0, xq, ldx);
 }
 
 template <typename T, int RC, typename CL>
-__device__ void down_box(const BoxRec<T>& R, T* xq, int64_t N, int nq, T* sm, size_t sm_cap, int rank, int Q, int qc,
+__device__ void down_box(const BoxRec<T>& R, T* xq, int64_t ldx, int nq, T* sm, size_t sm_cap, int rank, int Q, int qc,
                          bool wait_prev, CL cl) {
   const int k = R.k, r = R.r, c = R.c, n = k + r, tid = threadIdx.x, nt = blockDim.x;
   const int sl = qc / Q;   // slices of C of this CTA: rank sl ..
@@ -219,11 +221,11 @@ __device__ void down_box(const BoxRec<T>& R, T* xq, int64_t N, int nq, T* sm, si
   if (wait_prev) pdl_wait();
   for (int e = tid; e < rows * RC; e += nt) {
     const int i = e / RC, q = e % RC;
-    yc[e] = q < nq ? ld_l2(xq + R.idxC[i0 + i] + (int64_t)q * N) : zero<T>();
+    yc[e] = q < nq ? ld_l2(xq + R.idxC[i0 + i] * ldx + q) : zero<T>();
   }
   for (int e = tid; e < r * RC; e += nt) {
     const int j = e / RC, q = e % RC;
-    z[e] = q < nq ? ld_l2(xq + R.idxR[j] + (int64_t)q * N) : zero<T>();
+    z[e] = q < nq ? ld_l2(xq + R.idxR[j] * ldx + q) : zero<T>();
   }
   cp_async_wait_group<1>();
   __syncthreads();
@@ -272,26 +274,26 @@ __device__ void down_box(const BoxRec<T>& R, T* xq, int64_t N, int nq, T* sm, si
   row_products<T, RC>(lw, r, nq, tid, nt, z, stw ? Ws : R.We + l0, stw ? ldw : n,
                       [&](int l) { return max(0, l0 + l - k); },   // rows of U^{-1} are zero left of the diagonal
                       [&](int l) { return (int64_t)(l0 + l < k ? R.idxC[l0 + l] : R.idxR[l0 + l - k]); },
-                      [&](int l) { return l0 + l < k; }, 1.0, xq, N);
+                      [&](int l) { return l0 + l < k; }, 1.0, xq, ldx);
   cl.wait();   // no CTA ends while its sums are read
 }
 
 // One colour class: cluster of Q CTAs per (box, RC columns).
 template <typename T, int RC, bool UP>
-__global__ void __launch_bounds__(SW_NT) k_sweep_cl(const BoxRec<T>* __restrict__ recs, T* __restrict__ x, int64_t N,
+__global__ void __launch_bounds__(SW_NT) k_sweep_cl(const BoxRec<T>* __restrict__ recs, T* __restrict__ x, int64_t ldx,
                                                     int nrhs, int Q, int qc, int sm_cap) {
   extern __shared__ __align__(16) unsigned char smraw[];
   T* sm = reinterpret_cast<T*>(smraw);
   pdl_launch();
   const int rank = blockIdx.x % Q, q0 = blockIdx.y * RC, nq = min(RC, nrhs - q0);
   const BoxRec<T> R = recs[blockIdx.x / Q];
-  T* xq = x + (int64_t)q0 * N;
+  T* xq = x + q0;
   if (Q == 1) {
-    if (UP) up_box<T, RC>(R, xq, N, nq, sm, sm_cap, 0, 1, true, SoloCta{});
-    else down_box<T, RC>(R, xq, N, nq, sm, sm_cap, 0, 1, qc, true, SoloCta{});
+    if (UP) up_box<T, RC>(R, xq, ldx, nq, sm, sm_cap, 0, 1, true, SoloCta{});
+    else down_box<T, RC>(R, xq, ldx, nq, sm, sm_cap, 0, 1, qc, true, SoloCta{});
   } else {
-    if (UP) up_box<T, RC>(R, xq, N, nq, sm, sm_cap, rank, Q, true, ClusterCta{});
-    else down_box<T, RC>(R, xq, N, nq, sm, sm_cap, rank, Q, qc, true, ClusterCta{});
+    if (UP) up_box<T, RC>(R, xq, ldx, nq, sm, sm_cap, rank, Q, true, ClusterCta{});
+    else down_box<T, RC>(R, xq, ldx, nq, sm, sm_cap, rank, Q, qc, true, ClusterCta{});
   }
 }
 
@@ -312,7 +314,7 @@ template <typename T> struct SwpArgs {
   const SwpClass<T>* cls;   // colour classes in factor order
   int ncls;
   T* x;
-  int64_t N;
+  int64_t ldx;
   int nrhs;
   unsigned* bar;            // grid barrier counters (zeroed before the launch)
   int* err;                 // RSS_ETIMEOUT when a barrier wait runs out
@@ -329,9 +331,9 @@ template <typename T, int RC, bool UP> __global__ void __launch_bounds__(SWP_NT)
     for (int it = blockIdx.x; it < C.nrec * nz; it += gridDim.x) {
       const int q0 = (it / C.nrec) * RC;
       const BoxRec<T> R = C.recs[it % C.nrec];
-      T* xq = a.x + (int64_t)q0 * a.N;
-      if (UP) up_box<T, RC>(R, xq, a.N, min(RC, a.nrhs - q0), sm, a.sm_cap, 0, 1, false, SoloCta{});
-      else down_box<T, RC>(R, xq, a.N, min(RC, a.nrhs - q0), sm, a.sm_cap, 0, 1, C.qc, false, SoloCta{});
+      T* xq = a.x + q0;
+      if (UP) up_box<T, RC>(R, xq, a.ldx, min(RC, a.nrhs - q0), sm, a.sm_cap, 0, 1, false, SoloCta{});
+      else down_box<T, RC>(R, xq, a.ldx, min(RC, a.nrhs - q0), sm, a.sm_cap, 0, 1, C.qc, false, SoloCta{});
       __syncthreads();
     }
     if (step + 1 < a.ncls && !grid_barrier(a.bar, a.polls, a.err)) return;

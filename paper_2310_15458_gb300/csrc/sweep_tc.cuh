@@ -1,0 +1,407 @@
+// The sweeps with many right-hand sides on the 5th-generation tensor cores.  Per
+// colour class two products up, y = W_F^T [b_S; b_R] into b_R and b_C -= E b_R, and
+// two down, z = y_R - F y_C into y_R and [y_S; y_R] = [y_S; 0] + W_E y_R (see
+// sweep.cuh), each a launch of one CTA per box, 128 rows of the matrix and TW_NC real
+// columns.  Rows of the matrix and columns of the right-hand sides are scaled by
+// powers of two over the whole inner dimension K and cut into eight signed 7-bit
+// digits; the slice products of equal weight u = p + q <= 7 are summed exactly in
+// FP32 in tensor memory over at most TW_KX entries of K, gathered into one int64 per
+// output and added in FP64: the accuracy of an FP64 product.  A complex product is
+// the real one with K doubled, [A_re A_im] times [B_re; -B_im] and [B_im; B_re]: the
+// two column groups of a CTA are then the real and imaginary parts of 32 columns.
+//
+// K is staged 32 at a time in two to four buffers, so the digits of one stage are cut
+// while the products of the others run; the down sweep's F y_C (K = c, up to thousands)
+// is split over a cluster of up to 8 CTAs where a class has few boxes, each with scales
+// of its own range of K, and the parts are added in order.  A column that holds an
+// infinity or a NaN gives NaN.  Real factors keep the matrices' digits (SliceRec, built
+// by the first call of 32 and more columns), which then come by bulk copies; with fewer
+// columns and for complex factors they are cut on the fly.
+//
+// Bound by the products (36 slice pairs for 54 bits: about 80 clocks an instruction,
+// close to the tensor peak) and the gathering of x in the large classes, by latency
+// (about 20 us a launch) in the coarse ones.  64 columns, against mma.sync products of
+// one CTA per box (real) and the FP64 sweeps (complex): Laplace 512^2 23.3 -> 9.1 ms,
+// Helmholtz 256^2 30.3 -> 9.9 ms; 16 columns, against the FP64 sweeps: 4.6 -> 3.3 ms
+// (Laplace 256^2) and 15.8 -> 6.0 ms (Helmholtz 256^2).
+constexpr int TW_MAXN = 128;                             // rows of the products that write what they read
+constexpr int TW_MAXC = 6000;                            // entries of K whose places fit beside the stages
+enum { TW_UPW = 0, TW_UPE = 1, TW_DNF = 2, TW_DNW = 3 };
+
+// rows and inner dimension of a product
+template <int OP, typename T> __host__ __device__ inline int tw_rows(const BoxRec<T>& R) {
+  return OP == TW_UPE ? R.c : OP == TW_DNW ? R.k + R.r : R.r;
+}
+template <int OP, typename T> __host__ __device__ inline int tw_inner(const BoxRec<T>& R) {
+  return OP == TW_UPW ? R.k + R.r : OP == TW_DNF ? R.c : R.r;
+}
+// the matrix: entry (i, l) at p[i * si + l * sl]
+template <int OP, typename T> __device__ __forceinline__ const T* tw_mat(const BoxRec<T>& R, size_t& si, size_t& sl) {
+  if (OP == TW_UPW) { si = R.k + R.r; sl = 1; return R.Wf; }
+  if (OP == TW_UPE) { si = 1; sl = R.c; return R.E; }
+  if (OP == TW_DNF) { si = R.c; sl = 1; return R.Ft; }
+  si = 1; sl = R.k + R.r; return R.We;
+}
+constexpr bool tw_k_contiguous(int op) { return op == TW_UPW || op == TW_DNF; }
+
+// The CTA's rows i0 .. of the matrix: exponents (biased, at least 1) of the largest of
+// their entries K0 .. K, into reb[TW_M].  scr: 512 keys of shared memory.
+template <int OP, typename T>
+__device__ void tw_row_exps(const BoxRec<T>& R, int i0, int rows, int K0, int K, int* reb, unsigned long long* scr) {
+  size_t si, sl;
+  const T* A = tw_mat<OP>(R, si, sl);
+  const int tid = threadIdx.x;
+  if (tw_k_contiguous(OP)) {   // a warp per row
+    for (int i = tid / 32; i < rows; i += TW_NT / 32) {
+      unsigned long long mk = 0;
+      for (int l = K0 + tid % 32; l < K; l += 32) mk = max(mk, tw_key(A[(i0 + i) * si + l]));
+      mk = shfl_max_u64(mk, 32);
+      if (tid % 32 == 0) reb[i] = oz_emax_b(mk);
+    }
+  } else {                     // four threads per row, lanes over rows
+    const int i = tid % TW_M, part = tid / TW_M;
+    unsigned long long mk = 0;
+    if (i < rows)
+      for (int l = K0 + part; l < K; l += TW_NT / TW_M) mk = max(mk, tw_key(A[(i0 + i) + (size_t)l * sl]));
+    scr[tid] = mk;
+    __syncthreads();
+    if (tid < TW_M) {
+#pragma unroll
+      for (int p = 1; p < TW_NT / TW_M; ++p) mk = max(mk, scr[tid + p * TW_M]);
+      reb[tid] = oz_emax_b(mk);
+    }
+  }
+}
+
+// One stage (K entries 32 s ..; complex: 16 entries) of the rows' digits at d, slices
+// `stride` bytes apart.  Real: a thread cuts eight entries of a row; complex: eight
+// real and eight imaginary parts (half the threads).
+template <int OP, typename T>
+__device__ __forceinline__ void tw_cut_a(const BoxRec<T>& R, int i0, int rows, int K, int s, const int* reb,
+                                         unsigned char* d, size_t stride) {
+  size_t si, sl;
+  const T* A = tw_mat<OP>(R, si, sl);
+  constexpr bool cplx = sizeof(T) != sizeof(double);
+  constexpr int G = cplx ? 2 : 4;   // groups of eight entries of a stage
+  const int tid = threadIdx.x;
+  if (tid >= TW_M * G) return;
+  const int i = tw_k_contiguous(OP) ? tid / G : tid % TW_M, kg = tw_k_contiguous(OP) ? tid % G : tid / TW_M;
+  if (i >= ((rows + 7) & ~7)) return;
+  const int l0 = s * 8 * G + kg * 8, eb = i < rows ? reb[i] : 1;
+  const T* a = A + (size_t)(i0 + i) * si + (size_t)l0 * sl;
+  T v[8];
+#pragma unroll
+  for (int e = 0; e < 8; ++e) v[e] = (i < rows && l0 + e < K) ? a[(size_t)e * sl] : zero<T>();
+  long long X[8];
+  if constexpr (!cplx) {
+#pragma unroll
+    for (int e = 0; e < 8; ++e) X[e] = oz_scaled_int(v[e], eb);
+    tw_put8(X, d + tw_at(i, kg), stride, 0u);
+  } else {
+#pragma unroll
+    for (int e = 0; e < 8; ++e) X[e] = oz_scaled_int(v[e].x, eb);
+    tw_put8(X, d + tw_at(i, kg), stride, 0u);
+#pragma unroll
+    for (int e = 0; e < 8; ++e) X[e] = oz_scaled_int(v[e].y, eb);
+    tw_put8(X, d + tw_at(i, 2 + kg), stride, 0u);
+  }
+}
+
+// Digits of the four matrices of a real box, in the stages' layout: for the rows of
+// tile t (128 rows, the last one rounded up to 8) and stage s, slice p at
+// base + off(t) + (s * 8 + p) * rows8 * 64.
+__host__ __device__ inline size_t tw_tile_off(int t, int K) { return (size_t)t * TW_M * ((K + TW_K - 1) / TW_K) * (OZ_S * TW_K * 2); }
+inline size_t tw_cache_bytes(int rows, int K) {
+  return (size_t)((rows + 7) & ~7) * ((K + TW_K - 1) / TW_K) * (OZ_S * TW_K * 2);
+}
+template <int OP>
+__global__ void __launch_bounds__(TW_NT) k_tw_cache(const BoxRec<double>* __restrict__ recs, const SliceRec* __restrict__ sl) {
+  __shared__ int reb[TW_M];
+  __shared__ unsigned long long scr[TW_NT];
+  const BoxRec<double> R = recs[blockIdx.y];
+  const SliceRec S = sl[blockIdx.y];
+  const int M = tw_rows<OP>(R), K = tw_inner<OP>(R), i0 = blockIdx.x * TW_M, rows = min(TW_M, M - i0);
+  if (rows <= 0) return;
+  tw_row_exps<OP>(R, i0, rows, 0, K, reb, scr);
+  __syncthreads();
+  const int rows8 = (rows + 7) & ~7;
+  unsigned char* base = S.dig[OP] + tw_tile_off(blockIdx.x, K);
+  for (int s = 0; s * TW_K < K; ++s)
+    tw_cut_a<OP>(R, i0, rows, K, s, reb, base + (size_t)s * OZ_S * rows8 * 64, (size_t)rows8 * 64);
+  for (int i = threadIdx.x; i < rows; i += TW_NT) S.eb[OP][i0 + i] = reb[i];
+}
+
+// Shared memory of a launch: NST stages of the rows' digits (rows8 rows) and of 2 GW
+// real columns, then the places in x of the K rows.
+struct TwPlan {
+  int rows8, nst, smem;
+};
+inline TwPlan tw_plan(int max_rows, int max_k, int gw, int ks) {
+  TwPlan p;
+  p.rows8 = std::min(TW_M, (max_rows + 7) & ~7);
+  const int st = p.rows8 * OZ_S * TW_K * 2 + OZ_S * 2 * gw * TW_K * 2, ns = (max_k + ks - 1) / ks;
+  // the products of a short tile read (and ignore) up to 128 rows past each slice
+  const int tail = sizeof(int) * max_k + (TW_M - p.rows8) * 64;
+  p.nst = std::max(2, std::min({4, std::max(ns, 2), (222 * 1024 - tail) / st}));
+  p.smem = p.nst * st + tail;
+  return p;
+}
+
+// GW: columns of a group (32, or 16 for classes of few boxes: more and shorter CTAs)
+template <typename T, int OP, bool CACHE, int GW>
+__global__ void __launch_bounds__(TW_NT, 1) k_tw(const BoxRec<T>* __restrict__ recs, const SliceRec* __restrict__ sl,
+                                                 T* __restrict__ x, int64_t ldx, int nrhs, int srows, int nst, int* err) {
+  extern __shared__ __align__(1024) unsigned char sm[];
+  constexpr bool cplx = sizeof(T) != sizeof(double);
+  constexpr int KS = cplx ? TW_K / 2 : TW_K;       // entries of K per stage
+  constexpr int NC = cplx ? GW : 2 * GW;           // right-hand sides per CTA
+  constexpr int BG = OZ_S * GW * TW_K * 2;         // bytes of a group's stage
+  constexpr int CT = GW / 4;                       // columns of a group per thread
+  constexpr int LDO = NC + 1;
+  __shared__ __align__(8) uint64_t mb_mma[4], mb_full[4];
+  __shared__ uint32_t s_tmem;
+  __shared__ int s_ok, reb[TW_M], ceb[NC];
+  __shared__ unsigned long long scr[TW_NT];
+  const BoxRec<T> R = recs[blockIdx.z];
+  const int M = tw_rows<OP>(R), Kall = tw_inner<OP>(R), k = R.k;
+  // the down sweep's long inner dimension: a cluster of CTAs, each a range of stages
+  const int spl = OP == TW_DNF ? (int)cooperative_groups::this_cluster().num_blocks() : 1;
+  const int rank = OP == TW_DNF ? (int)cooperative_groups::this_cluster().block_rank() : 0;
+  const int tile0 = blockIdx.x / spl, i0 = tile0 * TW_M, rows = min(TW_M, M - i0);
+  const int nsall = (Kall + KS - 1) / KS, s0 = nsall * rank / spl, ns = nsall * (rank + 1) / spl - s0;
+  const int K0 = s0 * KS, K = min(Kall, (s0 + ns) * KS);   // this CTA's entries of K
+  pdl_launch();
+  if (rows <= 0) return;
+  const int q0 = blockIdx.y * NC, nq = min(NC, nrhs - q0);
+  const int gn = cplx || nq > GW ? 2 : 1;   // groups that hold columns
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int uwarp = __shfl_sync(0xffffffffu, warp, 0);   // (uniform)
+  T* xq = x + q0;
+  const int ABYTES = srows * OZ_S * TW_K * 2, ST = ABYTES + 2 * BG;   // (srows: of the launch)
+  int* kx = reinterpret_cast<int*>(sm + (size_t)nst * ST + (TW_M - srows) * 64);
+  const unsigned char* dig = nullptr;
+  const int rows8 = (rows + 7) & ~7;
+  if (CACHE) {
+    dig = sl[blockIdx.z].dig[OP] + tw_tile_off(tile0, Kall);
+    for (int i = tid; i < rows; i += TW_NT) reb[i] = sl[blockIdx.z].eb[OP][i0 + i];
+  } else {
+    tw_row_exps<OP>(R, i0, rows, K0, K, reb, scr);
+  }
+  if (tid < 4) {
+    mbar_init(&mb_mma[tid], 1);
+    mbar_init(&mb_full[tid], 1);
+  }
+  if (tid == 0) s_ok = 1;
+  if (warp == 0) tmem_alloc(&s_tmem, 16 * GW);
+  // where the entries of the right-hand side's K rows sit in x
+  for (int l = K0 + tid; l < K; l += TW_NT)
+    kx[l] = OP == TW_DNF ? R.idxC[l] : OP == TW_UPW ? (l < k ? R.idxC[l] : R.idxR[l - k]) : R.idxR[l];
+  const int pd = nst > 2 ? nst - 2 : 1;   // stages fetched ahead
+  auto fetch_a = [&](int s) {   // (thread 0)
+    const int b = s % nst;
+    mbar_expect_tx(&mb_full[b], (uint32_t)(OZ_S * rows8 * 64));
+    for (int p = 0; p < OZ_S; ++p)
+      bulk_g2s(sm + (size_t)b * ST + p * srows * 64, dig + ((size_t)(s0 + s) * OZ_S + p) * rows8 * 64, rows8 * 64, &mb_full[b]);
+  };
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  const uint32_t tmem = s_tmem;
+  int fetched = 0;
+  if (CACHE && tid == 0)
+    for (; fetched < min(ns, pd); ++fetched) fetch_a(fetched);
+  pdl_wait();
+  {   // column exponents over the whole K: lanes over columns
+    constexpr int PT = TW_NT / NC;
+    const int q = tid % NC, part = tid / NC;
+    unsigned long long mk = 0;
+    if (q < nq) {
+#pragma unroll 8
+      for (int l = K0 + part; l < K; l += PT) mk = max(mk, tw_key(ld_l2(xq + kx[l] * ldx + q)));
+    }
+    scr[tid] = mk;
+    __syncthreads();
+    if (tid < NC) {
+#pragma unroll
+      for (int p = 1; p < PT; ++p) mk = max(mk, scr[tid + p * NC]);
+      ceb[tid] = oz_emax_b(mk);
+    }
+  }
+  __syncthreads();
+  // outputs: row 32 (warp % 4) + lane, columns CT (warp / 4) .. of both groups
+  const int row = 32 * (warp & 3) + lane, cg = CT * (warp >> 2);
+  const bool live = 32 * (warp & 3) < rows;   // (warps past the tile's rows have no outputs)
+  double acc[2][CT];
+#pragma unroll
+  for (int g = 0; g < 2; ++g)
+#pragma unroll
+    for (int e = 0; e < CT; ++e) acc[g][e] = 0.0;
+  // the group sums of one stretch of K, scaled, into acc
+  auto gather = [&](bool add, auto narrow) {
+    if (!live) return;
+    const uint32_t base = tmem + ((uint32_t)(32 * (warp & 3)) << 16) + cg;
+    const int re = row < rows ? reb[row] - 1022 : 0;
+#pragma unroll
+    for (int g = 0; g < 2; ++g) {
+      if (g >= gn) break;
+      uint32_t gr[OZ_S][CT];
+#pragma unroll
+      for (int u = 0; u < OZ_S; ++u) tmem_ldn<CT>(gr[u], base + (OZ_S * GW) * g + GW * u);
+      tmem_ld_wait();
+#pragma unroll
+      for (int e = 0; e < CT; ++e) {
+        const int col = cplx ? cg + e : GW * g + cg + e;
+        const double v = oz_ldexp_int(tw_join(gr, e, narrow), re + (ceb[col] - 1022) - 53);
+        acc[g][e] = add ? acc[g][e] + v : v;
+      }
+    }
+  };
+  // the threads that cut columns: (column, group of eight entries, complex: part)
+  const int tb = tid - (TW_NT - NC * 4);
+  const int bq = tb & (NC - 1), bg = (tb / NC) & (cplx ? 1 : 3), bim = cplx ? tb / (2 * NC) : 0;
+  const int beb = tb >= 0 ? ceb[bq] : 1;
+  double bv[8];
+  auto load_b = [&](int s) {
+    const double* xc = reinterpret_cast<const double*>(xq + bq) + bim;
+    const int l0 = (s0 + s) * KS + bg * 8;
+#pragma unroll
+    for (int e = 0; e < 8; ++e) bv[e] = (bq < nq && l0 + e < K) ? __ldcg(xc + (cplx ? 2 : 1) * (kx[l0 + e] * ldx)) : 0.0;
+  };
+  if (tb >= 0) load_b(0);
+  // the products of stage s are done (each thread polls; a wait that runs out ends the CTA's work)
+  auto wait_mma = [&](int s) {
+    if (!mbar_wait(&mb_mma[s % nst], (s / nst) & 1, TW_POLLS)) s_ok = 0;
+  };
+  int ok = 1;
+  for (int s = 0; s < ns; ++s) {
+    const int b = s % nst;
+    unsigned char* As = sm + (size_t)b * ST;
+    unsigned char* Bs = As + ABYTES;
+    const bool fresh = (s * TW_K) % TW_KX == 0;   // the group sums start over
+    if (s >= nst) wait_mma(s - nst);              // the products that read this buffer
+    if (CACHE && tid == 0 && fetched < ns && s + pd < ns) {
+      if (s + pd >= nst) wait_mma(s + pd - nst);
+      fetch_a(fetched);
+      ++fetched;
+    }
+    if (fresh && s > 0) {   // the sums of the stretch of K before this stage
+      wait_mma(s - 1);
+      tc_fence_after();
+      gather(s > TW_KX / TW_K, std::false_type{});
+      tc_fence_before();
+    }
+    if (!CACHE) tw_cut_a<OP>(R, i0, rows, K, s0 + s, reb, As, srows * 64);
+    // columns: eight entries of K per thread, those of the next stage loaded meanwhile
+    if (tb >= 0) {
+      long long X[8];
+#pragma unroll
+      for (int e = 0; e < 8; ++e) X[e] = oz_scaled_int(bv[e], beb);
+      load_b(s + 1);
+      if constexpr (!cplx) {
+        tw_put8(X, Bs + (bq / GW) * BG + tw_at(bq % GW, bg), GW * 64, 0u);
+      } else if (!bim) {   // real parts: real outputs at the first half of the stage, imaginary ones at the second
+        tw_put8(X, Bs + tw_at(bq, bg), GW * 64, 0u);
+        tw_put8(X, Bs + BG + tw_at(bq, 2 + bg), GW * 64, 0u);
+      } else {
+        tw_put8(X, Bs + tw_at(bq, 2 + bg), GW * 64, 0x80008000u);
+        tw_put8(X, Bs + BG + tw_at(bq, bg), GW * 64, 0u);
+      }
+    }
+    fence_async_smem();
+    tc_fence_before();
+    __syncthreads();
+    ok = s_ok;
+    if (!ok) break;
+    if (uwarp == 0) {
+      // (a copy that never lands leaves the stage without products)
+      const bool got = !CACHE || mbar_wait(&mb_full[b], (s / nst) & 1, TW_POLLS);
+      __syncwarp();
+      if (!got) s_ok = 0;
+      tc_fence_after();
+      const uint32_t lead = __all_sync(0xffffffffu, got) ? elect_one() : 0u;
+      const uint32_t al = umma_lo(smem_u32(As)), bl = umma_lo(smem_u32(Bs));
+#pragma unroll
+      for (int h = 0; h < TW_K / 16; ++h)
+#pragma unroll
+        for (int g = 0; g < 2; ++g) {
+          if (g >= gn) break;
+#pragma unroll
+          for (int p = 0; p < OZ_S; ++p)
+            umma_bf16_w(tmem + OZ_S * GW * g + GW * p, al + (uint32_t)(p * srows * 4 + h * 16),
+                        bl + (uint32_t)(g * (BG / 16) + h * 16), umma_idesc_bf16(TW_M, GW * (OZ_S - p)),
+                        (fresh && h == 0 && p == 0) ? 0u : 1u, lead);
+        }
+      umma_commit_w(&mb_mma[b], lead);
+      __syncwarp();
+    }
+  }
+  __syncthreads();   // (s_ok of the last stage)
+  ok = ok && s_ok;
+  if (ok && ns > 0) wait_mma(ns - 1);
+  __syncthreads();
+  ok = ok && s_ok;
+  tc_fence_after();
+  if (ok) {
+    if (ns > 0) {
+      if ((ns - 1) % (TW_KX / TW_K) < TW_KN / TW_K) gather(ns > TW_KX / TW_K, std::true_type{});
+      else gather(ns > TW_KX / TW_K, std::false_type{});
+    }
+    // a column that holds an infinity or a NaN gives NaN
+#pragma unroll
+    for (int g = 0; g < 2; ++g)
+#pragma unroll
+      for (int e = 0; e < CT; ++e)
+        if (ceb[cplx ? cg + e : GW * g + cg + e] == 2047) acc[g][e] = __longlong_as_double(0x7FF8000000000000ll);
+    // through shared memory (the stages are free), so that a warp handles the columns
+    // of one point side by side
+    T* tile = reinterpret_cast<T*>(sm);
+    if (live) {
+#pragma unroll
+      for (int e = 0; e < CT; ++e) {
+        if constexpr (cplx) {
+          tile[row * LDO + cg + e] = zd{acc[0][e], acc[1][e]};
+        } else {
+          tile[row * LDO + cg + e] = acc[0][e];
+          tile[row * LDO + GW + cg + e] = acc[1][e];
+        }
+      }
+    }
+  } else if (tid == 0) {
+    atomicExch(err, (int)RSS_ETIMEOUT);
+    // what is in flight (products, copies) ends before the buffers and the tensor memory go
+    for (int b = 0; b < nst; ++b)
+      for (int ph = 0; ph < 2; ++ph) mbar_wait(&mb_mma[b], ph, TW_DRAIN / 64);
+    if (CACHE)
+      for (int q = max(0, fetched - nst); q < fetched; ++q) mbar_wait(&mb_full[q % nst], (q / nst) & 1, TW_DRAIN);
+  }
+  if (spl > 1) cooperative_groups::this_cluster().sync();
+  else __syncthreads();
+  if (ok) {
+    // (of a cluster: each CTA the sums of a share of the rows, parts added in order)
+    const T* tile = reinterpret_cast<const T*>(sm);
+    const int ra = rows * rank / spl, rb = rows * (rank + 1) / spl;
+    constexpr int RPW = 32 / (NC < 32 ? NC : 32);   // rows of a warp at a time
+    for (int i = ra + warp * RPW + lane / NC; i < rb; i += TW_NT / 32 * RPW) {
+      const int o = i0 + i;
+      const int64_t gi = OP == TW_UPE ? R.idxC[o] : OP == TW_DNW ? (o < k ? R.idxC[o] : R.idxR[o - k]) : R.idxR[o];
+      const bool keep = OP == TW_UPE || OP == TW_DNF || (OP == TW_DNW && o < k);
+#pragma unroll
+      for (int c0 = 0; c0 < NC; c0 += 32) {
+        const int q = c0 + (lane & (NC - 1));
+        if (q < nq) {
+          T v = tile[i * LDO + q];
+          if (spl > 1) {
+            v = zero<T>();
+            for (int j = 0; j < spl; ++j) v = v + cooperative_groups::this_cluster().map_shared_rank(tile, j)[i * LDO + q];
+          }
+          T* g = xq + gi * ldx + q;
+          *g = !keep ? v : (OP == TW_UPE || OP == TW_DNF) ? ld_l2(g) - v : ld_l2(g) + v;
+        }
+      }
+    }
+  }
+  if (spl > 1) cooperative_groups::this_cluster().sync();   // (the parts have been read)
+  tc_fence_before();
+  __syncthreads();
+  if (warp == 0) tmem_free(tmem, 16 * GW);
+}

@@ -27,14 +27,14 @@ def test_panels_and_forms_give_the_bits_of_single_columns(kind, side, leaf, eps)
     tree = P.rss_build_tree(W.grid_points(side), leaf)
     arg = dict(kind=P.HELMHOLTZ if cplx else P.LAPLACE, eps=eps, h=1.0 / side, kappa=25.0 if cplx else 0.0)
     f = P.rss_factor(tree, **arg)
-    b = W.gaussian_rhs(side * side, 31, cplx, 21)
+    b = W.gaussian_rhs(side * side, 15, cplx, 21)
     bt = torch.from_numpy(np.ascontiguousarray(b.T)).cuda().T
     one = {}
-    for j in (0, 2, 4, 8, 30):
+    for j in (0, 2, 4, 8, 14):
         one[j] = P.rss_solve(f, bt[:, j].clone())
     r = P.rss_matvec(f, one[0]) - bt[:, 0]
     assert float(torch.linalg.vector_norm(r) / torch.linalg.vector_norm(bt[:, 0])) <= 10 * eps
-    for nrhs in (3, 5, 9, 31):
+    for nrhs in (3, 5, 9, 15):
         x = P.rss_solve(f, bt[:, :nrhs].T.clone().T)   # (the solve overwrites its argument)
         for j in one:
             if j < nrhs:
