@@ -283,16 +283,18 @@ __device__ __forceinline__ int oz_fint(float g) {
 // Eight group sums G_u (g(u), integers in FP32) as W = sum_u G_u 2^(39-7u), the pairs
 // (G_u 2^7 + G_{u+1}) 2^(32-7u) exact in 32 bits, the last one rounded to weight 1.
 // WIDE: for |G_u| up to 2^24 instead of 2^22 (a conversion in place of an addition).
-template <bool WIDE = false, class G> __device__ __forceinline__ long long oz_join(G g) {
+// X: that many more bits below the weight of W, whose value is then W 2^(.. - X); over K
+// entries, |W| <= K 2^(53 + X).
+template <bool WIDE = false, int X = 0, class G> __device__ __forceinline__ long long oz_join(G g) {
   int v[4];
 #pragma unroll
   for (int u = 0; u < 4; ++u) {
     const float f0 = g(2 * u), f1 = g(2 * u + 1);
     v[u] = WIDE ? __float2int_rn(f0) * 128 + __float2int_rn(f1) : oz_fint(f0) * 128 + oz_fint(f1);
   }
-  long long w = ((long long)v[0] << 32) + ((v[3] + 512) >> 10);
-  asm("mad.wide.s32 %0, %1, 262144, %0;\n" : "+l"(w) : "r"(v[1]));
-  asm("mad.wide.s32 %0, %1, 16, %0;\n" : "+l"(w) : "r"(v[2]));
+  long long w = ((long long)v[0] << (32 + X)) + ((v[3] + (1 << (9 - X))) >> (10 - X));
+  asm("mad.wide.s32 %0, %1, %2, %0;\n" : "+l"(w) : "r"(v[1]), "n"(1 << (18 + X)));
+  asm("mad.wide.s32 %0, %1, %2, %0;\n" : "+l"(w) : "r"(v[2]), "n"(1 << (4 + X)));
   return w;
 }
 static_assert(OZ_S == 8 && OZ_BITS == 7, "");

@@ -82,7 +82,7 @@ __global__ void __launch_bounds__(NT) k_perm_out(T* __restrict__ b, int64_t ldb,
 #include "sweep_tc.cuh"
 
 // Right-hand sides from which a call takes the tensor-core sweeps.  16 complex columns at
-// 256^2: 6.0 ms against 15.8 in FP64; 16 real ones: 3.3 ms against 4.6 (with the classes
+// 256^2: 7 ms against 15.8 in FP64; 16 real ones: 3.4 ms against 4.6 (with the classes
 // of fewer than TCMIN boxes, where four launches of the products take longer than one of
 // the FP64 sweep, left to the latter; at 64^2 every class).  From TCB on a real factor
 // keeps its digits, which a first call builds, and all classes that fit take the products.
@@ -352,7 +352,7 @@ SliceSize slice_size(const BoxRec<double>& R) {
   SliceSize s;
   for (int op = 0; op < 4; ++op) {
     s.dig[op] = al(tw_cache_bytes(rows[op], inner[op]));
-    s.eb[op] = al(sizeof(int) * rows[op]);
+    s.eb[op] = al(sizeof(int) * rows[op] * ((inner[op] + TW_KX - 1) / TW_KX));
   }
   return s;
 }
@@ -431,7 +431,7 @@ cudaError_t launch_tw_gw(const Batch& b, const SliceRec* sl, T* x, int64_t ldx, 
   constexpr bool real = sizeof(T) == sizeof(double);
   const int mr = OP == TW_UPE ? std::max(1, b.max_c) : OP == TW_DNW ? b.max_n : b.max_r;
   const int mk = OP == TW_UPW ? b.max_n : OP == TW_DNF ? b.max_c : b.max_r;
-  const TwPlan p = tw_plan(mr, mk, GW, real ? TW_K : TW_K / 2);
+  const TwPlan p = tw_plan(mr, mk, GW, real ? TW_K : TW_K / 2, tw_stretch<T>());
   const cudaError_t e = cudaFuncSetAttribute(k_tw<T, OP, CACHE, GW>, cudaFuncAttributeMaxDynamicSharedMemorySize, p.smem);
   if (e != cudaSuccess) return e;
   // a property of the class alone, so that a column's bits do not depend on the others
@@ -439,7 +439,7 @@ cudaError_t launch_tw_gw(const Batch& b, const SliceRec* sl, T* x, int64_t ldx, 
   if (OP == TW_DNF)
     while (spl < 8 && b.nrec * spl <= 76 && mk >= 16 * spl * (real ? TW_K : TW_K / 2)) spl *= 2;
   return launch_pdl(k_tw<T, OP, CACHE, GW>, dim3(spl * cdiv(mr, TW_M), cdiv(nrhs, real ? 2 * GW : GW), b.nrec), TW_NT,
-                    p.smem, st, spl, static_cast<const BoxRec<T>*>(b.d_recs), sl, x, ldx, nrhs, p.rows8, p.nst, err);
+                    p.smem, st, spl, static_cast<const BoxRec<T>*>(b.d_recs), sl, x, ldx, nrhs, p.rows8, p.nst, p.nstr, err);
 }
 
 // 16 columns to a group where 32 would leave half of the SMs without a CTA

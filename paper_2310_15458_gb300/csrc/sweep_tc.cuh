@@ -3,17 +3,17 @@
 // two down, z = y_R - F y_C into y_R and [y_S; y_R] = [y_S; 0] + W_E y_R (see
 // sweep.cuh), each a launch of one CTA per box, 128 rows of the matrix and TW_NC real
 // columns.  Rows of the matrix and columns of the right-hand sides are scaled by
-// powers of two over the whole inner dimension K and cut into eight signed 7-bit
+// powers of two over stretches of K (tw_stretch) and cut into eight signed 7-bit
 // digits; the slice products of equal weight u = p + q <= 7 are summed exactly in
-// FP32 in tensor memory over at most TW_KX entries of K, gathered into one int64 per
+// FP32 in tensor memory over a stretch, gathered into one int64 per
 // output and added in FP64: the accuracy of an FP64 product.  A complex product is
 // the real one with K doubled, [A_re A_im] times [B_re; -B_im] and [B_im; B_re]: the
 // two column groups of a CTA are then the real and imaginary parts of 32 columns.
 //
 // K is staged 32 at a time in two to four buffers, so the digits of one stage are cut
 // while the products of the others run; the down sweep's F y_C (K = c, up to thousands)
-// is split over a cluster of up to 8 CTAs where a class has few boxes, each with scales
-// of its own range of K, and the parts are added in order.  A column that holds an
+// is split over a cluster of up to 8 CTAs where a class has few boxes, and the
+// parts are added in order.  A column that holds an
 // infinity or a NaN gives NaN.  Real factors keep the matrices' digits (SliceRec, built
 // by the first call of 32 and more columns), which then come by bulk copies; with fewer
 // columns and for complex factors they are cut on the fly.
@@ -21,11 +21,17 @@
 // Bound by the products (36 slice pairs for 54 bits: about 80 clocks an instruction,
 // close to the tensor peak) and the gathering of x in the large classes, by latency
 // (about 20 us a launch) in the coarse ones.  64 columns, against mma.sync products of
-// one CTA per box (real) and the FP64 sweeps (complex): Laplace 512^2 23.3 -> 9.1 ms,
-// Helmholtz 256^2 30.3 -> 9.9 ms; 16 columns, against the FP64 sweeps: 4.6 -> 3.3 ms
-// (Laplace 256^2) and 15.8 -> 6.0 ms (Helmholtz 256^2).
+// one CTA per box (real) and the FP64 sweeps (complex): Laplace 512^2 23.3 -> 9.2 ms,
+// Helmholtz 256^2 30.3 -> 11.9 ms; 16 columns, against the FP64 sweeps: 4.6 -> 3.4 ms
+// (Laplace 256^2).
 constexpr int TW_MAXN = 128;                             // rows of the products that write what they read
 constexpr int TW_MAXC = 6000;                            // entries of K whose places fit beside the stages
+// Stages of K that share scales and sums.  Complex sums restart more often: against the
+// records applied in quadruple precision (Helmholtz, 64^2, leaf 64) a panel's error is
+// then 9.8e-16, of one-column FP64 solves 1.00e-15; stretches of 128, 192 and 384 give
+// 1.06e-15, 1.08e-15 and 1.14e-15, in 11.0, 10.7 and 10.2 ms instead of 11.9 (256^2, 64
+// columns).  Laplace: 3.34e-16, FP64 3.36e-16.
+template <typename T> __host__ __device__ constexpr int tw_stretch() { return (sizeof(T) == sizeof(double) ? TW_KX : TW_KN) / TW_K; }
 enum { TW_UPW = 0, TW_UPE = 1, TW_DNF = 2, TW_DNW = 3 };
 
 // rows and inner dimension of a product
@@ -44,31 +50,31 @@ template <int OP, typename T> __device__ __forceinline__ const T* tw_mat(const B
 }
 constexpr bool tw_k_contiguous(int op) { return op == TW_UPW || op == TW_DNF; }
 
-// The CTA's rows i0 .. of the matrix: exponents (biased, at least 1) of the largest of
-// their entries K0 .. K, into reb[TW_M].  scr: 512 keys of shared memory.
+// Exponents (biased, at least 1) of the largest of the entries K0 .. K of the CTA's rows
+// i0 .., for each stretch st of K (from the one of K0 on), into reb[st * TW_M + i], which
+// holds 1s.  (A barrier must follow.)
 template <int OP, typename T>
-__device__ void tw_row_exps(const BoxRec<T>& R, int i0, int rows, int K0, int K, int* reb, unsigned long long* scr) {
+__device__ void tw_row_exps(const BoxRec<T>& R, int i0, int rows, int K0, int K, int* reb) {
+  constexpr int KX = tw_stretch<T>() * (sizeof(T) == sizeof(double) ? TW_K : TW_K / 2);
   size_t si, sl;
   const T* A = tw_mat<OP>(R, si, sl);
   const int tid = threadIdx.x;
-  if (tw_k_contiguous(OP)) {   // a warp per row
-    for (int i = tid / 32; i < rows; i += TW_NT / 32) {
+  for (int l0 = K0, st = 0; l0 < K; l0 = (l0 / KX + 1) * KX, ++st) {
+    const int l1 = min(K, (l0 / KX + 1) * KX);
+    if (tw_k_contiguous(OP)) {   // a warp per row
+      for (int i = tid / 32; i < rows; i += TW_NT / 32) {
+        unsigned long long mk = 0;
+        for (int l = l0 + tid % 32; l < l1; l += 32) mk = max(mk, tw_key(A[(i0 + i) * si + l]));
+        mk = shfl_max_u64(mk, 32);
+        if (tid % 32 == 0) reb[st * TW_M + i] = oz_emax_b(mk);
+      }
+    } else {                     // four threads per row, lanes over rows
+      const int i = tid % TW_M, part = tid / TW_M;
       unsigned long long mk = 0;
-      for (int l = K0 + tid % 32; l < K; l += 32) mk = max(mk, tw_key(A[(i0 + i) * si + l]));
-      mk = shfl_max_u64(mk, 32);
-      if (tid % 32 == 0) reb[i] = oz_emax_b(mk);
-    }
-  } else {                     // four threads per row, lanes over rows
-    const int i = tid % TW_M, part = tid / TW_M;
-    unsigned long long mk = 0;
-    if (i < rows)
-      for (int l = K0 + part; l < K; l += TW_NT / TW_M) mk = max(mk, tw_key(A[(i0 + i) + (size_t)l * sl]));
-    scr[tid] = mk;
-    __syncthreads();
-    if (tid < TW_M) {
-#pragma unroll
-      for (int p = 1; p < TW_NT / TW_M; ++p) mk = max(mk, scr[tid + p * TW_M]);
-      reb[tid] = oz_emax_b(mk);
+      if (i < rows) {
+        for (int l = l0 + part; l < l1; l += TW_NT / TW_M) mk = max(mk, tw_key(A[(i0 + i) + (size_t)l * sl]));
+        atomicMax(&reb[st * TW_M + i], oz_emax_b(mk));
+      }
     }
   }
 }
@@ -116,32 +122,36 @@ inline size_t tw_cache_bytes(int rows, int K) {
 }
 template <int OP>
 __global__ void __launch_bounds__(TW_NT) k_tw_cache(const BoxRec<double>* __restrict__ recs, const SliceRec* __restrict__ sl) {
-  __shared__ int reb[TW_M];
-  __shared__ unsigned long long scr[TW_NT];
+  __shared__ int reb[TW_MAXC / TW_KX + 1][TW_M];
   const BoxRec<double> R = recs[blockIdx.y];
   const SliceRec S = sl[blockIdx.y];
   const int M = tw_rows<OP>(R), K = tw_inner<OP>(R), i0 = blockIdx.x * TW_M, rows = min(TW_M, M - i0);
   if (rows <= 0) return;
-  tw_row_exps<OP>(R, i0, rows, 0, K, reb, scr);
+  for (int i = threadIdx.x; i < (TW_MAXC / TW_KX + 1) * TW_M; i += TW_NT) reb[0][i] = 1;
+  __syncthreads();
+  tw_row_exps<OP>(R, i0, rows, 0, K, reb[0]);
   __syncthreads();
   const int rows8 = (rows + 7) & ~7;
   unsigned char* base = S.dig[OP] + tw_tile_off(blockIdx.x, K);
   for (int s = 0; s * TW_K < K; ++s)
-    tw_cut_a<OP>(R, i0, rows, K, s, reb, base + (size_t)s * OZ_S * rows8 * 64, (size_t)rows8 * 64);
-  for (int i = threadIdx.x; i < rows; i += TW_NT) S.eb[OP][i0 + i] = reb[i];
+    tw_cut_a<OP>(R, i0, rows, K, s, reb[s / (TW_KX / TW_K)], base + (size_t)s * OZ_S * rows8 * 64, (size_t)rows8 * 64);
+  for (int st = 0; st * TW_KX < K; ++st)
+    for (int i = threadIdx.x; i < rows; i += TW_NT) S.eb[OP][(size_t)st * M + i0 + i] = reb[st][i];
 }
 
 // Shared memory of a launch: NST stages of the rows' digits (rows8 rows) and of 2 GW
-// real columns, then the places in x of the K rows.
+// real columns, then the places in x of the K rows and the exponents of rows and
+// columns in up to nstr stretches of K.
 struct TwPlan {
-  int rows8, nst, smem;
+  int rows8, nst, nstr, smem;
 };
-inline TwPlan tw_plan(int max_rows, int max_k, int gw, int ks) {
+inline TwPlan tw_plan(int max_rows, int max_k, int gw, int ks, int sx) {
   TwPlan p;
   p.rows8 = std::min(TW_M, (max_rows + 7) & ~7);
   const int st = p.rows8 * OZ_S * TW_K * 2 + OZ_S * 2 * gw * TW_K * 2, ns = (max_k + ks - 1) / ks;
   // the products of a short tile read (and ignore) up to 128 rows past each slice
-  const int tail = sizeof(int) * max_k + (TW_M - p.rows8) * 64;
+  p.nstr = (ns + sx - 1) / sx + 1;   // (a share of K may start inside a stretch)
+  const int tail = sizeof(int) * (max_k + p.nstr * (TW_M + 2 * gw)) + (TW_M - p.rows8) * 64;
   p.nst = std::max(2, std::min({4, std::max(ns, 2), (222 * 1024 - tail) / st}));
   p.smem = p.nst * st + tail;
   return p;
@@ -150,7 +160,7 @@ inline TwPlan tw_plan(int max_rows, int max_k, int gw, int ks) {
 // GW: columns of a group (32, or 16 for classes of few boxes: more and shorter CTAs)
 template <typename T, int OP, bool CACHE, int GW>
 __global__ void __launch_bounds__(TW_NT, 1) k_tw(const BoxRec<T>* __restrict__ recs, const SliceRec* __restrict__ sl,
-                                                 T* __restrict__ x, int64_t ldx, int nrhs, int srows, int nst, int* err) {
+                                                 T* __restrict__ x, int64_t ldx, int nrhs, int srows, int nst, int nstr, int* err) {
   extern __shared__ __align__(1024) unsigned char sm[];
   constexpr bool cplx = sizeof(T) != sizeof(double);
   constexpr int KS = cplx ? TW_K / 2 : TW_K;       // entries of K per stage
@@ -160,8 +170,8 @@ __global__ void __launch_bounds__(TW_NT, 1) k_tw(const BoxRec<T>* __restrict__ r
   constexpr int LDO = NC + 1;
   __shared__ __align__(8) uint64_t mb_mma[4], mb_full[4];
   __shared__ uint32_t s_tmem;
-  __shared__ int s_ok, reb[TW_M], ceb[NC];
-  __shared__ unsigned long long scr[TW_NT];
+  constexpr int SX = tw_stretch<T>();              // stages of a stretch of K
+  __shared__ int s_ok;
   const BoxRec<T> R = recs[blockIdx.z];
   const int M = tw_rows<OP>(R), Kall = tw_inner<OP>(R), k = R.k;
   // the down sweep's long inner dimension: a cluster of CTAs, each a range of stages
@@ -178,15 +188,23 @@ __global__ void __launch_bounds__(TW_NT, 1) k_tw(const BoxRec<T>* __restrict__ r
   const int uwarp = __shfl_sync(0xffffffffu, warp, 0);   // (uniform)
   T* xq = x + q0;
   const int ABYTES = srows * OZ_S * TW_K * 2, ST = ABYTES + 2 * BG;   // (srows: of the launch)
-  int* kx = reinterpret_cast<int*>(sm + (size_t)nst * ST + (TW_M - srows) * 64);
+  int* reb = reinterpret_cast<int*>(sm + (size_t)nst * ST + (TW_M - srows) * 64);   // stretch st, row i: st * 128 + i
+  int* ceb = reb + nstr * TW_M;                                                    // stretch st, column q: st * NC + q
+  int* kx = ceb + nstr * 2 * GW - K0;                                              // entry l of this CTA's K
+  auto stretch = [&](int s) { return (s0 + s) / SX - s0 / SX; };
   const unsigned char* dig = nullptr;
   const int rows8 = (rows + 7) & ~7;
   if (CACHE) {
     dig = sl[blockIdx.z].dig[OP] + tw_tile_off(tile0, Kall);
-    for (int i = tid; i < rows; i += TW_NT) reb[i] = sl[blockIdx.z].eb[OP][i0 + i];
+    for (int st = 0; st < nstr && (s0 / SX + st) * SX < nsall; ++st)
+      for (int i = tid; i < rows; i += TW_NT)
+        reb[st * TW_M + i] = sl[blockIdx.z].eb[OP][(size_t)(s0 / SX + st) * M + i0 + i];
   } else {
-    tw_row_exps<OP>(R, i0, rows, K0, K, reb, scr);
+    for (int i = tid; i < nstr * TW_M; i += TW_NT) reb[i] = 1;
+    __syncthreads();
+    tw_row_exps<OP>(R, i0, rows, K0, K, reb);
   }
+  for (int i = tid; i < nstr * NC; i += TW_NT) ceb[i] = 1;
   if (tid < 4) {
     mbar_init(&mb_mma[tid], 1);
     mbar_init(&mb_full[tid], 1);
@@ -211,21 +229,17 @@ __global__ void __launch_bounds__(TW_NT, 1) k_tw(const BoxRec<T>* __restrict__ r
   if (CACHE && tid == 0)
     for (; fetched < min(ns, pd); ++fetched) fetch_a(fetched);
   pdl_wait();
-  {   // column exponents over the whole K: lanes over columns
+  {   // column exponents of each stretch of K: lanes over columns
     constexpr int PT = TW_NT / NC;
     const int q = tid % NC, part = tid / NC;
-    unsigned long long mk = 0;
-    if (q < nq) {
+    if (q < nq)
+      for (int sa = 0, st = 0; sa < ns; sa = (s0 + sa) / SX * SX + SX - s0, ++st) {
+        const int l1 = min(K, ((s0 + sa) / SX * SX + SX) * KS);
+        unsigned long long mk = 0;
 #pragma unroll 8
-      for (int l = K0 + part; l < K; l += PT) mk = max(mk, tw_key(ld_l2(xq + kx[l] * ldx + q)));
-    }
-    scr[tid] = mk;
-    __syncthreads();
-    if (tid < NC) {
-#pragma unroll
-      for (int p = 1; p < PT; ++p) mk = max(mk, scr[tid + p * NC]);
-      ceb[tid] = oz_emax_b(mk);
-    }
+        for (int l = (s0 + sa) * KS + part; l < l1; l += PT) mk = max(mk, tw_key(ld_l2(xq + kx[l] * ldx + q)));
+        atomicMax(&ceb[st * NC + q], oz_emax_b(mk));
+      }
   }
   __syncthreads();
   // outputs: row 32 (warp % 4) + lane, columns CT (warp / 4) .. of both groups
@@ -237,10 +251,11 @@ __global__ void __launch_bounds__(TW_NT, 1) k_tw(const BoxRec<T>* __restrict__ r
 #pragma unroll
     for (int e = 0; e < CT; ++e) acc[g][e] = 0.0;
   // the group sums of one stretch of K, scaled, into acc
-  auto gather = [&](bool add, auto narrow) {
+  auto gather = [&](int st, auto narrow) {
+    constexpr int XB = cplx || decltype(narrow)::value ? 2 : 1;   // (|W| <= K 2^(53 + XB))
     if (!live) return;
     const uint32_t base = tmem + ((uint32_t)(32 * (warp & 3)) << 16) + cg;
-    const int re = row < rows ? reb[row] - 1022 : 0;
+    const int re = row < rows ? reb[st * TW_M + row] - 1022 : 0;
 #pragma unroll
     for (int g = 0; g < 2; ++g) {
       if (g >= gn) break;
@@ -251,15 +266,16 @@ __global__ void __launch_bounds__(TW_NT, 1) k_tw(const BoxRec<T>* __restrict__ r
 #pragma unroll
       for (int e = 0; e < CT; ++e) {
         const int col = cplx ? cg + e : GW * g + cg + e;
-        const double v = oz_ldexp_int(tw_join(gr, e, narrow), re + (ceb[col] - 1022) - 53);
-        acc[g][e] = add ? acc[g][e] + v : v;
+        const int ce = ceb[st * NC + col];
+        double v = oz_ldexp_int(tw_join<XB>(gr, e, narrow), re + (ce - 1022) - 53 - XB);
+        if (ce == 2047) v = __longlong_as_double(0x7FF8000000000000ll);   // an infinity or a NaN in the column
+        acc[g][e] = st > 0 ? acc[g][e] + v : v;
       }
     }
   };
   // the threads that cut columns: (column, group of eight entries, complex: part)
   const int tb = tid - (TW_NT - NC * 4);
   const int bq = tb & (NC - 1), bg = (tb / NC) & (cplx ? 1 : 3), bim = cplx ? tb / (2 * NC) : 0;
-  const int beb = tb >= 0 ? ceb[bq] : 1;
   double bv[8];
   auto load_b = [&](int s) {
     const double* xc = reinterpret_cast<const double*>(xq + bq) + bim;
@@ -277,7 +293,7 @@ __global__ void __launch_bounds__(TW_NT, 1) k_tw(const BoxRec<T>* __restrict__ r
     const int b = s % nst;
     unsigned char* As = sm + (size_t)b * ST;
     unsigned char* Bs = As + ABYTES;
-    const bool fresh = (s * TW_K) % TW_KX == 0;   // the group sums start over
+    const bool fresh = s == 0 || (s0 + s) % SX == 0;   // the group sums start over
     if (s >= nst) wait_mma(s - nst);              // the products that read this buffer
     if (CACHE && tid == 0 && fetched < ns && s + pd < ns) {
       if (s + pd >= nst) wait_mma(s + pd - nst);
@@ -287,12 +303,13 @@ __global__ void __launch_bounds__(TW_NT, 1) k_tw(const BoxRec<T>* __restrict__ r
     if (fresh && s > 0) {   // the sums of the stretch of K before this stage
       wait_mma(s - 1);
       tc_fence_after();
-      gather(s > TW_KX / TW_K, std::false_type{});
+      gather(stretch(s - 1), std::false_type{});
       tc_fence_before();
     }
-    if (!CACHE) tw_cut_a<OP>(R, i0, rows, K, s0 + s, reb, As, srows * 64);
+    if (!CACHE) tw_cut_a<OP>(R, i0, rows, K, s0 + s, reb + stretch(s) * TW_M, As, srows * 64);
     // columns: eight entries of K per thread, those of the next stage loaded meanwhile
     if (tb >= 0) {
+      const int beb = ceb[stretch(s) * NC + bq];
       long long X[8];
 #pragma unroll
       for (int e = 0; e < 8; ++e) X[e] = oz_scaled_int(bv[e], beb);
@@ -343,15 +360,10 @@ __global__ void __launch_bounds__(TW_NT, 1) k_tw(const BoxRec<T>* __restrict__ r
   tc_fence_after();
   if (ok) {
     if (ns > 0) {
-      if ((ns - 1) % (TW_KX / TW_K) < TW_KN / TW_K) gather(ns > TW_KX / TW_K, std::true_type{});
-      else gather(ns > TW_KX / TW_K, std::false_type{});
+      const int st = stretch(ns - 1);
+      if ((s0 + ns - 1) % SX < TW_KN / TW_K || ns <= TW_KN / TW_K) gather(st, std::true_type{});
+      else gather(st, std::false_type{});
     }
-    // a column that holds an infinity or a NaN gives NaN
-#pragma unroll
-    for (int g = 0; g < 2; ++g)
-#pragma unroll
-      for (int e = 0; e < CT; ++e)
-        if (ceb[cplx ? cg + e : GW * g + cg + e] == 2047) acc[g][e] = __longlong_as_double(0x7FF8000000000000ll);
     // through shared memory (the stages are free), so that a warp handles the columns
     // of one point side by side
     T* tile = reinterpret_cast<T*>(sm);

@@ -58,11 +58,11 @@ template <int N> __device__ __forceinline__ void tmem_ldn(uint32_t* v, uint32_t 
   }
 }
 // eight group sums (weights u = 0 .. 7) of one output as W, its value W 2^(row and
-// column exponents - 53); narrow: over at most TW_KN entries of K, an FP32 addition in
+// column exponents - 53 - X); narrow: over at most TW_KN entries of K, an FP32 addition in
 // place of a conversion
-template <int C, bool NARROW>
+template <int X, int C, bool NARROW>
 __device__ __forceinline__ long long tw_join(const uint32_t (&gr)[OZ_S][C], int e, std::integral_constant<bool, NARROW>) {
-  return oz_join<!NARROW>([&](int u) { return __uint_as_float(gr[u][e]); });
+  return oz_join<!NARROW, X>([&](int u) { return __uint_as_float(gr[u][e]); });
 }
 
 }  // namespace
