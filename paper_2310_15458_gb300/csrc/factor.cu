@@ -28,7 +28,6 @@
 #include <cuda_bf16.h>
 
 #include "internal.h"
-#include "tc_gemm.cuh"
 #include "tw_common.cuh"
 
 namespace {
@@ -884,7 +883,6 @@ template <typename T> struct ElimArgs {
   const T* T_ws;
   int* err;
   int smem_cap;             // scalars of dynamic shared memory available
-  int sym;                  // A is symmetric (real Laplace): A_BC^T = A_CB
 };
 
 constexpr int PKC = 16;     // rows of a panel product's right operand staged per chunk
@@ -1354,208 +1352,7 @@ template <typename T, int MA> __global__ void __launch_bounds__(NT, 2) k_elim_pa
 }
 
 
-// Real factors: the columns of W_E and W_F cut into digit slices once per box
-// (every panel CTA of the box reads them).  32 columns per CTA, eight threads per
-// column.
-__global__ void __launch_bounds__(NT) k_w_split(ElimArgs<double> a) {
-  const BoxRec<double> R = a.recs[blockIdx.x];
-  if (!R.ozp) return;
-  const int r = R.r, n = R.k + r, np = (n + 15) & ~15, rp = (r + 31) & ~31;
-  if ((int)blockIdx.y * (NT / 8) >= 2 * rp) return;
-  const int col = (int)blockIdx.y * (NT / 8) + (int)threadIdx.x / 8, pass = col / rp, j = col % rp;
-  const double* w = (pass ? R.Wf : R.We) + (size_t)j * n;
-  oz_split_vec<8>([&](int l) { return w[l]; }, j < r ? n : 0, np, R.Wsl + (size_t)col * OZ_S * np, np, &R.Wexp[col],
-                  true);
-}
-
-// Real factors: E = A_CB W_E and F^T = A_BC^T W_F for one 64-row panel of C,
-// with the panel rows and the columns of W cut into digit slices (row and
-// column scales) and the slice products summed exactly on the tensor cores as
-// in the Schur update; E (F^T) = W 2^(e_i + f_j - 53) from one int64 per entry.
-// W is taken 32 columns at a time from its precomputed slices.  A symmetric A
-// gives A_BC^T = A_CB, so the panel is cut once for both products.  The rows of
-// E and F^T are then sliced for the Schur update.
-constexpr int OZ_NCH = 32;
-
-__global__ void __launch_bounds__(NT, 2) k_elim_oz(ElimArgs<double> a) {
-  extern __shared__ __align__(16) unsigned char smraw[];
-  const BoxRec<double> R = a.recs[blockIdx.y];
-  if (!R.ozp) return;
-  const int p0 = blockIdx.x * 64;
-  if (p0 >= R.c) return;
-  const LevelDev<double>& L = a.L;
-  const int nmax = L.nmax, g = L.g, B = R.box, k = R.k, r = R.r, c = R.c, n = k + r;
-  const int np = (n + 15) & ~15, SA = OZ_S * np + 8, rp = (r + 31) & ~31;
-  const size_t nn = (size_t)nmax * nmax;
-  const int* perm = a.perm_in + (size_t)a.cls_idx[blockIdx.y] * nmax;
-  uint16_t* As = reinterpret_cast<uint16_t*>(smraw);   // 64 x SA: panel rows
-  uint16_t* Bs = As + 64 * SA;                         // OZ_NCH x SA: columns of W
-  __shared__ int rexp[64], cexp[OZ_NCH], ru[64], rpos[64];
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, gq = lane >> 2, t4 = lane & 3;
-  const int rows = min(64, c - p0);
-  if (tid < 64) {
-    ru[tid] = -1;
-    rpos[tid] = 0;
-    if (tid < rows) {
-      const int cm = R.cmap[p0 + tid], s = cm >> 16;
-      ru[tid] = nbr_box(B, g, s % 3 - 1, s / 3 - 1);
-      rpos[tid] = cm & 0xffff;
-    }
-  }
-  __syncthreads();
-  const int m0 = (warp >> 1) * 16, n0 = (warp & 1) * 16;
-  const int a_row = lane & 15, a_k = (lane >> 4) * 8;
-  const int b_row = ((lane >> 4) << 3) + (lane & 7), b_k = ((lane >> 3) & 1) * 8;
-  const int npass = a.sym ? 1 : 2;
-  for (int pass = 0; pass < npass; ++pass) {
-    {   // panel rows: A(u, B)[pos, perm[l]] (pass 0) or A(B, u)[perm[l], pos] (pass 1)
-      const int row = tid >> 2, u = ru[row], pos = rpos[row];
-      const double* base = nullptr;
-      if (u >= 0)
-        base = pass == 0 ? L.blk + ((size_t)u * 25 + off_index(u, B, g)) * nn + pos
-                         : L.blk + ((size_t)B * 25 + off_index(B, u, g)) * nn + (size_t)pos * nmax;
-      const size_t ls = pass == 0 ? (size_t)nmax : 1;
-      oz_split_vec<4>([&](int l) { return base[(size_t)perm[l] * ls]; }, u >= 0 ? n : 0, np, As + row * SA, np,
-                      &rexp[row], true);
-    }
-    // columns of [W_E W_F] (symmetric A) or of the pass's W
-    const int c_lo = a.sym ? 0 : pass * rp, c_hi = a.sym ? 2 * rp : (pass + 1) * rp;
-    for (int cc = c_lo; cc < c_hi; cc += OZ_NCH) {
-      const int j0 = cc % rp;
-      if (j0 >= r) continue;   // padding columns only
-      __syncthreads();
-      {   // one (column, slice) row of the chunk's W slices per thread
-        const int col = tid >> 3, sl = tid & 7;
-        const uint16_t* src = R.Wsl + (size_t)(cc + col) * OZ_S * np + (size_t)sl * np;
-        uint16_t* dst = Bs + col * SA + sl * np;
-        for (int q = 0; q < np; q += 8) cp_async16(dst + q, src + q);
-      }
-      if (tid < OZ_NCH) cexp[tid] = R.Wexp[cc + tid];
-      cp_async_wait_all();
-      __syncthreads();
-      // all eight group sums in FP32 over the whole K (K <= 128: exact), B slices
-      // loaded four at a time with the A slices that pair with them
-      float acc[OZ_S][2][4];
-#pragma unroll
-      for (int u = 0; u < OZ_S; ++u)
-#pragma unroll
-        for (int ni = 0; ni < 2; ++ni)
-#pragma unroll
-          for (int e = 0; e < 4; ++e) acc[u][ni][e] = 0.f;
-      for (int kk = 0; kk < np; kk += 16) {
-#pragma unroll
-        for (int h = 0; h < 2; ++h) {
-          uint32_t bq[4][4];
-#pragma unroll
-          for (int q = 0; q < 4; ++q) ldsm_x4(bq[q], Bs + (4 * h + q) * np + (n0 + b_row) * SA + kk + b_k);
-#pragma unroll
-          for (int p = 0; p + 4 * h < OZ_S; ++p) {
-            uint32_t af[4];
-            ldsm_x4(af, As + p * np + (m0 + a_row) * SA + kk + a_k);
-#pragma unroll
-            for (int q = 0; q < 4; ++q)
-              if (p + 4 * h + q < OZ_S) {
-                mma_bf16(acc[p + 4 * h + q][0], af, bq[q]);
-                mma_bf16(acc[p + 4 * h + q][1], af, bq[q] + 2);
-              }
-          }
-        }
-      }
-      // W = sum_u G_u 2^(39-7u), groups u and u + 1 as (G_u 2^7 + G_{u+1}) 2^(32-7u)
-      long long W[2][4];
-#pragma unroll
-      for (int ni = 0; ni < 2; ++ni)
-#pragma unroll
-        for (int e = 0; e < 4; ++e) {
-          W[ni][e] = oz_join([&](int u) { return acc[u][ni][e]; });
-        }
-      double* out = cc < rp ? R.E : R.Ft;
-#pragma unroll
-      for (int ni = 0; ni < 2; ++ni)
-#pragma unroll
-        for (int e = 0; e < 4; ++e) {
-          const int row = m0 + gq + (e >= 2 ? 8 : 0);
-          const int col = n0 + ni * 8 + 2 * t4 + (e & 1), j = j0 + col;
-          if (row < rows && j < r)
-            out[(size_t)(p0 + row) + (size_t)j * c] = oz_ldexp_int(W[ni][e], rexp[row] + cexp[col] - 53);
-        }
-    }
-    __syncthreads();
-  }
-  if (R.Esl != nullptr) {   // digit slices of this panel's rows of E and F^T for the Schur update
-    const int row = tid >> 2;
-    const bool act = row < rows;
-    for (int q = 0; q < 2; ++q) {
-      const double* src = (q == 0 ? R.E : R.Ft) + (size_t)(p0 + row);
-      uint16_t* dst = (q == 0 ? R.Esl : R.Fsl) + (size_t)(p0 + (act ? row : 0)) * OZ_S * R.kp;
-      int* ex = (q == 0 ? R.Eexp : R.Fexp) + p0 + (act ? row : 0);
-      oz_split_vec<4>([&](int l) { return src[(size_t)l * c]; }, act ? r : 0, R.kp, dst, R.kp, ex, act);
-    }
-  }
-}
-
-// ------------------------------------------------------------------ complex E and F on the tensor cores
-
-
-// Complex factors: E = A_CB W_E and F^T = A_BC^T W_F for one 64-row panel of C
-// (any n_B: K is taken in chunks), then the rows' digit slices for the Schur
-// update.
-__global__ void __launch_bounds__(NT, 2) k_elim_ozc(ElimArgs<zd> a) {
-  extern __shared__ __align__(16) unsigned char smraw[];
-  const BoxRec<zd> R = a.recs[blockIdx.y];
-  if (!R.ozp) return;
-  const int p0 = blockIdx.x * ZCM;
-  if (p0 >= R.c) return;
-  const LevelDev<zd>& L = a.L;
-  const int nmax = L.nmax, g = L.g, B = R.box, k = R.k, r = R.r, c = R.c, n = k + r;
-  const size_t nn = (size_t)nmax * nmax;
-  const int* perm = a.perm_in + (size_t)a.cls_idx[blockIdx.y] * nmax;
-  uint16_t* As = reinterpret_cast<uint16_t*>(smraw);
-  uint16_t* Bs = As + ZCM * ZSA;
-  __shared__ int rexp[ZCM], cexp[ZCN], ru[ZCM], rpos[ZCM], sperm[256];
-  const int tid = threadIdx.x, rows = min(ZCM, c - p0);
-  if (tid < ZCM) {
-    ru[tid] = -1;
-    rpos[tid] = 0;
-    if (tid < rows) {
-      const int cm = R.cmap[p0 + tid], s = cm >> 16;
-      ru[tid] = nbr_box(B, g, s % 3 - 1, s / 3 - 1);
-      rpos[tid] = cm & 0xffff;
-    }
-  }
-  const bool pin = n <= 256;
-  if (pin)
-    for (int i = tid; i < n; i += blockDim.x) sperm[i] = perm[i];
-  __syncthreads();
-  auto pm = [&](int l) { return pin ? sperm[l] : perm[l]; };
-  for (int pass = 0; pass < 2; ++pass) {
-    const zd* __restrict__ Wm = pass == 0 ? R.We : R.Wf;
-    zd* out = pass == 0 ? R.E : R.Ft;
-    for (int jc = 0; jc < r; jc += ZCN) {
-      auto aval = [&](int i, int l) -> zd {
-        const int u = ru[i], pos = rpos[i];
-        return pass == 0 ? L.blk[((size_t)u * 25 + off_index(u, B, g)) * nn + (size_t)pm(l) * nmax + pos]
-                         : L.blk[((size_t)B * 25 + off_index(B, u, g)) * nn + (size_t)pos * nmax + pm(l)];
-      };
-      auto bval = [&](int l, int q) -> zd {
-        const int j = jc + q;
-        return j < r ? Wm[(size_t)l + (size_t)j * n] : zd{0.0, 0.0};
-      };
-      tc_gemm_c(rows, n, aval, bval,
-                [&](int i, int q, zd v) {
-                  const int j = jc + q;
-                  if (j < r) out[(size_t)(p0 + i) + (size_t)j * c] = v;
-                },
-                As, Bs, rexp, cexp);
-    }
-    if (R.Esl != nullptr) {   // digit slices of this panel's rows for the Schur update
-      for (int e = tid; e < rows; e += blockDim.x)
-        oz_split_row(out + p0 + e, c, r, R.kp, (pass == 0 ? R.Esl : R.Fsl) + (size_t)(p0 + e) * 2 * OZ_S * R.kp,
-                     (pass == 0 ? R.Eexp : R.Fexp) + p0 + e);
-      __syncthreads();
-    }
-  }
-}
+#include "elim_panels.cuh"
 
 // ------------------------------------------------------------------ Schur update A_CC -= E F
 template <typename T> __global__ void __launch_bounds__(NT) k_schur(LevelDev<T> L, const BoxRec<T>* recs) {
@@ -3072,42 +2869,40 @@ rss_status factor_impl(const rss_tree* tree, const rss_params* prm, cudaStream_t
           R.panels = pb <= 200 * 1024 ? 1 : 0;
         }
       }
-      // E = A_CB W_E and F^T = A_BC^T W_F on the tensor cores: real factors,
-      // n <= 128 (the slices of a 64-row panel and of 32 columns of W fit in
-      // shared memory)
-      // (complex factors: any n_B, K taken in chunks by k_elim_ozc)
-      int ozp_np = 0;
-      const int ozp_nmax = sizeof(T) == sizeof(double) ? 128 : (1 << 30);
-      // (real factors also keep the digit slices of the columns of W_E and W_F)
-      auto wsl_bytes = [&](const BoxRec<T>& R) -> size_t {
-        if (sizeof(T) != sizeof(double)) return 0;
-        const size_t np = (R.k + R.r + 15) & ~15, rp = (R.r + 31) & ~31;
-        return ((2 * rp * OZ_S * np * sizeof(uint16_t) + 255) & ~size_t(255)) + ((2 * rp * sizeof(int) + 255) & ~size_t(255));
-      };
+      // E = A_CB W_E and F^T = A_BC^T W_F on the tensor cores (elim_panels.cuh): real
+      // boxes up to the n whose digits stay in shared memory, complex ones up to the n
+      // whose rows' exponents do
+      const bool sym = sizeof(T) == sizeof(double) && prm->kind == RSS_LAPLACE;
+      EpArgs<T> ep = {};
+      int ep_r = 0, ep_n = 0;
       if (prm->schur_path == 0 || prm->schur_path == 2) {
-        size_t bytes = 0;
-        for (const BoxRec<T>& R : recs)
-          if (R.k + R.r <= ozp_nmax) bytes += wsl_bytes(R);
-        {
-          if (!gb_w.ensure(bytes)) {
-            rss_set_error("rss_factor: device workspace allocation failed");
-            return RSS_ENOMEM;
-          }
-          char* p = static_cast<char*>(gb_w.p);
-          for (BoxRec<T>& R : recs) {
-            if (R.k + R.r > ozp_nmax) continue;
-            if (sizeof(T) == sizeof(double)) {
-              const size_t np = (R.k + R.r + 15) & ~15, rp = (R.r + 31) & ~31;
-              const size_t bs = (2 * rp * OZ_S * np * sizeof(uint16_t) + 255) & ~size_t(255);
-              R.Wsl = reinterpret_cast<uint16_t*>(p);
-              R.Wexp = reinterpret_cast<int*>(p + bs);
-              p += wsl_bytes(R);
-            }
-            R.ozp = 1;
-            ozp_np = std::max(ozp_np, (R.k + R.r + 15) & ~15);
-          }
-          f->peak_transient = std::max(f->peak_transient, transient + bytes);
+        constexpr int ozp_nmax = sizeof(T) == sizeof(double) ? 4 * TW_K : 3840;
+        for (BoxRec<T>& R : recs) {
+          if (R.k + R.r > ozp_nmax) continue;
+          R.ozp = 1;
+          ep_r = std::max(ep_r, R.r);
+          ep_n = std::max(ep_n, R.k + R.r);
         }
+      }
+      if (ep_n > 0) {
+        ep.sets = sym ? 1 : 2;
+        ep.ns = cdiv(ep_n, ep_ks<T>());
+        ep.ng = cdiv(sym ? 2 * ep_r : ep_r, 32);
+        ep.nstr = cdiv(ep.ns, ep_smax<T>());
+        ep.o_ew = (size_t)ep.sets * ep.ng * ep.ns * ep_parts<T>() * EP_GB;
+        ep.slot = (ep.o_ew + (size_t)ep.sets * ep.ng * ep.nstr * 32 * sizeof(int) + 255) & ~size_t(255);
+        if (!gb_w.ensure(ep.slot * nrec)) {
+          rss_set_error("rss_factor: device workspace allocation failed");
+          return RSS_ENOMEM;
+        }
+        ep.ws = static_cast<unsigned char*>(gb_w.p);
+        f->peak_transient = std::max(f->peak_transient, transient + ep.slot * nrec);
+        // real: the tile's digits over all of K, complex: two stages of them, beside
+        // two or three stages of W and the rows' exponents
+        ep.rows = sizeof(T) == sizeof(double) && ep.ns > 3 ? 96 : TW_M;
+        ep.ad = sizeof(T) == sizeof(double) ? std::max(2, ep.ns) : 2;
+        ep.wd = sizeof(T) == sizeof(double) && ep.ns <= 2 ? 3 : 2;
+        ep.spn = TW_M;
       }
       for (const BoxRec<T>& R : recs)
         if (R.panels && !R.ozp) pan_max = std::max(pan_max, panel_smem_bytes<T>(pan_ma, R.k + R.r, R.r));
@@ -3181,7 +2976,6 @@ rss_status factor_impl(const rss_tree* tree, const rss_params* prm, cudaStream_t
       ea.perm_in = d_perm;
       ea.T_ws = d_Tws;
       ea.err = d_err;
-      ea.sym = (sizeof(T) == sizeof(double) && prm->kind == RSS_LAPLACE) ? 1 : 0;
       // shared memory of the per-box kernel: T and the LU of the largest box that fits
       const size_t ints = (2 * (size_t)max_r * sizeof(int) + 15) & ~size_t(15);
       const size_t want =
@@ -3234,21 +3028,24 @@ rss_status factor_impl(const rss_tree* tree, const rss_params* prm, cudaStream_t
         RSS_LAUNCHED();
         f->launches += 1;
       }
-      if constexpr (sizeof(T) == sizeof(double)) {
-        if (ozp_np > 0) {
-          k_w_split<<<dim3(nrec, 2 * ((max_r + 31) / 32)), NT, 0, st>>>(ea);
-          RSS_LAUNCHED();
-          const int smem = (64 + OZ_NCH) * (OZ_S * ozp_np + 8) * (int)sizeof(uint16_t);
-          RSS_CUDA(cudaFuncSetAttribute(k_elim_oz, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
-          k_elim_oz<<<dim3((max_c + 63) / 64, nrec), NT, smem, st>>>(ea);
-          RSS_LAUNCHED();
-          f->launches += 2;
-        }
-      } else {
-        if (ozp_np > 0) {
-          const int smem = (ZCM + ZCN) * ZSA * (int)sizeof(uint16_t);
-          RSS_CUDA(cudaFuncSetAttribute(k_elim_ozc, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
-          k_elim_ozc<<<dim3((max_c + ZCM - 1) / ZCM, nrec), NT, smem, st>>>(ea);
+      if (ep_n > 0) {
+        ep.L = cur.d;
+        ep.recs = d_recs;
+        ep.cls_idx = d_clsidx;
+        ep.perm_in = d_perm;
+        ep.err = d_err;
+        // the passes of a tile over as many CTAs as the tiles leave SMs
+        const int tiles = cdiv(max_c, ep.rows);
+        ep.psplit = std::max(1, std::min<int>(ep.ng, 152 / std::max<long long>(1, (long long)tiles * ep.sets * nrec)));
+        const int smem = ep.ad * ep.rows * OZ_S * TW_K * 2 + ep.wd * ep_parts<T>() * EP_GB + (ep.spn + ep.nstr * TW_M) * (int)sizeof(int);
+        RSS_CUDA(cudaFuncSetAttribute(k_ep<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+        k_ep_cut_w<T><<<dim3(ep.ng, ep.sets, nrec), EP_WT, 0, st>>>(ep);
+        RSS_LAUNCHED();
+        k_ep<T><<<dim3(tiles, ep.sets * ep.psplit, nrec), EP_NT, smem, st>>>(ep);
+        RSS_LAUNCHED();
+        f->launches += 2;
+        if (ep.psplit > 1 && oz) {
+          k_ep_slices<T><<<dim3(cdiv(max_c, TW_M), 2, nrec), 512, 0, st>>>(d_recs);
           RSS_LAUNCHED();
           f->launches += 1;
         }

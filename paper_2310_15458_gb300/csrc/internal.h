@@ -57,14 +57,7 @@ template <typename T> struct BoxRec {
   // (L^{-1} P)^T]; the solve applies W_F^T and W_E to the points of B
   T* We;
   T* Wf;
-  // factor-time only, tensor-core panel path (ozp = 1) of real factors:
-  // the columns of W_E then W_F (2 rp columns, rp = r rounded up to 32, the
-  // padding columns zero), each cut into OZ_S bf16 digit slices of np = n
-  // rounded up to 16 entries: column j at Wsl + j * OZ_S * np, slice p at
-  // + p * np; Wexp[j] its power-of-two scale
-  uint16_t* Wsl;
-  int* Wexp;
-  int ozp;
+  int ozp;      // 1: E and F^T are formed on the tensor cores
 };
 
 
