@@ -37,6 +37,7 @@ template <typename T> struct EpArgs {
   int rows, ad, wd;    // rows of a tile; stages of A and of W in shared memory
   int psplit;          // CTAs that share the passes of a tile
   int spn;             // entries of the pivot order kept in shared memory
+  int staged;          // complex: the slices in the layout of k_schur_z
   int* err;
 };
 template <typename T> __host__ __device__ constexpr int ep_ks() { return sizeof(T) == sizeof(double) ? TW_K : TW_K / 2; }
@@ -113,10 +114,13 @@ template <typename T> __global__ void __launch_bounds__(EP_WT) k_ep_cut_w(EpArgs
 }
 
 // Digit slices of rows i0 .. of E (or F^T) for the Schur update: row i at
-// sl + i * S * kp, slice p at + p * kp (complex: 8 real slices, then 8 imaginary).  Four
-// threads per row; scr: 512 keys, reb: 128 ints of shared memory.  512 threads.
+// sl + i * S * kp, slice p at + p * kp (complex: 8 real slices, then 8 imaginary).  staged
+// (complex): in the layout of k_schur_z, slice p of stage s at (s * 8 + p) * c8 * 64
+// (c8: c rounded up to 8), rows as in a stage; of F^T two such forms, for real and for
+// imaginary parts.  Four threads per row; scr: 512 keys, reb: 128 ints of shared memory.
+// 512 threads.
 template <typename T>
-__device__ void ep_slices(const BoxRec<T>& R, int which, int i0, int rows, unsigned long long* scr, int* reb) {
+__device__ void ep_slices(const BoxRec<T>& R, int which, int i0, int rows, int staged, unsigned long long* scr, int* reb) {
   constexpr bool cplx = sizeof(T) != sizeof(double);
   const int c = R.c, r = R.r, kp = R.kp;
   const T* src = (which ? R.Ft : R.E) + i0;
@@ -140,6 +144,29 @@ __device__ void ep_slices(const BoxRec<T>& R, int which, int i0, int rows, unsig
   __syncthreads();
   if (!on) return;
   const int eb = reb[i];
+  if constexpr (cplx) {
+    if (staged) {
+      const size_t c8 = (size_t)((c + 7) & ~7) * 64, form = (size_t)((r + 15) / 16) * OZ_S * c8;
+      unsigned char* b = reinterpret_cast<unsigned char*>(which ? R.Fsl : R.Esl);
+      for (int q = part; q < (r + 15) / 16 * 2; q += 4) {   // stage q / 2, entries 8 (q % 2) ..
+        T v[8];
+#pragma unroll
+        for (int e = 0; e < 8; ++e) v[e] = q * 8 + e < r ? src[i + (size_t)(q * 8 + e) * c] : zero<T>();
+        unsigned char* d = b + (size_t)(q / 2) * OZ_S * c8;
+        const int at0 = tw_at(i0 + i, q % 2), at1 = tw_at(i0 + i, 2 + q % 2);
+        long long X[8];
+#pragma unroll
+        for (int e = 0; e < 8; ++e) X[e] = oz_scaled_int(v[e].x, eb);
+        tw_put8(X, d + at0, c8, 0u);
+        if (which) tw_put8(X, d + form + at1, c8, 0u);
+#pragma unroll
+        for (int e = 0; e < 8; ++e) X[e] = oz_scaled_int(v[e].y, eb);
+        tw_put8(X, d + at1, c8, which ? 0x80008000u : 0u);
+        if (which) tw_put8(X, d + form + at0, c8, 0u);
+      }
+      return;
+    }
+  }
   unsigned char* d = reinterpret_cast<unsigned char*>(dst + (size_t)i * (cplx ? 2 : 1) * OZ_S * kp);
   for (int kg = part; kg < kp / 8; kg += 4) {
     T v[8];
@@ -162,13 +189,13 @@ __device__ void ep_slices(const BoxRec<T>& R, int which, int i0, int rows, unsig
 }
 
 // the slices alone, where the passes of a tile are shared by CTAs
-template <typename T> __global__ void __launch_bounds__(512) k_ep_slices(const BoxRec<T>* __restrict__ recs) {
+template <typename T> __global__ void __launch_bounds__(512) k_ep_slices(const BoxRec<T>* __restrict__ recs, int staged) {
   __shared__ unsigned long long scr[512];
   __shared__ int reb[TW_M];
   const BoxRec<T> R = recs[blockIdx.z];
   const int i0 = blockIdx.x * TW_M;
   if (!R.ozp || i0 >= R.c || R.Esl == nullptr) return;
-  ep_slices(R, blockIdx.y, i0, min(TW_M, R.c - i0), scr, reb);
+  ep_slices(R, blockIdx.y, i0, min(TW_M, R.c - i0), staged, scr, reb);
 }
 
 template <typename T> __global__ void __launch_bounds__(EP_NT, 1) k_ep(EpArgs<T> a) {
@@ -452,7 +479,7 @@ template <typename T> __global__ void __launch_bounds__(EP_NT, 1) k_ep(EpArgs<T>
   if (a.psplit == 1 && R.Esl != nullptr) {
     const int last = a.sets == 1 ? 1 : set;
     for (int w = a.sets == 1 ? 0 : set; w <= last; ++w) {
-      ep_slices(R, w, i0, rows, scr, reb);
+      ep_slices(R, w, i0, rows, a.staged, scr, reb);
       __syncthreads();
     }
   }
