@@ -86,7 +86,7 @@ typedef struct {
                                      (any rank) and
                                      E = A_CB W_E and
                                      F^T = A_BC^T W_F (real factors with n_B <= 128,
-                                     complex with any n_B); operands split into eight 7-bit
+                                     complex with n_B <= 3840); operands split into eight 7-bit
                                      slices with row and column scales, exact integer
                                      products, FP64 recombination (accuracy of an FP64
                                      product); the Schur update runs on tcgen05

@@ -1438,15 +1438,16 @@ constexpr int SR_M = 64, SR_N = 32;              // CTA tile
 constexpr int SR_BUF = (SR_M + SR_N) * SRSA;     // one stage of slices (uint16)
 constexpr int SR_FLUSH = 12;                     // chunks between int64 gathers (12 x 32 = 384)
 
-__global__ void __launch_bounds__(NT, 2) k_schur_oz(LevelDev<double> L, const BoxRec<double>* recs) {
+__global__ void __launch_bounds__(NT, 2) k_schur_oz(LevelDev<double> L, const BoxRec<double>* recs, int sym) {
   extern __shared__ __align__(16) unsigned char smraw[];
   const BoxRec<double> R = recs[blockIdx.y];
   const int c = R.c, kp = R.kp, ntr = (c + SR_M - 1) / SR_M, ntc = (c + SR_N - 1) / SR_N;
   if ((int)blockIdx.x >= ntr * ntc) return;
   const int i0 = (blockIdx.x % ntr) * SR_M, j0 = (blockIdx.x / ntr) * SR_N;
+  if (sym && j0 + SR_N <= i0) return;   // symmetric A: entries j >= i, stored to both triangles
   const int SA = SRSA;
   uint16_t* stage = reinterpret_cast<uint16_t*>(smraw);   // two stages: A rows then B rows
-  __shared__ long long rowb[SR_M], colb[SR_N];
+  __shared__ long long rowb[SR_M], colb[SR_N], coli[SR_M], rowj[SR_N];
   __shared__ int rexp[SR_M], cexp[SR_N];
   const int nmax = L.nmax, g = L.g;
   const long long nn = (long long)nmax * nmax;
@@ -1457,6 +1458,7 @@ __global__ void __launch_bounds__(NT, 2) k_schur_oz(LevelDev<double> L, const Bo
       const int cm = R.cmap[i], s = cm >> 16, pos = cm & 0xffff;
       const int u = nbr_box(R.box, g, s % 3 - 1, s / 3 - 1);
       rowb[tid] = (long long)u * 25 * nn + pos - (long long)((s / 3) * 5 + s % 3) * nn;
+      coli[tid] = (long long)((s / 3) * 5 + s % 3 + 12) * nn + (long long)pos * nmax;
       rexp[tid] = R.Eexp[i];
     }
   } else if (tid < SR_M + SR_N) {
@@ -1464,6 +1466,7 @@ __global__ void __launch_bounds__(NT, 2) k_schur_oz(LevelDev<double> L, const Bo
     if (j < c) {
       const int cm = R.cmap[j], s = cm >> 16, pos = cm & 0xffff;
       colb[tid - SR_M] = (long long)((s / 3) * 5 + s % 3 + 12) * nn + (long long)pos * nmax;
+      rowj[tid - SR_M] = (long long)nbr_box(R.box, g, s % 3 - 1, s / 3 - 1) * 25 * nn + pos - (long long)((s / 3) * 5 + s % 3) * nn;
       cexp[tid - SR_M] = R.Fexp[j];
     }
   }
@@ -1560,9 +1563,10 @@ __global__ void __launch_bounds__(NT, 2) k_schur_oz(LevelDev<double> L, const Bo
     for (int e = 0; e < 4; ++e) {
       const int row = m0 + gq + (e >= 2 ? 8 : 0);
       const int col = n0 + ni * 8 + 2 * t4 + (e & 1);
-      if (i0 + row < c && j0 + col < c) {
-        const double v = oz_ldexp_int(W[ni][e], rexp[row] + cexp[col] - 53);
-        L.blk[rowb[row] + colb[col]] = Cs[row + col * SR_M] - v;
+      if (i0 + row < c && j0 + col < c && (!sym || j0 + col >= i0 + row)) {
+        const double v = Cs[row + col * SR_M] - oz_ldexp_int(W[ni][e], rexp[row] + cexp[col] - 53);
+        L.blk[rowb[row] + colb[col]] = v;
+        if (sym && j0 + col > i0 + row) L.blk[rowj[col] + coli[row]] = v;
       }
     }
 }
@@ -1593,16 +1597,17 @@ constexpr long long ST_POLLS = 1LL << 22;
 constexpr long long ST_DRAIN_POLLS = 1LL << 26;
 
 __global__ void __launch_bounds__(ST_NT, 2) k_schur_tc(LevelDev<double> L, const BoxRec<double>* recs, int* err,
-                                                        long long polls) {
+                                                        long long polls, int sym) {
   extern __shared__ __align__(1024) unsigned char smraw[];
   __shared__ __align__(8) uint64_t mbar;
   __shared__ uint32_t s_tmem;
-  __shared__ long long colb[ST_N];
+  __shared__ long long colb[ST_N], rowj[ST_N];
   __shared__ int cexp[ST_N];
   const BoxRec<double> R = recs[blockIdx.y];
   const int c = R.c, kp = R.kp, ntr = (c + ST_M - 1) / ST_M, ntc = (c + ST_N - 1) / ST_N;
   if ((int)blockIdx.x >= ntr * ntc) return;
   const int i0 = (blockIdx.x % ntr) * ST_M, j0 = (blockIdx.x / ntr) * ST_N;
+  if (sym && j0 + ST_N <= i0) return;   // (its entries come from the tile across the diagonal)
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int quarter = warp & 3, half = warp >> 2;   // TMEM lanes 32 quarter .., columns 16 half ..
   unsigned char* As = smraw;
@@ -1610,21 +1615,23 @@ __global__ void __launch_bounds__(ST_NT, 2) k_schur_tc(LevelDev<double> L, const
   const int nmax = L.nmax, g = L.g;
   const long long nn = (long long)nmax * nmax;
   const int i = i0 + 32 * quarter + lane;   // this thread's row of the tile (TMEM lane)
-  long long rowb = 0;
+  long long rowb = 0, coli = 0;
   int rexp = 0;
   if (i < c) {
     const int cm = R.cmap[i], s = cm >> 16, pos = cm & 0xffff;
     const int u = nbr_box(R.box, g, s % 3 - 1, s / 3 - 1);
     rowb = (long long)u * 25 * nn + pos - (long long)((s / 3) * 5 + s % 3) * nn;
+    coli = (long long)((s / 3) * 5 + s % 3 + 12) * nn + (long long)pos * nmax;
     rexp = R.Eexp[i];
   }
   if (tid < ST_N) {
     const int j = j0 + tid;
-    colb[tid] = 0;
+    colb[tid] = rowj[tid] = 0;
     cexp[tid] = 0;
     if (j < c) {
       const int cm = R.cmap[j], s = cm >> 16, pos = cm & 0xffff;
       colb[tid] = (long long)((s / 3) * 5 + s % 3 + 12) * nn + (long long)pos * nmax;
+      rowj[tid] = (long long)nbr_box(R.box, g, s % 3 - 1, s / 3 - 1) * 25 * nn + pos - (long long)((s / 3) * 5 + s % 3) * nn;
       cexp[tid] = R.Fexp[j];
     }
   }
@@ -1698,7 +1705,11 @@ __global__ void __launch_bounds__(ST_NT, 2) k_schur_tc(LevelDev<double> L, const
       for (int jj = 0; jj < 8; ++jj) {
         const long long w = oz_join([&](int u) { return __uint_as_float(gr[u][jj]); });
         const int j = CH * half + c0 + jj;
-        if (i < c && j0 + j < c) L.blk[rowb + colb[j]] = cv[c0 + jj] - oz_ldexp_int(w, rexp + cexp[j] - 53);
+        if (i < c && j0 + j < c && (!sym || j0 + j >= i)) {
+          const double x = cv[c0 + jj] - oz_ldexp_int(w, rexp + cexp[j] - 53);
+          L.blk[rowb + colb[j]] = x;
+          if (sym && j0 + j > i) L.blk[rowj[j] + coli] = x;
+        }
       }
     }
   } else {
@@ -1723,21 +1734,28 @@ __global__ void __launch_bounds__(ST_NT, 2) k_schur_tc(LevelDev<double> L, const
 // bits.  A barrier wait that runs out sets RSS_ETIMEOUT; the CTA then drains
 // the products it issued (up to two tiles, the long limit), frees its tensor
 // memory and returns.
+// Symmetric A (sym; E F = X_CR X_RR^{-1} X_RC is symmetric to rounding): only the entries
+// j >= i are formed, and stored to A_CC(j, i) too, four entries of a row of the mirror
+// block side by side.  Half the products and FP64 arithmetic: Schur phase at Laplace
+// 1024^2 34 -> 28 ms, 448^2 (leaf 49) 58.8 -> 56.0 ms a factorization.
 constexpr int SRW_KP = 64;                  // largest kp of the row-block form
 constexpr uint32_t SRW_TMEM_COLS = 2 * ST_TMEM_COLS;
 constexpr int SRW_NT = 512;   // four warps per 32 TMEM lanes, 8 columns of a tile per thread
+constexpr int SRW_XB = 32 * 5 * 8;   // bytes of a warp's transposition
 
 __global__ void __launch_bounds__(SRW_NT, 1) k_schur_tc_rows(LevelDev<double> L, const BoxRec<double>* recs, int* err,
-                                                             long long polls) {
+                                                             long long polls, int sym) {
   extern __shared__ __align__(1024) unsigned char smraw[];
   __shared__ __align__(8) uint64_t mbar[2];
   __shared__ uint32_t s_tmem;
-  __shared__ long long colb[3][ST_N];   // column data of tile t in buffer t % 3
+  __shared__ long long colb[3][ST_N], rowj[3][ST_N];   // column data of tile t in buffer t % 3
+  __shared__ long long coli[ST_M];      // the rows' places as columns
   __shared__ int cexp[3][ST_N];
   const BoxRec<double> R = recs[blockIdx.y];
-  const int c = R.c, kp = R.kp, ntr = (c + ST_M - 1) / ST_M, ntc = (c + ST_N - 1) / ST_N;
+  const int c = R.c, kp = R.kp, ntr = (c + ST_M - 1) / ST_M;
   if ((int)blockIdx.x >= ntr) return;
   const int i0 = blockIdx.x * ST_M;
+  const int tb = sym ? i0 / ST_N : 0, ntc = (c + ST_N - 1) / ST_N - tb;   // first tile, tiles
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int quarter = warp & 3, half = warp >> 2;   // TMEM lanes 32 quarter .., columns CH half ..
   const int nch = (kp + ST_KC - 1) / ST_KC;   // 1 or 2
@@ -1746,17 +1764,19 @@ __global__ void __launch_bounds__(SRW_NT, 1) k_schur_tc_rows(LevelDev<double> L,
   const int nmax = L.nmax, g = L.g;
   const long long nn = (long long)nmax * nmax;
   const int i = i0 + 32 * quarter + lane;
+  double* xb = reinterpret_cast<double*>(smraw + nch * (ST_A + 2 * ST_B)) + warp * (SRW_XB / 8);   // 32 x 5 of the warp
   long long rowb = 0;
   int rexp = 0;
   if (i < c) {
     const int cm = R.cmap[i], s = cm >> 16, pos = cm & 0xffff;
     const int u = nbr_box(R.box, g, s % 3 - 1, s / 3 - 1);
     rowb = (long long)u * 25 * nn + pos - (long long)((s / 3) * 5 + s % 3) * nn;
+    if (half == 0) coli[32 * quarter + lane] = (long long)((s / 3) * 5 + s % 3 + 12) * nn + (long long)pos * nmax;
     rexp = R.Eexp[i];
   }
   // stage the B slices of tile t into buffer t & 1 and its column data into buffer t % 3
   auto stage_b = [&](int t) {
-    const int j0 = t * ST_N;
+    const int j0 = (tb + t) * ST_N;
     unsigned char* Bb = Bs + (t & 1) * nch * ST_B;
     for (int ci = 0; ci < nch; ++ci) {
       const int kc = ci * ST_KC, kl = min(ST_KC, kp - kc), ng = kl / 8, lg = ng == 4 ? 2 : 1;
@@ -1771,14 +1791,16 @@ __global__ void __launch_bounds__(SRW_NT, 1) k_schur_tc_rows(LevelDev<double> L,
     }
     if (tid < ST_N) {
       const int j = j0 + tid;
-      long long cb = 0;
+      long long cb = 0, rj = 0;
       int ce = 0;
       if (j < c) {
         const int cm = R.cmap[j], s = cm >> 16, pos = cm & 0xffff;
         cb = (long long)((s / 3) * 5 + s % 3 + 12) * nn + (long long)pos * nmax;
+        rj = (long long)nbr_box(R.box, g, s % 3 - 1, s / 3 - 1) * 25 * nn + pos - (long long)((s / 3) * 5 + s % 3) * nn;
         ce = R.Fexp[j];
       }
       colb[t % 3][tid] = cb;
+      rowj[t % 3][tid] = rj;
       cexp[t % 3][tid] = ce;
     }
   };
@@ -1805,6 +1827,8 @@ __global__ void __launch_bounds__(SRW_NT, 1) k_schur_tc_rows(LevelDev<double> L,
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = s_tmem;
+  const int uwarp = __shfl_sync(0xffffffffu, warp, 0);   // (uniform)
+  const uint32_t lead = uwarp == 0 ? elect_one() : 0u;   // issues the products, always the same lane
   constexpr int CH = ST_N / (SRW_NT / 128);
   double cv[CH], cvn[CH];
 #pragma unroll
@@ -1819,26 +1843,24 @@ __global__ void __launch_bounds__(SRW_NT, 1) k_schur_tc_rows(LevelDev<double> L,
     // from tile 1 on, the barrier at the end of the previous step stands here:
     // the B slices of tile t staged, tensor memory half t & 1 drained (tile t - 2)
     if (t < ntc) {
-      if (tid == 0) {
+      if (uwarp == 0) {
         tc_fence_after();
-        const unsigned char* Bb = Bs + (t & 1) * nch * ST_B;
+        const uint32_t bl = umma_lo(smem_u32(Bs + (t & 1) * nch * ST_B)), al = umma_lo(smem_u32(As));
         const uint32_t dcol = tmem + (uint32_t)(t & 1) * ST_TMEM_COLS;
         for (int ci = 0; ci < nch; ++ci) {
           const int kl = min(ST_KC, kp - ci * ST_KC);
-          for (int s = 0; s < kl / 16; ++s) {
-            const uint64_t bd = umma_desc(smem_u32(Bb + ci * ST_B + s * 256), 128, 512);
+          for (int s = 0; s < kl / 16; ++s)
 #pragma unroll
-            for (int p = 0; p < OZ_S; ++p) {
-              const uint64_t ad = umma_desc(smem_u32(As + ci * ST_A + p * (ST_M * ST_KC * 2) + s * 256), 128, 512);
-              umma_bf16(dcol + ST_N * p, ad, bd, umma_idesc_bf16(ST_M, ST_N * (OZ_S - p)),
-                        (ci > 0 || s > 0 || p > 0) ? 1u : 0u);
-            }
-          }
+            for (int p = 0; p < OZ_S; ++p)
+              umma_bf16_w(dcol + ST_N * p, al + (uint32_t)(ci * (ST_A / 16) + p * (ST_M * ST_KC / 8) + s * 16),
+                          bl + (uint32_t)(ci * (ST_B / 16) + s * 16), umma_idesc_bf16(ST_M, ST_N * (OZ_S - p)),
+                          (ci > 0 || s > 0 || p > 0) ? 1u : 0u, lead);
         }
-        umma_commit(&mbar[t & 1]);
+        umma_commit_w(&mbar[t & 1], lead);
+        __syncwarp();
       }
       // the entries of A_CC of tile t, read while its products run
-      const int j0 = t * ST_N;
+      const int j0 = (tb + t) * ST_N;
       if (i < c) {
 #pragma unroll
         for (int j = 0; j < CH; ++j)
@@ -1855,7 +1877,7 @@ __global__ void __launch_bounds__(SRW_NT, 1) k_schur_tc_rows(LevelDev<double> L,
         // while this tile is gathered
         if (t + 1 < ntc) stage_b(t + 1);
         tc_fence_after();
-        const int j0 = tp * ST_N, cb3 = tp % 3;
+        const int j0 = (tb + tp) * ST_N, cb3 = tp % 3;
         const uint32_t lane_base = tmem + (uint32_t)b * ST_TMEM_COLS + ((uint32_t)(32 * quarter) << 16) + CH * half;
 #pragma unroll
         for (int c0 = 0; c0 < CH; c0 += 8) {
@@ -1867,7 +1889,23 @@ __global__ void __launch_bounds__(SRW_NT, 1) k_schur_tc_rows(LevelDev<double> L,
           for (int jj = 0; jj < 8; ++jj) {
             const long long w = oz_join([&](int u) { return __uint_as_float(gr[u][jj]); });
             const int j = CH * half + c0 + jj;
-            if (i < c && j0 + j < c) L.blk[rowb + colb[cb3][j]] = cv[c0 + jj] - oz_ldexp_int(w, rexp + cexp[cb3][j] - 53);
+            const double x = cv[c0 + jj] - oz_ldexp_int(w, rexp + cexp[cb3][j] - 53);
+            if (i < c && j0 + j < c && (!sym || j0 + j >= i)) L.blk[rowb + colb[cb3][j]] = x;
+            // across the diagonal: four columns at a time through shared memory, so that
+            // a warp stores the four entries of a row of the mirror block side by side
+            if (sym) {
+              if (jj % 4 == 0) __syncwarp();
+              xb[lane * 5 + jj % 4] = x;
+              if (jj % 4 == 3) {
+                __syncwarp();
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                  const int ii = 8 * q + (lane >> 2), jm = j - 3 + (lane & 3), im = i0 + 32 * quarter + ii;
+                  if (im < c && j0 + jm < c && j0 + jm > im)
+                    L.blk[rowj[cb3][jm] + coli[32 * quarter + ii]] = xb[ii * 5 + (lane & 3)];
+                }
+              }
+            }
           }
         }
       }
@@ -2912,19 +2950,19 @@ rss_status factor_impl(const rss_tree* tree, const rss_params* prm, cudaStream_t
           if (prm->schur_path == 0 && kp_max <= SRW_KP && (long long)nrec * ntr_rows >= 2 * 152) {
             // tcgen05, one CTA per 128-row block walking its column tiles (one CTA per SM)
             const int nchm = (kp_max + ST_KC - 1) / ST_KC;
-            const int smem = std::max(nchm * ST_A + 2 * nchm * ST_B, 120 * 1024);
+            const int smem = std::max(nchm * (ST_A + 2 * ST_B) + SRW_NT / 32 * SRW_XB, 120 * 1024);
             RSS_CUDA(cudaFuncSetAttribute(k_schur_tc_rows, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
-            k_schur_tc_rows<<<dim3(ntr_rows, nrec), SRW_NT, smem, st>>>(cur.d, d_recs, d_err, polls);
+            k_schur_tc_rows<<<dim3(ntr_rows, nrec), SRW_NT, smem, st>>>(cur.d, d_recs, d_err, polls, sym);
           } else if (prm->schur_path == 0 && kp_max <= 384) {   // tcgen05: FP32 group sums over the whole K
             const int smem = ST_A + ST_B;
             RSS_CUDA(cudaFuncSetAttribute(k_schur_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
             const int ntr = (max_c + ST_M - 1) / ST_M, ntc = (max_c + ST_N - 1) / ST_N;
-            k_schur_tc<<<dim3(ntr * ntc, nrec), ST_NT, smem, st>>>(cur.d, d_recs, d_err, polls);
+            k_schur_tc<<<dim3(ntr * ntc, nrec), ST_NT, smem, st>>>(cur.d, d_recs, d_err, polls, sym);
           } else {
             const size_t smem = 2 * (size_t)SR_BUF * sizeof(uint16_t);
             RSS_CUDA(cudaFuncSetAttribute(k_schur_oz, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
             const int ntr = (max_c + SR_M - 1) / SR_M, ntc = (max_c + SR_N - 1) / SR_N;
-            k_schur_oz<<<dim3(ntr * ntc, nrec), NT, smem, st>>>(cur.d, d_recs);
+            k_schur_oz<<<dim3(ntr * ntc, nrec), NT, smem, st>>>(cur.d, d_recs, sym);
           }
         } else {
           if (staged) {

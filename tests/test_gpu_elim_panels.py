@@ -6,8 +6,9 @@ stretches of K), r with a last group of at most and of more than 16 columns, one
 per colour class (passes shared by CTAs) and many.  Where the pivots agree, E and F
 agree to the tolerance of a record, t = (1 + depth) max(1e-10, 1e-14 / eps) (depth:
 levels eliminated before).  The blocks of later classes and levels hold the Schur
-updates of earlier ones, so the complex update (r up to 32, 48, 192 and above; boxes of
-one class with more and fewer stages) is compared with the FP64 one as well.
+updates of earlier ones, so those (complex: r up to 32, 48, 192 and above; real: tiles and
+row blocks, one triangle formed and mirrored; boxes of
+one class with more and fewer stages) are compared with the FP64 ones as well.
 """
 import numpy as np
 import pytest
@@ -23,7 +24,7 @@ pytestmark = pytest.mark.gpu
     ("laplace", 32, 16, 1e-6), ("laplace", 64, 4, 1e-8), ("laplace", 72, 81, 1e-6), ("laplace", 88, 121, 1e-6),
     ("laplace", 128, 64, 1e-4), ("laplace", 160, 100, 1e-6), ("helmholtz", 32, 16, 1e-6), ("helmholtz", 32, 4, 1e-8),
     ("helmholtz", 96, 144, 1e-6), ("helmholtz", 80, 100, 1e-4), ("helmholtz", 128, 64, 1e-6),
-    ("helmholtz", 64, 256, 1e-4)])
+    ("helmholtz", 64, 256, 1e-4), ("laplace", 256, 64, 1e-6), ("laplace", 256, 16, 1e-4)])
 def test_panels_on_tensor_cores_match_fp64(kind, side, leaf, eps):
     if not torch.cuda.is_available():
         pytest.skip("no CUDA device")
