@@ -2971,7 +2971,7 @@ rss_status factor_impl(const rss_tree* tree, const rss_params* prm, cudaStream_t
             const int smem = ad * trows * SZ_AST + nb * SZ_BP;
             const int csplit = std::max(1, std::min<int>(cdiv(max_c, 32), 152 / std::max(1, ntr * nrec)));
             RSS_CUDA(cudaFuncSetAttribute(k_schur_z, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
-            k_schur_z<<<dim3(ntr, csplit, nrec), EP_NT, smem, st>>>(cur.d, d_recs, trows, ad, nb, csplit, split ? 1 : 0, d_err, polls);
+            k_schur_z<<<dim3(nrec, csplit, ntr), EP_NT, smem, st>>>(cur.d, d_recs, trows, ad, nb, csplit, split ? 1 : 0, d_err, polls);
           } else {
             const size_t smem = (64 + 32) * (size_t)SCSA * sizeof(uint16_t);
             RSS_CUDA(cudaFuncSetAttribute(k_schur_oz_c, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));

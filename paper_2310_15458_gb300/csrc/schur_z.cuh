@@ -8,7 +8,8 @@
 // by bulk copies; those of the block's rows stay in shared memory where they fit (r <= 48).
 //
 // Symmetric A with a real T (X_RC = X_CR^T, so E F is symmetric to rounding): only the
-// entries j >= i are formed, and stored to A_CC(j, i) as well.
+// entries j >= i are formed, and stored to A_CC(j, i) as well; the row blocks with the
+// most tiles of every box start first (60.2 -> 59.5 ms at Helmholtz 256^2).
 //
 // Bound by the products (96 per tile at r = 48, 80 clocks each) and the join of the sums,
 // which cannot overlap (a tile's sums fill tensor memory); the FP64 arithmetic (a
@@ -26,8 +27,8 @@ __global__ void __launch_bounds__(EP_NT, 1) k_schur_z(LevelDev<zd> L, const BoxR
   __shared__ __align__(8) uint64_t afull[4], afree[4], bfull[8], bfree[8], tdone, tfree, drained;
   __shared__ uint32_t s_tmem;
   __shared__ volatile int s_ok;
-  const BoxRec<zd> R = recs[blockIdx.z];
-  const int c = R.c, r = R.r, i0 = blockIdx.x * trows, rows = min(trows, c - i0), c8 = (c + 7) & ~7;
+  const BoxRec<zd> R = recs[blockIdx.x];
+  const int c = R.c, r = R.r, i0 = blockIdx.z * trows, rows = min(trows, c - i0), c8 = (c + 7) & ~7;
   const int ns = (r + 15) / 16;
   // tiles of this CTA: t0, t0 + csplit, ..
   const int tend = (c + 31) / 32, t0 = (sym ? i0 / 32 : 0) + blockIdx.y;
