@@ -297,6 +297,14 @@ template <bool WIDE = false, int X = 0, class G> __device__ __forceinline__ long
   asm("mad.wide.s32 %0, %1, %2, %0;\n" : "+l"(w) : "r"(v[2]), "n"(1 << (4 + X)));
   return w;
 }
+// |G_u| <= 10 2^12 K over K entries of the inner dimension (digits of at most 64, the
+// first of at most 128): below 2^22 for K <= OZ_KN, below 2^24 for K <= OZ_KX.
+constexpr int OZ_KN = 96, OZ_KX = 384;
+static_assert(10 * 4096 * OZ_KN < (1 << 22) && 10 * 4096 * OZ_KX < (1 << 24), "");
+// the join for sums over K <= OZ_KX entries (K the same in every thread)
+template <class G> __device__ __forceinline__ long long oz_join_k(int K, G g) {
+  return K <= OZ_KN ? oz_join(g) : oz_join<true>(g);
+}
 static_assert(OZ_S == 8 && OZ_BITS == 7, "");
 
 // W 2^s as a double, W an exact integer (|W| < 2^63): one conversion, the

@@ -1436,7 +1436,7 @@ template <typename T> __global__ void __launch_bounds__(NT) k_schur(LevelDev<T> 
 constexpr int SRK = 32, SRSA = OZ_S * SRK + 8;   // real Schur: K chunk and slice-row stride
 constexpr int SR_M = 64, SR_N = 32;              // CTA tile
 constexpr int SR_BUF = (SR_M + SR_N) * SRSA;     // one stage of slices (uint16)
-constexpr int SR_FLUSH = 12;                     // chunks between int64 gathers (12 x 32 = 384)
+constexpr int SR_FLUSH = OZ_KX / SRK;            // chunks between int64 gathers (12 x 32 = 384)
 
 __global__ void __launch_bounds__(NT, 2) k_schur_oz(LevelDev<double> L, const BoxRec<double>* recs, int sym) {
   extern __shared__ __align__(16) unsigned char smraw[];
@@ -1500,14 +1500,13 @@ __global__ void __launch_bounds__(NT, 2) k_schur_oz(LevelDev<double> L, const Bo
 #pragma unroll
       for (int u = 0; u < OZ_S; ++u) acc[u][ni][e] = 0.f;
     }
-  // W += sum_u G_u 2^(39-7u), groups u and u + 1 as (G_u 2^7 + G_{u+1}) 2^(32-7u)
-  // (exact in int32: |G| < 2^23); then the FP32 sums restart from zero
-  auto gather = [&]() {
+  // W += the sums of the `entries` of K since the last gather; they restart from zero
+  auto gather = [&](int entries) {
 #pragma unroll
     for (int ni = 0; ni < 2; ++ni)
 #pragma unroll
       for (int e = 0; e < 4; ++e) {
-        W[ni][e] += oz_join([&](int u) { return acc[u][ni][e]; });
+        W[ni][e] += oz_join_k(entries, [&](int u) { return acc[u][ni][e]; });
 #pragma unroll
         for (int u = 0; u < OZ_S; ++u) acc[u][ni][e] = 0.f;
       }
@@ -1551,10 +1550,10 @@ __global__ void __launch_bounds__(NT, 2) k_schur_oz(LevelDev<double> L, const Bo
         }
       }
     }
-    if ((ci + 1) % SR_FLUSH == 0 && ci + 1 < nch) gather();
+    if ((ci + 1) % SR_FLUSH == 0 && ci + 1 < nch) gather(SR_FLUSH * SRK);
     __syncthreads();   // the stage read here is refilled by the next iteration's load
   }
-  gather();
+  gather(kp - (nch - 1) / SR_FLUSH * (SR_FLUSH * SRK));
   cp_async_wait_group<0>();
   __syncthreads();
 #pragma unroll
@@ -1575,7 +1574,7 @@ __global__ void __launch_bounds__(NT, 2) k_schur_oz(LevelDev<double> L, const Bo
 // issues the slice products into tensor memory.  A CTA of 256 threads owns 128
 // rows (of E) x 32 columns (rows of F^T) of A_CC; group sum G_u (u = p + q)
 // accumulates in TMEM columns 32u .. 32u + 31 (256 columns, two CTAs per SM) in
-// FP32 over the whole K (exact for kp <= 384, checked by the host); per K step
+// FP32 over the whole K (exact for kp <= OZ_KX, checked by the host); per K step
 // of 16 it takes eight products, A slice p against the stacked B slices
 // 0 .. 7 - p (N = 32 (8 - p)).  K is staged
 // in chunks of 32 in the no-swizzle K-major layout of 8-row x 16-byte core
@@ -1703,7 +1702,7 @@ __global__ void __launch_bounds__(ST_NT, 2) k_schur_tc(LevelDev<double> L, const
       tmem_ld_wait();
 #pragma unroll
       for (int jj = 0; jj < 8; ++jj) {
-        const long long w = oz_join([&](int u) { return __uint_as_float(gr[u][jj]); });
+        const long long w = oz_join_k(kp, [&](int u) { return __uint_as_float(gr[u][jj]); });
         const int j = CH * half + c0 + jj;
         if (i < c && j0 + j < c && (!sym || j0 + j >= i)) {
           const double x = cv[c0 + jj] - oz_ldexp_int(w, rexp + cexp[j] - 53);
@@ -2953,7 +2952,7 @@ rss_status factor_impl(const rss_tree* tree, const rss_params* prm, cudaStream_t
             const int smem = std::max(nchm * (ST_A + 2 * ST_B) + SRW_NT / 32 * SRW_XB, 120 * 1024);
             RSS_CUDA(cudaFuncSetAttribute(k_schur_tc_rows, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
             k_schur_tc_rows<<<dim3(ntr_rows, nrec), SRW_NT, smem, st>>>(cur.d, d_recs, d_err, polls, sym);
-          } else if (prm->schur_path == 0 && kp_max <= 384) {   // tcgen05: FP32 group sums over the whole K
+          } else if (prm->schur_path == 0 && kp_max <= OZ_KX) {   // tcgen05: FP32 group sums over the whole K
             const int smem = ST_A + ST_B;
             RSS_CUDA(cudaFuncSetAttribute(k_schur_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
             const int ntr = (max_c + ST_M - 1) / ST_M, ntc = (max_c + ST_N - 1) / ST_N;

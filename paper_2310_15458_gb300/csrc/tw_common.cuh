@@ -9,8 +9,8 @@
 namespace {
 
 constexpr int TW_M = 128, TW_NC = 64, TW_K = 32, TW_NT = 512;
-constexpr int TW_KX = 384;                               // 8 pairs of digits: 10 2^12 K < 2^24
-constexpr int TW_KN = 96;                                // ... < 2^22 (oz_fint)
+constexpr int TW_KX = OZ_KX;                             // sums exact in FP32
+constexpr int TW_KN = OZ_KN;                             // ... and below 2^22 (oz_fint)
 constexpr int TW_A = OZ_S * TW_M * TW_K * 2;             // bytes of a stage: 64 KB
 constexpr int TW_B = OZ_S * TW_NC * TW_K * 2;            // 32 KB
 constexpr long long TW_POLLS = 1LL << 22, TW_DRAIN = 1LL << 26;
