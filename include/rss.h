@@ -123,9 +123,11 @@ typedef struct {
                                      gives up, and rss_factor then returns RSS_ETIMEOUT (after
                                      the products already issued have finished, so nothing is
                                      left running); a CTA of the persistent solve sweeps polls a
-                                     grid barrier at most this many times, and a solve whose
-                                     barrier ran out writes NaN into every entry of its result.
-                                     0: the default limits (2^22 and 2^24 polls); n > 0: n polls;
+                                     grid barrier, and one of the tensor-core sweeps its
+                                     products' and copies' barriers, at most this many times, and
+                                     a solve with a wait that ran out writes NaN into every entry
+                                     of its result.  0: the default limits (2^24 polls of a grid
+                                     barrier, 2^22 of the others); n > 0: n polls;
                                      -1: give up without polling, which exercises the timeout
                                      paths on purpose (for tests) */
   const char* tune_table;         /* NULL, or the JSON object rss_tune_solve returned (read during

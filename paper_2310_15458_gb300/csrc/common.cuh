@@ -184,9 +184,9 @@ __device__ __forceinline__ void mbar_init(uint64_t* mbar, int count) {
   asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
 }
 // poll phase `parity` of the mbarrier at most `polls` times; false if it never completed
-__device__ __forceinline__ bool mbar_wait(uint64_t* mbar, uint32_t parity, long long polls) {
+template <typename I> __device__ __forceinline__ bool mbar_wait(uint64_t* mbar, uint32_t parity, I polls) {
   uint32_t done = 0;
-  for (long long it = 0; it < polls && !done; ++it)
+  for (I it = 0; it < polls && !done; ++it)
     asm volatile(
         "{\n.reg .pred p;\nmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\nselp.u32 %0, 1, 0, p;\n}\n"
         : "=r"(done)

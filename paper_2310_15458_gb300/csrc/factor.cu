@@ -2412,7 +2412,7 @@ rss_status factor_impl(const rss_tree* tree, const rss_params* prm, cudaStream_t
   // and the ID of [A_MB; K_PB] alone is the same ID.
   const int half = (prm->id_rows == 0 && prm->kind == RSS_LAPLACE && prm->diag_im == 0.0) ? 1 : 0;
   // poll limit of the first barrier wait of the tensor-core Schur updates
-  const long long polls = prm->wait_polls == 0 ? ST_POLLS : prm->wait_polls < 0 ? 0 : (long long)prm->wait_polls;
+  const long long polls = wait_limit(prm->wait_polls, ST_POLLS);
   // A complex symmetric kernel (Helmholtz): the ID of the real stack
   // [Re X; Im X], X = [A_MB; K_PB], which is the ID of the full stack (T real).
   const bool split = std::is_same<T, zd>::value && prm->id_rows == 0 &&

@@ -232,7 +232,7 @@ rss_status sweep_persistent_launch(const rss_factorization* f, T* x, int64_t ldx
   a.nrhs = nrhs;
   a.bar = bar;
   a.err = reinterpret_cast<int*>(bar + 2);
-  a.polls = f->params.wait_polls == 0 ? SWP_POLLS : f->params.wait_polls < 0 ? 0 : (long long)f->params.wait_polls;
+  a.polls = wait_limit(f->params.wait_polls, SWP_POLLS);
   a.sm_cap = (int)(smem / sizeof(T));
   void* args[] = {&a};
   const void* fn = up ? reinterpret_cast<const void*>(k_sweep<T, RC, true>)
@@ -427,7 +427,8 @@ rss_status ensure_slices(rss_factorization* f, cudaStream_t st) {
 }
 
 template <typename T, int OP, bool CACHE, int GW>
-cudaError_t launch_tw_gw(const Batch& b, const SliceRec* sl, T* x, int64_t ldx, int nrhs, int* err, cudaStream_t st) {
+cudaError_t launch_tw_gw(const Batch& b, const SliceRec* sl, T* x, int64_t ldx, int nrhs, int* err, int polls,
+                         cudaStream_t st) {
   constexpr bool real = sizeof(T) == sizeof(double);
   const int mr = OP == TW_UPE ? std::max(1, b.max_c) : OP == TW_DNW ? b.max_n : b.max_r;
   const int mk = OP == TW_UPW ? b.max_n : OP == TW_DNF ? b.max_c : b.max_r;
@@ -439,16 +440,18 @@ cudaError_t launch_tw_gw(const Batch& b, const SliceRec* sl, T* x, int64_t ldx, 
   if (OP == TW_DNF)
     while (spl < 8 && b.nrec * spl <= 76 && mk >= 16 * spl * (real ? TW_K : TW_K / 2)) spl *= 2;
   return launch_pdl(k_tw<T, OP, CACHE, GW>, dim3(spl * cdiv(mr, TW_M), cdiv(nrhs, real ? 2 * GW : GW), b.nrec), TW_NT,
-                    p.smem, st, spl, static_cast<const BoxRec<T>*>(b.d_recs), sl, x, ldx, nrhs, p.rows8, p.nst, p.nstr, err);
+                    p.smem, st, spl, static_cast<const BoxRec<T>*>(b.d_recs), sl, x, ldx, nrhs, p.rows8, p.nst, p.nstr, err,
+                    polls);
 }
 
 // 16 columns to a group where 32 would leave half of the SMs without a CTA
 template <typename T, int OP, bool CACHE>
-cudaError_t launch_tw(const Batch& b, const SliceRec* sl, T* x, int64_t ldx, int nrhs, int* err, cudaStream_t st) {
+cudaError_t launch_tw(const Batch& b, const SliceRec* sl, T* x, int64_t ldx, int nrhs, int* err, int polls,
+                      cudaStream_t st) {
   const long long tiles = OP == TW_UPE ? cdiv(std::max(1, b.max_c), TW_M) : 1;
   const bool few = tiles * b.nrec * cdiv(nrhs, sizeof(T) == sizeof(double) ? TW_NC : TW_NC / 2) <= 76;
-  return few || nrhs <= 16 ? launch_tw_gw<T, OP, CACHE, 16>(b, sl, x, ldx, nrhs, err, st)
-             : launch_tw_gw<T, OP, CACHE, 32>(b, sl, x, ldx, nrhs, err, st);
+  return few || nrhs <= 16 ? launch_tw_gw<T, OP, CACHE, 16>(b, sl, x, ldx, nrhs, err, polls, st)
+             : launch_tw_gw<T, OP, CACHE, 32>(b, sl, x, ldx, nrhs, err, polls, st);
 }
 
 // The tensor-core sweeps for the colour classes that take them, the FP64 sweeps for the
@@ -470,12 +473,13 @@ rss_status sweeps_tc(const rss_factorization* f, T* x, int64_t ldx, int nrhs, cu
   const SweepWs w = sweep_ws<T>(f, nrhs, RC);
   T* topz = reinterpret_cast<T*>(static_cast<char*>(ws) + w.topz_off);
   int* err = reinterpret_cast<int*>(static_cast<char*>(ws) + w.bar_off + 2 * sizeof(unsigned));
+  const int polls = (int)wait_limit(f->params.wait_polls, TW_POLLS);
   auto product = [&](size_t bi, auto op) -> cudaError_t {
     constexpr int OP = decltype(op)::value;
     const Batch& b = f->batches[bi];
     if constexpr (real)
-      if (sl) return launch_tw<T, OP, true>(b, f->d_slices[bi], x, ldx, nrhs, err, st);
-    return launch_tw<T, OP, false>(b, nullptr, x, ldx, nrhs, err, st);
+      if (sl) return launch_tw<T, OP, true>(b, f->d_slices[bi], x, ldx, nrhs, err, polls, st);
+    return launch_tw<T, OP, false>(b, nullptr, x, ldx, nrhs, err, polls, st);
   };
   for (size_t bi = 0; bi < f->batches.size(); ++bi) {
     if (!tw_takes(f->batches[bi], nrhs, real)) {

@@ -160,7 +160,8 @@ inline TwPlan tw_plan(int max_rows, int max_k, int gw, int ks, int sx) {
 // GW: columns of a group (32, or 16 for classes of few boxes: more and shorter CTAs)
 template <typename T, int OP, bool CACHE, int GW>
 __global__ void __launch_bounds__(TW_NT, 1) k_tw(const BoxRec<T>* __restrict__ recs, const SliceRec* __restrict__ sl,
-                                                 T* __restrict__ x, int64_t ldx, int nrhs, int srows, int nst, int nstr, int* err) {
+                                                 T* __restrict__ x, int64_t ldx, int nrhs, int srows, int nst, int nstr, int* err,
+                                                 int polls) {
   extern __shared__ __align__(1024) unsigned char sm[];
   constexpr bool cplx = sizeof(T) != sizeof(double);
   constexpr int KS = cplx ? TW_K / 2 : TW_K;       // entries of K per stage
@@ -170,8 +171,8 @@ __global__ void __launch_bounds__(TW_NT, 1) k_tw(const BoxRec<T>* __restrict__ r
   constexpr int LDO = NC + 1;
   __shared__ __align__(8) uint64_t mb_mma[4], mb_full[4];
   __shared__ uint32_t s_tmem;
+  __shared__ int s_bad[2];
   constexpr int SX = tw_stretch<T>();              // stages of a stretch of K
-  __shared__ int s_ok;
   const BoxRec<T> R = recs[blockIdx.z];
   const int M = tw_rows<OP>(R), Kall = tw_inner<OP>(R), k = R.k;
   // the down sweep's long inner dimension: a cluster of CTAs, each a range of stages
@@ -208,8 +209,8 @@ __global__ void __launch_bounds__(TW_NT, 1) k_tw(const BoxRec<T>* __restrict__ r
   if (tid < 4) {
     mbar_init(&mb_mma[tid], 1);
     mbar_init(&mb_full[tid], 1);
+    if (tid < 2) s_bad[tid] = 0;
   }
-  if (tid == 0) s_ok = 1;
   if (warp == 0) tmem_alloc(&s_tmem, 16 * GW);
   // where the entries of the right-hand side's K rows sit in x
   for (int l = K0 + tid; l < K; l += TW_NT)
@@ -284,24 +285,31 @@ __global__ void __launch_bounds__(TW_NT, 1) k_tw(const BoxRec<T>* __restrict__ r
     for (int e = 0; e < 8; ++e) bv[e] = (bq < nq && l0 + e < K) ? __ldcg(xc + (cplx ? 2 : 1) * (kx[l0 + e] * ldx)) : 0.0;
   };
   if (tb >= 0) load_b(0);
-  // the products of stage s are done (each thread polls; a wait that runs out ends the CTA's work)
-  auto wait_mma = [&](int s) {
-    if (!mbar_wait(&mb_mma[s % nst], (s / nst) & 1, TW_POLLS)) s_ok = 0;
+  // A wait that runs out ends the CTA's work at the next block barrier.  Barrier s reads
+  // flag s & 1, which is written before it and again only after barrier s + 1: every
+  // thread leaves it with the same verdict.
+  volatile int* bad = s_bad;
+  auto wait_mma = [&](int s, int at) {   // the products of stage s are done (each thread polls); verdict at barrier `at`
+    const bool done = mbar_wait(&mb_mma[s % nst], (s / nst) & 1, polls);
+    if (!done) bad[at & 1] = 1;
+    return done;
   };
-  int ok = 1;
+  int ok = 1, issued = 0;   // (issued: stages whose products were issued, known to warp 0)
   for (int s = 0; s < ns; ++s) {
     const int b = s % nst;
     unsigned char* As = sm + (size_t)b * ST;
     unsigned char* Bs = As + ABYTES;
     const bool fresh = s == 0 || (s0 + s) % SX == 0;   // the group sums start over
-    if (s >= nst) wait_mma(s - nst);              // the products that read this buffer
+    if (s >= nst) wait_mma(s - nst, s);           // the products that read this buffer
     if (CACHE && tid == 0 && fetched < ns && s + pd < ns) {
-      if (s + pd >= nst) wait_mma(s + pd - nst);
-      fetch_a(fetched);
-      ++fetched;
+      if (s + pd < nst || wait_mma(s + pd - nst, s)) {
+        fetch_a(fetched);
+        ++fetched;
+      }
     }
     if (fresh && s > 0) {   // the sums of the stretch of K before this stage
-      wait_mma(s - 1);
+      wait_mma(s - 1, s);
+      __syncwarp();
       tc_fence_after();
       gather(stretch(s - 1), std::false_type{});
       tc_fence_before();
@@ -327,15 +335,15 @@ __global__ void __launch_bounds__(TW_NT, 1) k_tw(const BoxRec<T>* __restrict__ r
     fence_async_smem();
     tc_fence_before();
     __syncthreads();
-    ok = s_ok;
+    ok = !bad[s & 1];
     if (!ok) break;
     if (uwarp == 0) {
       // (a copy that never lands leaves the stage without products)
-      const bool got = !CACHE || mbar_wait(&mb_full[b], (s / nst) & 1, TW_POLLS);
-      __syncwarp();
-      if (!got) s_ok = 0;
+      const bool got = __all_sync(0xffffffffu, !CACHE || mbar_wait(&mb_full[b], (s / nst) & 1, polls));
+      if (!got) bad[(s + 1) & 1] = 1;
+      issued += got;
       tc_fence_after();
-      const uint32_t lead = __all_sync(0xffffffffu, got) ? elect_one() : 0u;
+      const uint32_t lead = got ? elect_one() : 0u;
       const uint32_t al = umma_lo(smem_u32(As)), bl = umma_lo(smem_u32(Bs));
 #pragma unroll
       for (int h = 0; h < TW_K / 16; ++h)
@@ -352,11 +360,11 @@ __global__ void __launch_bounds__(TW_NT, 1) k_tw(const BoxRec<T>* __restrict__ r
       __syncwarp();
     }
   }
-  __syncthreads();   // (s_ok of the last stage)
-  ok = ok && s_ok;
-  if (ok && ns > 0) wait_mma(ns - 1);
   __syncthreads();
-  ok = ok && s_ok;
+  ok = ok && !bad[ns & 1];
+  if (ok && ns > 0) wait_mma(ns - 1, ns + 1);
+  __syncthreads();
+  ok = ok && !bad[(ns + 1) & 1];
   tc_fence_after();
   if (ok) {
     if (ns > 0) {
@@ -381,8 +389,7 @@ __global__ void __launch_bounds__(TW_NT, 1) k_tw(const BoxRec<T>* __restrict__ r
   } else if (tid == 0) {
     atomicExch(err, (int)RSS_ETIMEOUT);
     // what is in flight (products, copies) ends before the buffers and the tensor memory go
-    for (int b = 0; b < nst; ++b)
-      for (int ph = 0; ph < 2; ++ph) mbar_wait(&mb_mma[b], ph, TW_DRAIN / 64);
+    for (int q = max(0, issued - nst); q < issued; ++q) mbar_wait(&mb_mma[q % nst], (q / nst) & 1, TW_DRAIN);
     if (CACHE)
       for (int q = max(0, fetched - nst); q < fetched; ++q) mbar_wait(&mb_full[q % nst], (q / nst) & 1, TW_DRAIN);
   }
