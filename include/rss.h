@@ -118,7 +118,8 @@ typedef struct {
                                      other value: a permutation of each class drawn from this
                                      seed (same-colour boxes are independent, Algorithm 1 with
                                      nine colours, so the factorization must not change) */
-  int wait_polls;                 /* device waits are bounded: a CTA of the tensor-core Schur
+  int wait_polls;                 /* device waits are bounded: with schur_path 0 a CTA of the tensor-core
+                                     products of the ID, of the panels and of the Schur
                                      update polls its barrier at most this many times before it
                                      gives up, and rss_factor then returns RSS_ETIMEOUT (after
                                      the products already issued have finished, so nothing is

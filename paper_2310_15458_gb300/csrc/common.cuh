@@ -183,6 +183,8 @@ __device__ __forceinline__ void mbar_init(uint64_t* mbar, int count) {
   asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;\n" ::"r"(smem_u32(mbar)), "r"(count) : "memory");
   asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
 }
+// the first error of a call stands (what follows it may run on void numbers)
+__device__ __forceinline__ void set_error(int* err, int code) { atomicCAS(err, 0, code); }
 // poll phase `parity` of the mbarrier at most `polls` times; false if it never completed
 template <typename I> __device__ __forceinline__ bool mbar_wait(uint64_t* mbar, uint32_t parity, I polls) {
   uint32_t done = 0;

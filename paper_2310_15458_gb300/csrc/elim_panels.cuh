@@ -42,6 +42,7 @@ template <typename T> struct EpArgs {
   int spn;             // entries of the pivot order kept in shared memory
   int staged;          // complex: the slices in the layout of k_schur_z
   int* err;
+  int polls;           // of the waits that wait_polls governs
 };
 template <typename T> __host__ __device__ constexpr int ep_ks() { return sizeof(T) == sizeof(double) ? TW_K : TW_K / 2; }
 // stages of K that share scales and sums
@@ -320,7 +321,8 @@ template <typename T> __global__ void __launch_bounds__(EP_NT, 1) k_ep(EpArgs<T>
     };
     while (loaded < min(wd, nu)) load_w();
     int t = 0, seq = 0, u = 0;   // stages of A, joins, stages of W
-    bool ok = true;
+    // (a.polls governs the first wait; constants in the issuing loop, as in k_schur_z)
+    bool ok = __all_sync(0xffffffffu, mbar_wait(&wfull[0], 0, a.polls));
     for (int q = 0; q < np_mine && ok; ++q) {
       const int cw = ep_cols(nc, p0 + a.psplit * q);
       for (int s = 0; s < ns && ok; ++s, ++u) {
@@ -376,7 +378,7 @@ template <typename T> __global__ void __launch_bounds__(EP_NT, 1) k_ep(EpArgs<T>
     // sums of join `sq`: pass p, the stages sa .. sb of its K
     auto join = [&](int sq, int p, int sa, int sb) {
       const int h = sq % NBUF, cw = ep_cols(nc, p);
-      ok = ok && mbar_wait(&tdone[h], (sq / NBUF) & 1, TW_POLLS);
+      ok = ok && mbar_wait(&tdone[h], (sq / NBUF) & 1, a.polls);
       ok = __all_sync(0xffffffffu, ok) && s_ok;
       if (!ok) return;
       tc_fence_after();
@@ -440,7 +442,7 @@ template <typename T> __global__ void __launch_bounds__(EP_NT, 1) k_ep(EpArgs<T>
               if (!cplx && s < 2) v[e] = s == 0 ? keep[0][e] : keep[KEEP - 1][e];
               else v[e] = arow && l0 + e < n ? arow[sp[l0 + e] * ls] : zero<T>();
             }
-            if (!resident && t >= ad) ok = mbar_wait(&afree[ab], (t / ad - 1) & 1, TW_POLLS);
+            if (!resident && t >= ad) ok = mbar_wait(&afree[ab], (t / ad - 1) & 1, a.polls);
             ok = __all_sync(0xffffffffu, ok) && s_ok;
             if (!ok) break;
             if (ci < srows8) {
@@ -476,7 +478,7 @@ template <typename T> __global__ void __launch_bounds__(EP_NT, 1) k_ep(EpArgs<T>
   __syncthreads();
   if (warp == EP_W) tmem_free(tmem, 512);
   if (!s_ok) {
-    if (tid == 0) atomicExch(a.err, (int)RSS_ETIMEOUT);
+    if (tid == 0) set_error(a.err, RSS_ETIMEOUT);
     return;
   }
   if (a.psplit == 1 && R.Esl != nullptr) {

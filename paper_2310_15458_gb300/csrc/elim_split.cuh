@@ -181,7 +181,7 @@ template <typename T> __global__ void __launch_bounds__(256) k_elim_lu2(ElimArgs
   for (int j = 0; j < r; ++j) {
     __syncthreads();
     if (s_zero[j & 1]) {   // every later kernel of the level still indexes within bounds
-      if (tid == 0) atomicExch(a.err, (int)RSS_ENUMERIC);
+      if (tid == 0) set_error(a.err, RSS_ENUMERIC);
       for (int i = j + tid; i < r; i += blockDim.x) R.piv[i] = i;
       break;
     }

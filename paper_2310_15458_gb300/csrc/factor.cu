@@ -1025,7 +1025,7 @@ template <typename T> __device__ bool lu_pp_block(T* LU, int r, int* piv, int* e
     }
     __syncthreads();
     if (s_zero) {
-      if (tid == 0) atomicExch(err, (int)RSS_ENUMERIC);
+      if (tid == 0) set_error(err, RSS_ENUMERIC);
       for (int i = j + tid; i < r; i += bs) piv[i] = i;
       __syncthreads();
       return false;
@@ -1592,11 +1592,11 @@ constexpr int ST_M = 128, ST_N = 32, ST_KC = 32, ST_NT = 256;
 constexpr int ST_A = OZ_S * ST_M * ST_KC * 2;   // bytes of one chunk of A slices (64 KB)
 constexpr int ST_B = OZ_S * ST_N * ST_KC * 2;   // 16 KB
 constexpr uint32_t ST_TMEM_COLS = OZ_S * ST_N;  // 256
-constexpr long long ST_POLLS = 1LL << 22;
-constexpr long long ST_DRAIN_POLLS = 1LL << 26;
+constexpr int ST_POLLS = 1 << 22;
+constexpr int ST_DRAIN_POLLS = 1 << 26;
 
 __global__ void __launch_bounds__(ST_NT, 2) k_schur_tc(LevelDev<double> L, const BoxRec<double>* recs, int* err,
-                                                        long long polls, int sym) {
+                                                        int polls, int sym) {
   extern __shared__ __align__(1024) unsigned char smraw[];
   __shared__ __align__(8) uint64_t mbar;
   __shared__ uint32_t s_tmem;
@@ -1712,7 +1712,7 @@ __global__ void __launch_bounds__(ST_NT, 2) k_schur_tc(LevelDev<double> L, const
       }
     }
   } else {
-    if (tid == 0) atomicExch(err, (int)RSS_ETIMEOUT);
+    if (tid == 0) set_error(err, RSS_ETIMEOUT);
     if (warp == 0) mbar_wait(&mbar, parity, ST_DRAIN_POLLS);   // products in flight finish before the TMEM is freed
   }
   tc_fence_before();
@@ -1743,7 +1743,7 @@ constexpr int SRW_NT = 512;   // four warps per 32 TMEM lanes, 8 columns of a ti
 constexpr int SRW_XB = 32 * 5 * 8;   // bytes of a warp's transposition
 
 __global__ void __launch_bounds__(SRW_NT, 1) k_schur_tc_rows(LevelDev<double> L, const BoxRec<double>* recs, int* err,
-                                                             long long polls, int sym) {
+                                                             int polls, int sym) {
   extern __shared__ __align__(1024) unsigned char smraw[];
   __shared__ __align__(8) uint64_t mbar[2];
   __shared__ uint32_t s_tmem;
@@ -1922,7 +1922,7 @@ __global__ void __launch_bounds__(SRW_NT, 1) k_schur_tc_rows(LevelDev<double> L,
     for (int j = 0; j < CH; ++j) cv[j] = cvn[j];
   }
   if (!ok) {
-    if (tid == 0) atomicExch(err, (int)RSS_ETIMEOUT);
+    if (tid == 0) set_error(err, RSS_ETIMEOUT);
     if (warp == 0) {   // products in flight (tiles failed_at and failed_at + 1) finish before the TMEM is freed
       mbar_wait(&mbar[failed_at & 1], (uint32_t)(failed_at >> 1) & 1u, ST_DRAIN_POLLS);
       if (failed_at + 1 < ntc)
@@ -2411,8 +2411,23 @@ rss_status factor_impl(const rss_tree* tree, const rss_params* prm, cudaStream_t
   // eliminations, so the conjugate half of the proxy stack repeats the first half
   // and the ID of [A_MB; K_PB] alone is the same ID.
   const int half = (prm->id_rows == 0 && prm->kind == RSS_LAPLACE && prm->diag_im == 0.0) ? 1 : 0;
-  // poll limit of the first barrier wait of the tensor-core Schur updates
-  const long long polls = wait_limit(prm->wait_polls, ST_POLLS);
+  // poll limits of the Schur update's waits on tcgen05 and of the ID's and the panels'
+  const int polls = wait_limit(prm->wait_polls, ST_POLLS);
+  const int tc_polls = prm->schur_path == 0 ? polls : ST_POLLS;
+  // status of the kernels so far (waits for them)
+  auto device_status = [&]() -> rss_status {
+    int herr = 0;
+    RSS_CUDA(cudaMemcpy(&herr, d_err, sizeof(int), cudaMemcpyDeviceToHost));
+    if (herr == RSS_ETIMEOUT) {
+      rss_set_error("rss_factor: a tensor-core barrier wait of the ID, the panels or the Schur update ran out");
+      return RSS_ETIMEOUT;
+    }
+    if (herr) {
+      rss_set_error("rss_factor: zero pivot in the LU of a redundant block");
+      return RSS_ENUMERIC;
+    }
+    return RSS_OK;
+  };
   // A complex symmetric kernel (Helmholtz): the ID of the real stack
   // [Re X; Im X], X = [A_MB; K_PB], which is the ID of the full stack (T real).
   const bool split = std::is_same<T, zd>::value && prm->id_rows == 0 &&
@@ -2660,9 +2675,9 @@ rss_status factor_impl(const rss_tree* tree, const rss_params* prm, cudaStream_t
           const int ntc = cnt <= 152 ? (nmax > 64 ? 1024 : 512) : nmax > 72 ? 512 : nmax > 32 ? 256 : 128;
           k_idg_split<T><<<dim3(w.J * (GI_B / 8), w.nch, cnt), 256, 0, st>>>(a, w);
           RSS_LAUNCHED();
-          k_idg_gram<<<dim3(idg_items(w.J), w.nch, cnt), 256, GI_ST, st>>>(cur.d.n, d_cls + seg0 + c0, w, d_err);
+          k_idg_gram<<<dim3(idg_items(w.J), w.nch, cnt), 256, GI_ST, st>>>(cur.d.n, d_cls + seg0 + c0, w, d_err, tc_polls);
           RSS_LAUNCHED();
-          k_idg_chol<T><<<cnt, ntc, smc, st>>>(a, w);
+          k_idg_chol<T><<<cnt, ntc, smc, st>>>(a, w, d_err);
           RSS_LAUNCHED();
           k_idg_tsolve<T><<<dim3((nmax + 31) / 32, cnt), 128, smt, st>>>(a, w);
           RSS_LAUNCHED();
@@ -2678,6 +2693,7 @@ rss_status factor_impl(const rss_tree* tree, const rss_params* prm, cudaStream_t
       evs.back().second->stop(st);
       RSS_CUDA(cudaMemcpyAsync(hk.data(), d_k, sizeof(int) * nb, cudaMemcpyDeviceToHost, st));
       RSS_CUDA(cudaStreamSynchronize(st));
+      if (nb > 0 && *std::min_element(hk.begin(), hk.begin() + nb) < 0) return device_status();
       f->t_id += tid_.ms();
       const double cf = (sizeof(T) == sizeof(double) || split) ? 1.0 : 4.0;
       for (int q = 0; q < nb; ++q) {   // k steps of Householder QR on the m x n stack
@@ -2922,6 +2938,7 @@ rss_status factor_impl(const rss_tree* tree, const rss_params* prm, cudaStream_t
         ep.cls_idx = d_clsidx;
         ep.perm_in = d_perm;
         ep.err = d_err;
+        ep.polls = tc_polls;
         ep.staged = staged;
         // the passes of a tile over as many CTAs as the tiles leave SMs
         const int tiles = cdiv(max_c, ep.rows);
@@ -3001,13 +3018,8 @@ rss_status factor_impl(const rss_tree* tree, const rss_params* prm, cudaStream_t
       (pe.first == 0 ? info.g_id : pe.first == 1 ? info.g_elim : info.g_schur) += ms;
       (pe.first == 1 ? f->t_elim : pe.first == 2 ? f->t_schur : f->t_gen) += pe.first ? ms : 0.0;
     }
-    int herr = 0;
-    RSS_CUDA(cudaMemcpy(&herr, d_err, sizeof(int), cudaMemcpyDeviceToHost));
-    if (herr == RSS_ETIMEOUT) {
-      rss_set_error("rss_factor: a tensor-core barrier wait of the ID or of the Schur update ran out");
-      return RSS_ETIMEOUT;
-    }
-    if (herr) { rss_set_error("rss_factor: zero pivot in the LU of a redundant block"); return RSS_ENUMERIC; }
+    const rss_status s_dev = device_status();
+    if (s_dev != RSS_OK) return s_dev;
     f->levels.push_back(info);
 
     // merge to the parent level

@@ -176,7 +176,8 @@ __host__ __device__ inline int idg_items(int J) {   // column blocks c and row t
 // Thread 0 of warp 0 feeds the stages by bulk copies, thread 0 of warp 1 issues
 // the products; every wait is bounded, and a wait that runs out sets RSS_ETIMEOUT
 // once the products and copies already issued have finished.
-__global__ void __launch_bounds__(256, 1) k_idg_gram(const int* npts, const int* boxes, GramWs w, int* err) {
+__global__ void __launch_bounds__(256, 1) k_idg_gram(const int* npts, const int* boxes, GramWs w, int* err,
+                                                       int polls) {
   extern __shared__ __align__(1024) unsigned char sm[];
   __shared__ __align__(8) uint64_t full[8], empty[8], done;
   __shared__ uint32_t s_tmem;
@@ -215,7 +216,7 @@ __global__ void __launch_bounds__(256, 1) k_idg_gram(const int* npts, const int*
     const unsigned char* src = slot + (size_t)(part * (w.ch / GI_B)) * OZ_S * J * GI_BLK;
     for (int it = 0; it < nkb; ++it, ++fed) {
       const int s = it % nst;
-      if (it >= nst && !mbar_wait(&empty[s], ((it / nst) - 1) & 1, ST_POLLS)) {
+      if (it >= nst && !mbar_wait(&empty[s], ((it / nst) - 1) & 1, polls)) {
         s_ok = 0;
         break;
       }
@@ -231,7 +232,7 @@ __global__ void __launch_bounds__(256, 1) k_idg_gram(const int* npts, const int*
     int ok = 1;
     for (int it = 0; it < nkb; ++it) {
       const int s = it % nst;
-      if (!mbar_wait(&full[s], (it / nst) & 1, ST_POLLS)) {
+      if (!mbar_wait(&full[s], (it / nst) & 1, polls)) {
         ok = 0;
         break;
       }
@@ -268,7 +269,7 @@ __global__ void __launch_bounds__(256, 1) k_idg_gram(const int* npts, const int*
   tc_fence_after();
   const int ok = s_ok;
   if (!ok && tid == 0) {
-    atomicExch(err, (int)RSS_ETIMEOUT);   // the copies in flight land before the CTA ends
+    set_error(err, RSS_ETIMEOUT);   // the copies in flight land before the CTA ends
     for (int q = max(0, fed - nst); q < fed; ++q) mbar_wait(&full[q % nst], (q / nst) & 1, ST_DRAIN_POLLS);
   }
   if (ok) {
@@ -408,12 +409,17 @@ __host__ __device__ inline size_t idg_chol_bytes(int nmax) {
   return tri * 12 + (size_t)nmax * (sizeof(uint4) + sizeof(double) + 5 * sizeof(int)) + 16;
 }
 
-// One CTA per box: pivoted Cholesky of G.  R (row l of column j at R[j * nmax + l],
+// One CTA per box: pivoted Cholesky of G (k = -1 after an error, *err).  R (row l of column j at R[j * nmax + l],
 // in the columns' scaled units), k, the permutation; then k_idg_tsolve.
-template <typename S> __global__ void __launch_bounds__(1024, 1) k_idg_chol(IdArgs<double, S> a, GramWs w) {
+template <typename S> __global__ void __launch_bounds__(1024, 1) k_idg_chol(IdArgs<double, S> a, GramWs w,
+                                                                             const int* err) {
   extern __shared__ __align__(16) unsigned char sm[];
   const LevelDev<S>& L = a.L;
   const int nmax = L.nmax, box = blockIdx.x, bi = a.base + box, B = a.boxes[bi], n = L.n[B];
+  if (*err != 0) {   // the products did not end: no rank, which ends the factorization
+    if (threadIdx.x == 0) a.k_out[bi] = -1;
+    return;
+  }
   const int J = (n + GI_B - 1) / GI_B;
   const size_t tri = ((size_t)nmax * (nmax + 1) / 2 + 3) & ~size_t(3);
   uint4* row = reinterpret_cast<uint4*>(sm);   // limbs and sign of the new row of R
@@ -606,7 +612,7 @@ template <typename S> __global__ void __launch_bounds__(128) k_idg_tsolve(IdArgs
   const LevelDev<S>& L = a.L;
   const int nmax = L.nmax, box = blockIdx.y, bi = a.base + box, B = a.boxes[bi], n = L.n[B];
   const int k = a.k_out[bi], r = n - k, c0 = blockIdx.x * 32;
-  if (c0 >= r || k == 0) return;
+  if (c0 >= r || k <= 0) return;
   unsigned char* slot = w.p + (size_t)box * w.slot;
   const double* R = reinterpret_cast<const double*>(slot + w.o_R);
   const double* rinv = R + (size_t)nmax * nmax;

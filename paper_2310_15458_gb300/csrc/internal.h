@@ -12,8 +12,8 @@
 constexpr int SWP_SPREAD_DEFAULT = 4;   // reported for tables that carry a spread; no launch form uses it
 
 // polls of a bounded device wait: rss_params.wait_polls, 0 for the wait's own limit, -1 for none
-inline long long wait_limit(int wait_polls, long long limit) {
-  return wait_polls == 0 ? limit : wait_polls < 0 ? 0 : (long long)wait_polls;
+inline int wait_limit(int wait_polls, int limit) {
+  return wait_polls == 0 ? limit : std::max(wait_polls, 0);
 }
 
 enum : uint32_t { RSS_TAG_TREE = 0x52545245u, RSS_TAG_FACTOR = 0x52464143u, RSS_TAG_SERVER = 0x52535256u };

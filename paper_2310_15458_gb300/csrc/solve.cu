@@ -202,7 +202,7 @@ rss_status top_apply(const rss_factorization* f, T* x, int64_t ldx, int nrhs, cu
 // block.  Shared memory: the most any class needs without staging its matrices
 // (at least 16 KB; more room lets them be staged); the grid: as many CTAs as fit
 // on the device at once (a cooperative launch needs all of them resident).
-constexpr long long SWP_POLLS = 1LL << 24;
+constexpr int SWP_POLLS = 1 << 24;
 
 template <typename T, int RC> size_t sweep_persistent_smem(const rss_factorization* f, int k0) {
   size_t need = 0;
@@ -473,7 +473,7 @@ rss_status sweeps_tc(const rss_factorization* f, T* x, int64_t ldx, int nrhs, cu
   const SweepWs w = sweep_ws<T>(f, nrhs, RC);
   T* topz = reinterpret_cast<T*>(static_cast<char*>(ws) + w.topz_off);
   int* err = reinterpret_cast<int*>(static_cast<char*>(ws) + w.bar_off + 2 * sizeof(unsigned));
-  const int polls = (int)wait_limit(f->params.wait_polls, TW_POLLS);
+  const int polls = wait_limit(f->params.wait_polls, TW_POLLS);
   auto product = [&](size_t bi, auto op) -> cudaError_t {
     constexpr int OP = decltype(op)::value;
     const Batch& b = f->batches[bi];

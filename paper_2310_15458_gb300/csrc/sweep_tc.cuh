@@ -387,7 +387,7 @@ __global__ void __launch_bounds__(TW_NT, 1) k_tw(const BoxRec<T>* __restrict__ r
       }
     }
   } else if (tid == 0) {
-    atomicExch(err, (int)RSS_ETIMEOUT);
+    set_error(err, RSS_ETIMEOUT);
     // what is in flight (products, copies) ends before the buffers and the tensor memory go
     for (int q = max(0, issued - nst); q < issued; ++q) mbar_wait(&mb_mma[q % nst], (q / nst) & 1, TW_DRAIN);
     if (CACHE)

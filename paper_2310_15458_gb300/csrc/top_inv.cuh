@@ -73,7 +73,7 @@ __global__ void __launch_bounds__(512) k_gj_panel(const T* __restrict__ in, int 
   for (int j = 0; j < w; ++j) {
     __syncthreads();
     if (s_zero[j & 1]) {   // the inverse does not exist: every index stays within bounds
-      if (tid == 0) atomicExch(err, (int)RSS_ENUMERIC);
+      if (tid == 0) set_error(err, RSS_ENUMERIC);
       for (int i = j + tid; i < w; i += blockDim.x) piv[jb + i] = jb + i;
       break;
     }

@@ -13,7 +13,7 @@ constexpr int TW_KX = OZ_KX;                             // sums exact in FP32
 constexpr int TW_KN = OZ_KN;                             // ... and below 2^22 (oz_fint)
 constexpr int TW_A = OZ_S * TW_M * TW_K * 2;             // bytes of a stage: 64 KB
 constexpr int TW_B = OZ_S * TW_NC * TW_K * 2;            // 32 KB
-constexpr long long TW_POLLS = 1LL << 22, TW_DRAIN = 1LL << 26;
+constexpr int TW_POLLS = 1 << 22, TW_DRAIN = 1 << 26;
 
 __device__ __forceinline__ unsigned long long tw_key(double x) { return oz_abs_bits(x); }
 __device__ __forceinline__ unsigned long long tw_key(zd x) { return max(oz_abs_bits(x.x), oz_abs_bits(x.y)); }

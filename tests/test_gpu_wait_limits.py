@@ -49,3 +49,20 @@ def test_tensor_core_sweeps(P, kind, side, leaf):
     P.rss_solve(good, x.T)
     P.rss_solve(bad, one)   # (one column: no bounded wait)
     assert float(torch.linalg.vector_norm(x[3] - one) / torch.linalg.vector_norm(one)) <= 1e-12
+
+
+@pytest.mark.parametrize("kind,side,leaf,id_cluster", [
+    ("laplace", 64, 64, 0), ("helmholtz", 64, 64, 0), ("laplace", 256, 16, 0),    # the ID's products, first
+    ("laplace", 64, 64, 1), ("laplace", 128, 16, 1), ("laplace", 96, 36, 1),      # reflectors: panels, then Schur
+    ("helmholtz", 64, 64, 1), ("helmholtz", 128, 16, 1), ("helmholtz", 96, 144, 1),
+    ("laplace", 96, 144, 1), ("laplace", 64, 256, 1)])                            # FP64 panels: Schur alone
+def test_factorization(P, kind, side, leaf, id_cluster):
+    cplx, tree, arg = problem(P, kind, side, leaf, id_cluster=id_cluster)
+    for _ in range(2):
+        with pytest.raises(P.RSSError, match="ETIMEOUT") as ei:
+            P.rss_factor(tree, wait_polls=-1, **arg)
+        assert ei.value.status == 5
+    b = torch.from_numpy(W.gaussian_rhs(tree.n, 1, cplx, 6)[:, 0].copy()).cuda()
+    f = P.rss_factor(tree, **arg)
+    r = P.rss_matvec(f, P.rss_solve(f, b.clone())) - b
+    assert float(torch.linalg.vector_norm(r) / torch.linalg.vector_norm(b)) <= 1e-5
