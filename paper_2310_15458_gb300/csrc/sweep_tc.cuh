@@ -182,7 +182,12 @@ __global__ void __launch_bounds__(TW_NT, 1) k_tw(const BoxRec<T>* __restrict__ r
   const int nsall = (Kall + KS - 1) / KS, s0 = nsall * rank / spl, ns = nsall * (rank + 1) / spl - s0;
   const int K0 = s0 * KS, K = min(Kall, (s0 + ns) * KS);   // this CTA's entries of K
   pdl_launch();
-  if (rows <= 0) return;
+  // (a launch without a row, E where every box has c = 0, must not end before the launch
+  // before it: the next launch waits for this one alone)
+  if (rows <= 0) {
+    pdl_wait();
+    return;
+  }
   const int q0 = blockIdx.y * NC, nq = min(NC, nrhs - q0);
   const int gn = cplx || nq > GW ? 2 : 1;   // groups that hold columns
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
