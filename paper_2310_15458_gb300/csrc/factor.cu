@@ -2570,12 +2570,12 @@ rss_status factor_impl(const rss_tree* tree, const rss_params* prm, cudaStream_t
           rss_set_error("rss_factor: proxy stack of a box too tall for the on-chip reflector buffer");
           return RSS_EINVAL;
         }
-        RSS_CUDA(cudaFuncSetAttribute(k_id<TC, T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_id));
+        RSS_CUDA(allow_smem(k_id<TC, T>));
         auto kcl = k_id_cl<TC, T, 256>;
         if constexpr (sizeof(TC) == sizeof(double))
           if (ntc == 512) kcl = k_id_cl<TC, T, 512>;
         if (Q > 1) {
-          RSS_CUDA(cudaFuncSetAttribute(kcl, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_cl));
+          RSS_CUDA(allow_smem(kcl));
           if (Q > 8) RSS_CUDA(cudaFuncSetAttribute(kcl, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
         }
         f->peak_transient = std::max(f->peak_transient, transient + slot * chunk);
@@ -2650,9 +2650,9 @@ rss_status factor_impl(const rss_tree* tree, const rss_params* prm, cudaStream_t
         w.p = static_cast<unsigned char*>(gb_Y.p);
         f->peak_transient = std::max(f->peak_transient, transient + w.slot * chunk);
         const size_t smc = idg_chol_bytes(nmax), smt = idg_tsolve_bytes(nmax);
-        RSS_CUDA(cudaFuncSetAttribute(k_idg_gram, cudaFuncAttributeMaxDynamicSharedMemorySize, GI_ST));
-        RSS_CUDA(cudaFuncSetAttribute(k_idg_chol<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smc));
-        RSS_CUDA(cudaFuncSetAttribute(k_idg_tsolve<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smt));
+        RSS_CUDA(allow_smem(k_idg_gram));
+        RSS_CUDA(allow_smem(k_idg_chol<T>));
+        RSS_CUDA(allow_smem(k_idg_tsolve<T>));
         IdArgs<double, T> a{};
         a.L = cur.d;
         a.boxes = d_cls + seg0;
@@ -2891,14 +2891,14 @@ rss_status factor_impl(const rss_tree* tree, const rss_params* prm, cudaStream_t
       if (elim_cols) {
         // columns per CTA: as many as still give every SM two CTAs
         auto launch_x = [&](auto kern, int jc, size_t smem) -> cudaError_t {
-          cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+          cudaError_t e = allow_smem(kern);
           if (e != cudaSuccess) return e;
           kern<<<dim3((max_r + jc - 1) / jc, nrec), 256, smem, st>>>(ea);
           return cudaGetLastError();
         };
         auto launch_inv = [&](auto kern, int nbc) -> cudaError_t {
           const size_t smem = elim_inv_bytes<T>(nbc, max_r);
-          cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+          cudaError_t e = allow_smem(kern);
           if (e != cudaSuccess) return e;
           kern<<<dim3((max_r + nbc - 1) / nbc, 2, nrec), 16 * nbc, smem, st>>>(ea);
           return cudaGetLastError();
@@ -2909,19 +2909,19 @@ rss_status factor_impl(const rss_tree* tree, const rss_params* prm, cudaStream_t
         const size_t lub = std::min<size_t>(sizeof(T) * (size_t)max_r * (max_r | 1), 224 * 1024) + sizeof(int) * (size_t)max_r;
         const size_t lus = std::min<size_t>(lub, 224 * 1024);
         ea.smem_cap = (int)(lus / sizeof(T));
-        RSS_CUDA(cudaFuncSetAttribute(k_elim_lu2<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)lus));
+        RSS_CUDA(allow_smem(k_elim_lu2<T>));
         k_elim_lu2<T><<<nrec, 256, lus, st>>>(ea);
         RSS_LAUNCHED();
         RSS_CUDA(2 * groups < 2 * 152 ? launch_inv(k_elim_inv<T, 8>, 8) : launch_inv(k_elim_inv<T, 16>, 16));
         f->launches += 2;
       } else {
-        RSS_CUDA(cudaFuncSetAttribute(k_elim_lu<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ecap));
+        RSS_CUDA(allow_smem(k_elim_lu<T>));
         k_elim_lu<T><<<nrec, NT, ecap, st>>>(ea);
       }
       RSS_LAUNCHED();
       if (pan_max > 0) {
         auto launch_panels = [&](auto kern, int rows) -> cudaError_t {
-          cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)pan_max);
+          cudaError_t e = allow_smem(kern);
           if (e != cudaSuccess) return e;
           kern<<<dim3((max_c + rows - 1) / rows, nrec), NT, pan_max, st>>>(ea);
           return cudaGetLastError();
@@ -2944,7 +2944,7 @@ rss_status factor_impl(const rss_tree* tree, const rss_params* prm, cudaStream_t
         const int tiles = cdiv(max_c, ep.rows);
         ep.psplit = std::max(1, std::min<int>(ep.ng, 152 / std::max<long long>(1, (long long)tiles * ep.sets * nrec)));
         const int smem = ep.ad * ep.rows * OZ_S * TW_K * 2 + ep.wd * ep_parts<T>() * EP_GB + (ep.spn + ep.nstr * TW_M) * (int)sizeof(int);
-        RSS_CUDA(cudaFuncSetAttribute(k_ep<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+        RSS_CUDA(allow_smem(k_ep<T>, 225 * 1024));
         k_ep_cut_w<T><<<dim3(ep.ng, ep.sets, nrec), EP_WT, 0, st>>>(ep);
         RSS_LAUNCHED();
         k_ep<T><<<dim3(tiles, ep.sets * ep.psplit, nrec), EP_NT, smem, st>>>(ep);
@@ -2967,16 +2967,16 @@ rss_status factor_impl(const rss_tree* tree, const rss_params* prm, cudaStream_t
             // tcgen05, one CTA per 128-row block walking its column tiles (one CTA per SM)
             const int nchm = (kp_max + ST_KC - 1) / ST_KC;
             const int smem = std::max(nchm * (ST_A + 2 * ST_B) + SRW_NT / 32 * SRW_XB, 120 * 1024);
-            RSS_CUDA(cudaFuncSetAttribute(k_schur_tc_rows, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+            RSS_CUDA(allow_smem(k_schur_tc_rows));
             k_schur_tc_rows<<<dim3(ntr_rows, nrec), SRW_NT, smem, st>>>(cur.d, d_recs, d_err, polls, sym);
           } else if (prm->schur_path == 0 && kp_max <= OZ_KX) {   // tcgen05: FP32 group sums over the whole K
             const int smem = ST_A + ST_B;
-            RSS_CUDA(cudaFuncSetAttribute(k_schur_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+            RSS_CUDA(allow_smem(k_schur_tc));
             const int ntr = (max_c + ST_M - 1) / ST_M, ntc = (max_c + ST_N - 1) / ST_N;
             k_schur_tc<<<dim3(ntr * ntc, nrec), ST_NT, smem, st>>>(cur.d, d_recs, d_err, polls, sym);
           } else {
             const size_t smem = 2 * (size_t)SR_BUF * sizeof(uint16_t);
-            RSS_CUDA(cudaFuncSetAttribute(k_schur_oz, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+            RSS_CUDA(allow_smem(k_schur_oz));
             const int ntr = (max_c + SR_M - 1) / SR_M, ntc = (max_c + SR_N - 1) / SR_N;
             k_schur_oz<<<dim3(ntr * ntc, nrec), NT, smem, st>>>(cur.d, d_recs, sym);
           }
@@ -2986,11 +2986,11 @@ rss_status factor_impl(const rss_tree* tree, const rss_params* prm, cudaStream_t
             const int ad = nst > 2 ? 3 : 2, nb = ad == 3 ? 5 : 6;   // stages of rows, pieces of columns in shared memory
             const int smem = ad * trows * SZ_AST + nb * SZ_BP;
             const int csplit = std::max(1, std::min<int>(cdiv(max_c, 32), 152 / std::max(1, ntr * nrec)));
-            RSS_CUDA(cudaFuncSetAttribute(k_schur_z, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+            RSS_CUDA(allow_smem(k_schur_z));
             k_schur_z<<<dim3(nrec, csplit, ntr), EP_NT, smem, st>>>(cur.d, d_recs, trows, ad, nb, csplit, split ? 1 : 0, d_err, polls);
           } else {
             const size_t smem = (64 + 32) * (size_t)SCSA * sizeof(uint16_t);
-            RSS_CUDA(cudaFuncSetAttribute(k_schur_oz_c, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+            RSS_CUDA(allow_smem(k_schur_oz_c));
             const int ntc = (max_c + 31) / 32;
             k_schur_oz_c<<<dim3(ntile * ntc, nrec), NT, smem, st>>>(cur.d, d_recs);
           }
@@ -3087,7 +3087,7 @@ rss_status factor_impl(const rss_tree* tree, const rss_params* prm, cudaStream_t
     {
       const size_t msmem = (size_t)par.d.nmax * (2 * sizeof(int) + 2 * sizeof(int2));
       if (msmem > 48 * 1024)
-        RSS_CUDA(cudaFuncSetAttribute(k_merge_blk<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)msmem));
+        RSS_CUDA(allow_smem(k_merge_blk<T>));
       k_merge_blk<T><<<gp * gp * 25, NT, msmem, st>>>(cur.d, par.d, d_ixy, d_tab, f->kp, side);
     }
     RSS_LAUNCHED();

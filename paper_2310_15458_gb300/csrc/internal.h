@@ -11,6 +11,16 @@
 
 constexpr int SWP_SPREAD_DEFAULT = 4;   // reported for tables that carry a spread; no launch form uses it
 
+// Lets a kernel be launched with up to `bytes` of dynamic shared memory.  The attribute
+// belongs to the function on the device, not to the call: set to a launch's own size, it
+// could be lowered by another host thread before that launch, which is then refused.  So
+// every caller sets the same value, the most that any launch of the kernel takes (beside
+// up to 3 KB of static shared memory).
+constexpr int SMEM_DYN = 224 * 1024;
+template <typename K> cudaError_t allow_smem(K kern, int bytes = SMEM_DYN) {
+  return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+}
+
 // polls of a bounded device wait: rss_params.wait_polls, 0 for the wait's own limit, -1 for none
 inline int wait_limit(int wait_polls, int limit) {
   return wait_polls == 0 ? limit : std::max(wait_polls, 0);

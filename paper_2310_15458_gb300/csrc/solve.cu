@@ -237,7 +237,7 @@ rss_status sweep_persistent_launch(const rss_factorization* f, T* x, int64_t ldx
   void* args[] = {&a};
   const void* fn = up ? reinterpret_cast<const void*>(k_sweep<T, RC, true>)
                       : reinterpret_cast<const void*>(k_sweep<T, RC, false>);
-  RSS_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  RSS_CUDA(allow_smem(fn));
   int per_sm = 0;
   RSS_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, SWP_NT, smem));
   if (per_sm < 1) {
@@ -296,7 +296,7 @@ rss_status sweep_class(const Batch& b, T* x, int64_t ldx, int nrhs, cudaStream_t
     }
   }
   const size_t smem = fills ? s.need * sizeof(T) : std::min<size_t>(s.full * sizeof(T), 220 * 1024);
-  RSS_CUDA(cudaFuncSetAttribute(k_sweep_cl<T, RC, UP>, cudaFuncAttributeMaxDynamicSharedMemorySize, 220 * 1024));
+  RSS_CUDA(allow_smem(k_sweep_cl<T, RC, UP>));
   RSS_CUDA(launch_pdl(k_sweep_cl<T, RC, UP>, dim3(b.nrec * Q, (unsigned)nz), fills ? 128 : SW_NT, smem, st, Q,
                       static_cast<const BoxRec<T>*>(b.d_recs), x, ldx, nrhs, Q, qc, (int)(smem / sizeof(T))));
   return RSS_OK;
@@ -433,7 +433,7 @@ cudaError_t launch_tw_gw(const Batch& b, const SliceRec* sl, T* x, int64_t ldx, 
   const int mr = OP == TW_UPE ? std::max(1, b.max_c) : OP == TW_DNW ? b.max_n : b.max_r;
   const int mk = OP == TW_UPW ? b.max_n : OP == TW_DNF ? b.max_c : b.max_r;
   const TwPlan p = tw_plan(mr, mk, GW, real ? TW_K : TW_K / 2, tw_stretch<T>());
-  const cudaError_t e = cudaFuncSetAttribute(k_tw<T, OP, CACHE, GW>, cudaFuncAttributeMaxDynamicSharedMemorySize, p.smem);
+  const cudaError_t e = allow_smem(k_tw<T, OP, CACHE, GW>);
   if (e != cudaSuccess) return e;
   // a property of the class alone, so that a column's bits do not depend on the others
   int spl = 1;

@@ -204,7 +204,7 @@ int gj_inverse(T* const buf[2], T* inv, int n, T* D, int* src, int* piv, int* er
   if (ib > 200 * 1024) return -1;
   const bool onchip = full <= 200 * 1024;
   const size_t smem = onchip ? full : ib;
-  if (cudaFuncSetAttribute(k_gj_panel<T, NB>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) return -1;
+  if (allow_smem(k_gj_panel<T, NB>) != cudaSuccess) return -1;
   int cur = 0, launches = 0;
   for (int jb = 0; jb < n; jb += NB) {
     k_gj_panel<T, NB><<<1, 512, smem, st>>>(buf[cur], n, jb, D, src, piv, err, onchip ? nullptr : scratch);
