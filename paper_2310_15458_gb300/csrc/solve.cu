@@ -16,6 +16,7 @@
 
 #include "internal.h"
 #include "tw_common.cuh"
+#include "tw_plan.h"
 
 namespace {
 
@@ -338,10 +339,10 @@ rss_status sweeps(const rss_factorization* f, T* x, int64_t ldx, int nrhs, cudaS
 // The digits of a real factor's matrices for the tensor-core sweeps: built once per
 // factor by the first solve that needs them (on its stream, which it then waits for),
 // kept until the factor is freed.
-bool tw_fits(const Batch& b) { return b.max_n <= TW_MAXN && b.max_c <= TW_MAXC; }
+bool tw_fits(const Batch& b, bool real) { return tw_shape_fits(b.max_n, b.max_r, b.max_c, real); }
 // whether a class takes the tensor-core products in a call with nrhs right-hand sides
 bool tw_takes(const Batch& b, int64_t nrhs, bool real) {
-  return tw_fits(b) && (nrhs >= TCB || !real || b.nrec >= TCMIN);
+  return tw_fits(b, real) && (nrhs >= TCB || !real || b.nrec >= TCMIN);
 }
 struct SliceSize {
   size_t dig[4], eb[4];
@@ -364,7 +365,7 @@ size_t slice_total(const rss_factorization* f) {
     const Batch& b = f->batches[bi];
     const BoxRec<double>* hr = static_cast<const BoxRec<double>*>(f->rec_host[bi]);
     total += al(sizeof(SliceRec) * b.nrec);
-    if (!tw_fits(b)) continue;
+    if (!tw_fits(b, true)) continue;
     for (int q = 0; q < b.nrec; ++q) {
       const SliceSize z = slice_size(hr[q]);
       for (int op = 0; op < 4; ++op) total += z.dig[op] + z.eb[op];
@@ -393,7 +394,7 @@ rss_status ensure_slices(rss_factorization* f, cudaStream_t st) {
     const Batch& b = f->batches[bi];
     const BoxRec<double>* hr = static_cast<const BoxRec<double>*>(f->rec_host[bi]);
     recs[bi] = reinterpret_cast<SliceRec*>(take(sizeof(SliceRec) * b.nrec));
-    if (!tw_fits(b)) continue;
+    if (!tw_fits(b, true)) continue;
     hs[bi].assign(b.nrec, SliceRec{});
     for (int q = 0; q < b.nrec; ++q) {
       const SliceSize z = slice_size(hr[q]);
@@ -432,7 +433,7 @@ cudaError_t launch_tw_gw(const Batch& b, const SliceRec* sl, T* x, int64_t ldx, 
   constexpr bool real = sizeof(T) == sizeof(double);
   const int mr = OP == TW_UPE ? std::max(1, b.max_c) : OP == TW_DNW ? b.max_n : b.max_r;
   const int mk = OP == TW_UPW ? b.max_n : OP == TW_DNF ? b.max_c : b.max_r;
-  const TwPlan p = tw_plan(mr, mk, GW, real ? TW_K : TW_K / 2, tw_stretch<T>());
+  const TwPlan p = tw_plan_op(OP, b.max_n, b.max_r, b.max_c, GW, real);
   const cudaError_t e = allow_smem(k_tw<T, OP, CACHE, GW>);
   if (e != cudaSuccess) return e;
   // a property of the class alone, so that a column's bits do not depend on the others

@@ -24,15 +24,14 @@
 // one CTA per box (real) and the FP64 sweeps (complex): Laplace 512^2 23.3 -> 9.2 ms,
 // Helmholtz 256^2 30.3 -> 11.9 ms; 16 columns, against the FP64 sweeps: 4.6 -> 3.4 ms
 // (Laplace 256^2).
-constexpr int TW_MAXN = 128;                             // rows of the products that write what they read
-constexpr int TW_MAXC = 6000;                            // entries of K whose places fit beside the stages
 // Stages of K that share scales and sums.  Complex sums restart more often: against the
 // records applied in quadruple precision (Helmholtz, 64^2, leaf 64) a panel's error is
 // then 9.8e-16, of one-column FP64 solves 1.00e-15; stretches of 128, 192 and 384 give
 // 1.06e-15, 1.08e-15 and 1.14e-15, in 11.0, 10.7 and 10.2 ms instead of 11.9 (256^2, 64
 // columns).  Laplace: 3.34e-16, FP64 3.36e-16.
 template <typename T> __host__ __device__ constexpr int tw_stretch() { return (sizeof(T) == sizeof(double) ? TW_KX : TW_KN) / TW_K; }
-enum { TW_UPW = 0, TW_UPE = 1, TW_DNF = 2, TW_DNW = 3 };
+// (tw_plan.h sizes the launches)
+static_assert(TW_M == 128 && TW_K == 32 && OZ_S == 8 && tw_stretch<double>() == 12 && tw_stretch<zd>() == 3, "");
 
 // rows and inner dimension of a product
 template <int OP, typename T> __host__ __device__ inline int tw_rows(const BoxRec<T>& R) {
@@ -137,24 +136,6 @@ __global__ void __launch_bounds__(TW_NT) k_tw_cache(const BoxRec<double>* __rest
     tw_cut_a<OP>(R, i0, rows, K, s, reb[s / (TW_KX / TW_K)], base + (size_t)s * OZ_S * rows8 * 64, (size_t)rows8 * 64);
   for (int st = 0; st * TW_KX < K; ++st)
     for (int i = threadIdx.x; i < rows; i += TW_NT) S.eb[OP][(size_t)st * M + i0 + i] = reb[st][i];
-}
-
-// Shared memory of a launch: NST stages of the rows' digits (rows8 rows) and of 2 GW
-// real columns, then the places in x of the K rows and the exponents of rows and
-// columns in up to nstr stretches of K.
-struct TwPlan {
-  int rows8, nst, nstr, smem;
-};
-inline TwPlan tw_plan(int max_rows, int max_k, int gw, int ks, int sx) {
-  TwPlan p;
-  p.rows8 = std::min(TW_M, (max_rows + 7) & ~7);
-  const int st = p.rows8 * OZ_S * TW_K * 2 + OZ_S * 2 * gw * TW_K * 2, ns = (max_k + ks - 1) / ks;
-  // the products of a short tile read (and ignore) up to 128 rows past each slice
-  p.nstr = (ns + sx - 1) / sx + 1;   // (a share of K may start inside a stretch)
-  const int tail = sizeof(int) * (max_k + p.nstr * (TW_M + 2 * gw)) + (TW_M - p.rows8) * 64;
-  p.nst = std::max(2, std::min({4, std::max(ns, 2), (222 * 1024 - tail) / st}));
-  p.smem = p.nst * st + tail;
-  return p;
 }
 
 // GW: columns of a group (32, or 16 for classes of few boxes: more and shorter CTAs)
