@@ -87,7 +87,7 @@ __global__ void __launch_bounds__(NT) k_perm_out(T* __restrict__ b, int64_t ldb,
 // of fewer than TCMIN boxes, where four launches of the products take longer than one of
 // the FP64 sweep, left to the latter; at 64^2 every class).  From TCB on a real factor
 // keeps its digits, which a first call builds, and all classes that fit take the products.
-constexpr int TCN = 16, TCB = 32, TCMIN = 16;
+constexpr int TCN = 16, TCB = 32, TCL = 64, TCMIN = 16;
 
 // Top block: x_top <- A_top^{-1} x_top with the inverse formed at factor time.
 template <typename T>
@@ -341,19 +341,24 @@ rss_status sweeps(const rss_factorization* f, T* x, int64_t ldx, int nrhs, cudaS
 // kept until the factor is freed.
 bool tw_fits(const Batch& b, bool real) { return tw_shape_fits(b.max_n, b.max_r, b.max_c, real); }
 // whether a class takes the tensor-core products in a call with nrhs right-hand sides
+// (real classes of at most four boxes of 129 to 192 points: FP64 below TCL; 128^2, eps
+// 1e-9: 32 columns 2.64 ms so, 2.77 with products; boxes of 256 points, 64^2: 1.83 and 1.51)
 bool tw_takes(const Batch& b, int64_t nrhs, bool real) {
-  return tw_fits(b, real) && (nrhs >= TCB || !real || b.nrec >= TCMIN);
+  if (!tw_fits(b, real)) return false;
+  if (!real || nrhs >= TCL) return true;
+  if (b.nrec <= 4 && b.max_n > TW_M && b.max_n <= 192) return false;
+  return nrhs >= TCB || b.nrec >= TCMIN;
 }
 struct SliceSize {
   size_t dig[4], eb[4];
 };
-SliceSize slice_size(const BoxRec<double>& R) {
+SliceSize slice_size(const BoxRec<double>& R, int kx) {   // kx: entries of K of a stretch
   auto al = [](size_t b) { return (b + 255) & ~size_t(255); };
   const int n = R.k + R.r, rows[4] = {R.r, R.c, R.r, n}, inner[4] = {n, R.r, R.c, R.r};
   SliceSize s;
   for (int op = 0; op < 4; ++op) {
     s.dig[op] = al(tw_cache_bytes(rows[op], inner[op]));
-    s.eb[op] = al(sizeof(int) * rows[op] * ((inner[op] + TW_KX - 1) / TW_KX));
+    s.eb[op] = al(sizeof(int) * rows[op] * ((inner[op] + kx - 1) / kx));
   }
   return s;
 }
@@ -367,7 +372,7 @@ size_t slice_total(const rss_factorization* f) {
     total += al(sizeof(SliceRec) * b.nrec);
     if (!tw_fits(b, true)) continue;
     for (int q = 0; q < b.nrec; ++q) {
-      const SliceSize z = slice_size(hr[q]);
+      const SliceSize z = slice_size(hr[q], TW_K * tw_stages(true, b.max_n));
       for (int op = 0; op < 4; ++op) total += z.dig[op] + z.eb[op];
     }
   }
@@ -397,7 +402,7 @@ rss_status ensure_slices(rss_factorization* f, cudaStream_t st) {
     if (!tw_fits(b, true)) continue;
     hs[bi].assign(b.nrec, SliceRec{});
     for (int q = 0; q < b.nrec; ++q) {
-      const SliceSize z = slice_size(hr[q]);
+      const SliceSize z = slice_size(hr[q], TW_K * tw_stages(true, b.max_n));
       for (int op = 0; op < 4; ++op) {
         hs[bi][q].dig[op] = reinterpret_cast<unsigned char*>(take(z.dig[op]));
         hs[bi][q].eb[op] = reinterpret_cast<int*>(take(z.eb[op]));
@@ -406,11 +411,16 @@ rss_status ensure_slices(rss_factorization* f, cudaStream_t st) {
     e = cudaMemcpyAsync(recs[bi], hs[bi].data(), sizeof(SliceRec) * b.nrec, cudaMemcpyHostToDevice, st);
     if (e != cudaSuccess) break;
     const BoxRec<double>* dr = static_cast<const BoxRec<double>*>(b.d_recs);
-    const unsigned tc = std::max(1u, cdiv(b.max_c, TW_M));
-    k_tw_cache<TW_UPW><<<dim3(1, b.nrec), TW_NT, 0, st>>>(dr, recs[bi]);
-    k_tw_cache<TW_UPE><<<dim3(tc, b.nrec), TW_NT, 0, st>>>(dr, recs[bi]);
-    k_tw_cache<TW_DNF><<<dim3(1, b.nrec), TW_NT, 0, st>>>(dr, recs[bi]);
-    k_tw_cache<TW_DNW><<<dim3(1, b.nrec), TW_NT, 0, st>>>(dr, recs[bi]);
+    const unsigned tr = cdiv(b.max_r, TW_M), tc = std::max(1u, cdiv(b.max_c, TW_M)), tn = cdiv(b.max_n, TW_M);
+    auto cut = [&](auto sx) {
+      constexpr int SX = decltype(sx)::value;
+      k_tw_cache<TW_UPW, SX><<<dim3(tr, b.nrec), TW_NT, 0, st>>>(dr, recs[bi]);
+      k_tw_cache<TW_UPE, SX><<<dim3(tc, b.nrec), TW_NT, 0, st>>>(dr, recs[bi]);
+      k_tw_cache<TW_DNF, SX><<<dim3(tr, b.nrec), TW_NT, 0, st>>>(dr, recs[bi]);
+      k_tw_cache<TW_DNW, SX><<<dim3(tn, b.nrec), TW_NT, 0, st>>>(dr, recs[bi]);
+    };
+    if (tw_stages(true, b.max_n) == TW_SX) cut(std::integral_constant<int, TW_SX>{});
+    else cut(std::integral_constant<int, TW_SX_LONG>{});
     e = cudaGetLastError();
   }
   if (e == cudaSuccess) e = cudaStreamSynchronize(st);   // other streams may use the digits from here on
@@ -427,32 +437,44 @@ rss_status ensure_slices(rss_factorization* f, cudaStream_t st) {
   return RSS_OK;
 }
 
-template <typename T, int OP, bool CACHE, int GW>
+template <typename T, int OP, bool CACHE, int GW, int SX>
 cudaError_t launch_tw_gw(const Batch& b, const SliceRec* sl, T* x, int64_t ldx, int nrhs, int* err, int polls,
                          cudaStream_t st) {
   constexpr bool real = sizeof(T) == sizeof(double);
   const int mr = OP == TW_UPE ? std::max(1, b.max_c) : OP == TW_DNW ? b.max_n : b.max_r;
   const int mk = OP == TW_UPW ? b.max_n : OP == TW_DNF ? b.max_c : b.max_r;
   const TwPlan p = tw_plan_op(OP, b.max_n, b.max_r, b.max_c, GW, real);
-  const cudaError_t e = allow_smem(k_tw<T, OP, CACHE, GW>);
+  const int tiles = cdiv(mr, TW_M);
+  const cudaError_t e = allow_smem(k_tw<T, OP, CACHE, GW, SX>);
   if (e != cudaSuccess) return e;
   // a property of the class alone, so that a column's bits do not depend on the others
   int spl = 1;
   if (OP == TW_DNF)
-    while (spl < 8 && b.nrec * spl <= 76 && mk >= 16 * spl * (real ? TW_K : TW_K / 2)) spl *= 2;
-  return launch_pdl(k_tw<T, OP, CACHE, GW>, dim3(spl * cdiv(mr, TW_M), cdiv(nrhs, real ? 2 * GW : GW), b.nrec), TW_NT,
-                    p.smem, st, spl, static_cast<const BoxRec<T>*>(b.d_recs), sl, x, ldx, nrhs, p.rows8, p.nst, p.nstr, err,
+    while (spl < 8 && b.nrec * tiles * spl <= 76 && mk >= 16 * spl * (real ? TW_K : TW_K / 2)) spl *= 2;
+  return launch_pdl(k_tw<T, OP, CACHE, GW, SX>, dim3(spl * tiles, cdiv(nrhs, real ? 2 * GW : GW), b.nrec), TW_NT,
+                    p.smem, st, OP == TW_UPW || OP == TW_DNW ? tiles : spl, static_cast<const BoxRec<T>*>(b.d_recs), sl, x, ldx, nrhs, p.rows8, p.nst, p.nstr, err,
                     polls);
 }
 
-// 16 columns to a group where 32 would leave half of the SMs without a CTA
+// 16 columns to a group where 32 would leave half of the SMs without a CTA, or do not fit.
+// Real classes of more than 128 points take stretches of 64 entries: a panel's error against
+// quadruple precision is then 3.65e-16 (96^2, leaf 144; FP64 columns 4.03e-16, stretches of
+// 384 4.56e-16) and 3.61e-16 (64^2, leaf 256; 4.47e-16 and 5.41e-16).
 template <typename T, int OP, bool CACHE>
 cudaError_t launch_tw(const Batch& b, const SliceRec* sl, T* x, int64_t ldx, int nrhs, int* err, int polls,
                       cudaStream_t st) {
-  const long long tiles = OP == TW_UPE ? cdiv(std::max(1, b.max_c), TW_M) : 1;
-  const bool few = tiles * b.nrec * cdiv(nrhs, sizeof(T) == sizeof(double) ? TW_NC : TW_NC / 2) <= 76;
-  return few || nrhs <= 16 ? launch_tw_gw<T, OP, CACHE, 16>(b, sl, x, ldx, nrhs, err, polls, st)
-             : launch_tw_gw<T, OP, CACHE, 32>(b, sl, x, ldx, nrhs, err, polls, st);
+  constexpr bool real = sizeof(T) == sizeof(double);
+  const long long tiles = cdiv(OP == TW_UPE ? std::max(1, b.max_c) : OP == TW_DNW ? b.max_n : b.max_r, TW_M);
+  const bool few = tiles * b.nrec * cdiv(nrhs, real ? TW_NC : TW_NC / 2) <= 76;
+  const bool g16 = few || nrhs <= 16 || tw_group(OP, b.max_n, b.max_r, b.max_c, real) == 16;
+  auto go = [&](auto sx) {
+    constexpr int SX = decltype(sx)::value;
+    return g16 ? launch_tw_gw<T, OP, CACHE, 16, SX>(b, sl, x, ldx, nrhs, err, polls, st)
+               : launch_tw_gw<T, OP, CACHE, 32, SX>(b, sl, x, ldx, nrhs, err, polls, st);
+  };
+  if constexpr (!real) return go(std::integral_constant<int, TW_SXZ>{});
+  else if (tw_stages(true, b.max_n) == TW_SX) return go(std::integral_constant<int, TW_SX>{});
+  else return go(std::integral_constant<int, TW_SX_LONG>{});
 }
 
 // The tensor-core sweeps for the colour classes that take them, the FP64 sweeps for the

@@ -2,8 +2,11 @@
 // colour class two products up, y = W_F^T [b_S; b_R] into b_R and b_C -= E b_R, and
 // two down, z = y_R - F y_C into y_R and [y_S; y_R] = [y_S; 0] + W_E y_R (see
 // sweep.cuh), each a launch of one CTA per box, 128 rows of the matrix and TW_NC real
-// columns.  Rows of the matrix and columns of the right-hand sides are scaled by
-// powers of two over stretches of K (tw_stretch) and cut into eight signed 7-bit
+// columns.  The products with W_F and W_E write what they read: of a box of more than 128
+// points the row tiles form a cluster and meet between the two (64 columns, FP64 sweeps
+// before, this after: Laplace 384^2, leaf 144 36.5 -> 6.5 ms, 512^2, leaf 256 112 -> 13.1;
+// Helmholtz 192^2, leaf 144 31.6 -> 9.1).  Rows of the matrix and columns of the right-hand sides are scaled by
+// powers of two over stretches of K (SX) and cut into eight signed 7-bit
 // digits; the slice products of equal weight u = p + q <= 7 are summed exactly in
 // FP32 in tensor memory over a stretch, gathered into one int64 per
 // output and added in FP64: the accuracy of an FP64 product.  A complex product is
@@ -24,14 +27,15 @@
 // one CTA per box (real) and the FP64 sweeps (complex): Laplace 512^2 23.3 -> 9.2 ms,
 // Helmholtz 256^2 30.3 -> 11.9 ms; 16 columns, against the FP64 sweeps: 4.6 -> 3.4 ms
 // (Laplace 256^2).
-// Stages of K that share scales and sums.  Complex sums restart more often: against the
-// records applied in quadruple precision (Helmholtz, 64^2, leaf 64) a panel's error is
-// then 9.8e-16, of one-column FP64 solves 1.00e-15; stretches of 128, 192 and 384 give
-// 1.06e-15, 1.08e-15 and 1.14e-15, in 11.0, 10.7 and 10.2 ms instead of 11.9 (256^2, 64
-// columns).  Laplace: 3.34e-16, FP64 3.36e-16.
-template <typename T> __host__ __device__ constexpr int tw_stretch() { return (sizeof(T) == sizeof(double) ? TW_KX : TW_KN) / TW_K; }
-// (tw_plan.h sizes the launches)
-static_assert(TW_M == 128 && TW_K == 32 && OZ_S == 8 && tw_stretch<double>() == 12 && tw_stretch<zd>() == 3, "");
+// Stages of K that share scales and sums (SX below; tw_stages).  Shorter stretches follow
+// the entries' range more closely and cost a gather each.  Errors of a panel against the
+// records applied in quadruple precision, and 64 columns' times:
+//   complex (Helmholtz, 64^2, leaf 64): 9.8e-16 in stretches of 48 entries, of one-column
+//     FP64 solves 1.00e-15; of 128, 192 and 384: 1.06e-15, 1.08e-15 and 1.14e-15, in 11.0,
+//     10.7 and 10.2 ms instead of 11.9 (256^2);
+//   real, n <= 128 (Laplace, 64^2, leaf 64): 3.36e-16 in stretches of 384, FP64 3.25e-16;
+//   real, n > 128: see TW_SX_LONG in launch_tw.
+static_assert(TW_M == 128 && TW_K == 32 && OZ_S == 8 && TW_SX == TW_KX / TW_K && TW_SXZ == TW_KN / TW_K, "");
 
 // rows and inner dimension of a product
 template <int OP, typename T> __host__ __device__ inline int tw_rows(const BoxRec<T>& R) {
@@ -52,9 +56,9 @@ constexpr bool tw_k_contiguous(int op) { return op == TW_UPW || op == TW_DNF; }
 // Exponents (biased, at least 1) of the largest of the entries K0 .. K of the CTA's rows
 // i0 .., for each stretch st of K (from the one of K0 on), into reb[st * TW_M + i], which
 // holds 1s.  (A barrier must follow.)
-template <int OP, typename T>
+template <int OP, int SX, typename T>
 __device__ void tw_row_exps(const BoxRec<T>& R, int i0, int rows, int K0, int K, int* reb) {
-  constexpr int KX = tw_stretch<T>() * (sizeof(T) == sizeof(double) ? TW_K : TW_K / 2);
+  constexpr int KX = SX * (sizeof(T) == sizeof(double) ? TW_K : TW_K / 2);
   size_t si, sl;
   const T* A = tw_mat<OP>(R, si, sl);
   const int tid = threadIdx.x;
@@ -119,27 +123,28 @@ __host__ __device__ inline size_t tw_tile_off(int t, int K) { return (size_t)t *
 inline size_t tw_cache_bytes(int rows, int K) {
   return (size_t)((rows + 7) & ~7) * ((K + TW_K - 1) / TW_K) * (OZ_S * TW_K * 2);
 }
-template <int OP>
+template <int OP, int SX>
 __global__ void __launch_bounds__(TW_NT) k_tw_cache(const BoxRec<double>* __restrict__ recs, const SliceRec* __restrict__ sl) {
-  __shared__ int reb[TW_MAXC / TW_KX + 1][TW_M];
+  constexpr int KX = SX * TW_K, NS = TW_MAXC / KX + 1;
+  __shared__ int reb[NS][TW_M];
   const BoxRec<double> R = recs[blockIdx.y];
   const SliceRec S = sl[blockIdx.y];
   const int M = tw_rows<OP>(R), K = tw_inner<OP>(R), i0 = blockIdx.x * TW_M, rows = min(TW_M, M - i0);
   if (rows <= 0) return;
-  for (int i = threadIdx.x; i < (TW_MAXC / TW_KX + 1) * TW_M; i += TW_NT) reb[0][i] = 1;
+  for (int i = threadIdx.x; i < NS * TW_M; i += TW_NT) reb[0][i] = 1;
   __syncthreads();
-  tw_row_exps<OP>(R, i0, rows, 0, K, reb[0]);
+  tw_row_exps<OP, SX>(R, i0, rows, 0, K, reb[0]);
   __syncthreads();
   const int rows8 = (rows + 7) & ~7;
   unsigned char* base = S.dig[OP] + tw_tile_off(blockIdx.x, K);
   for (int s = 0; s * TW_K < K; ++s)
-    tw_cut_a<OP>(R, i0, rows, K, s, reb[s / (TW_KX / TW_K)], base + (size_t)s * OZ_S * rows8 * 64, (size_t)rows8 * 64);
-  for (int st = 0; st * TW_KX < K; ++st)
+    tw_cut_a<OP>(R, i0, rows, K, s, reb[s / SX], base + (size_t)s * OZ_S * rows8 * 64, (size_t)rows8 * 64);
+  for (int st = 0; st * KX < K; ++st)
     for (int i = threadIdx.x; i < rows; i += TW_NT) S.eb[OP][(size_t)st * M + i0 + i] = reb[st][i];
 }
 
 // GW: columns of a group (32, or 16 for classes of few boxes: more and shorter CTAs)
-template <typename T, int OP, bool CACHE, int GW>
+template <typename T, int OP, bool CACHE, int GW, int SX>
 __global__ void __launch_bounds__(TW_NT, 1) k_tw(const BoxRec<T>* __restrict__ recs, const SliceRec* __restrict__ sl,
                                                  T* __restrict__ x, int64_t ldx, int nrhs, int srows, int nst, int nstr, int* err,
                                                  int polls) {
@@ -153,12 +158,13 @@ __global__ void __launch_bounds__(TW_NT, 1) k_tw(const BoxRec<T>* __restrict__ r
   __shared__ __align__(8) uint64_t mb_mma[4], mb_full[4];
   __shared__ uint32_t s_tmem;
   __shared__ int s_bad[2];
-  constexpr int SX = tw_stretch<T>();              // stages of a stretch of K
   const BoxRec<T> R = recs[blockIdx.z];
   const int M = tw_rows<OP>(R), Kall = tw_inner<OP>(R), k = R.k;
   // the down sweep's long inner dimension: a cluster of CTAs, each a range of stages
   const int spl = OP == TW_DNF ? (int)cooperative_groups::this_cluster().num_blocks() : 1;
   const int rank = OP == TW_DNF ? (int)cooperative_groups::this_cluster().block_rank() : 0;
+  // the row tiles of a product that writes what the others read meet before they write
+  const bool meet = (OP == TW_UPW || OP == TW_DNW) && gridDim.x > 1;
   const int tile0 = blockIdx.x / spl, i0 = tile0 * TW_M, rows = min(TW_M, M - i0);
   const int nsall = (Kall + KS - 1) / KS, s0 = nsall * rank / spl, ns = nsall * (rank + 1) / spl - s0;
   const int K0 = s0 * KS, K = min(Kall, (s0 + ns) * KS);   // this CTA's entries of K
@@ -167,6 +173,7 @@ __global__ void __launch_bounds__(TW_NT, 1) k_tw(const BoxRec<T>* __restrict__ r
   // before it: the next launch waits for this one alone)
   if (rows <= 0) {
     pdl_wait();
+    if (meet) cooperative_groups::this_cluster().sync();
     return;
   }
   const int q0 = blockIdx.y * NC, nq = min(NC, nrhs - q0);
@@ -189,7 +196,7 @@ __global__ void __launch_bounds__(TW_NT, 1) k_tw(const BoxRec<T>* __restrict__ r
   } else {
     for (int i = tid; i < nstr * TW_M; i += TW_NT) reb[i] = 1;
     __syncthreads();
-    tw_row_exps<OP>(R, i0, rows, K0, K, reb);
+    tw_row_exps<OP, SX>(R, i0, rows, K0, K, reb);
   }
   for (int i = tid; i < nstr * NC; i += TW_NT) ceb[i] = 1;
   if (tid < 4) {
@@ -297,7 +304,7 @@ __global__ void __launch_bounds__(TW_NT, 1) k_tw(const BoxRec<T>* __restrict__ r
       wait_mma(s - 1, s);
       __syncwarp();
       tc_fence_after();
-      gather(stretch(s - 1), std::false_type{});
+      gather(stretch(s - 1), std::integral_constant<bool, !cplx && SX <= TW_KN / TW_K>{});
       tc_fence_before();
     }
     if (!CACHE) tw_cut_a<OP>(R, i0, rows, K, s0 + s, reb + stretch(s) * TW_M, As, srows * 64);
@@ -379,7 +386,7 @@ __global__ void __launch_bounds__(TW_NT, 1) k_tw(const BoxRec<T>* __restrict__ r
     if (CACHE)
       for (int q = max(0, fetched - nst); q < fetched; ++q) mbar_wait(&mb_full[q % nst], (q / nst) & 1, TW_DRAIN);
   }
-  if (spl > 1) cooperative_groups::this_cluster().sync();
+  if (spl > 1 || meet) cooperative_groups::this_cluster().sync();
   else __syncthreads();
   if (ok) {
     // (of a cluster: each CTA the sums of a share of the rows, parts added in order)

@@ -30,3 +30,33 @@ def test_classes_without_neighbours_left(P, cplx, side, leaf, nrhs):
     x = [P.rss_solve(f, v.clone().T) for v in b]
     for v, w in zip(b, x):
         assert float(torch.linalg.vector_norm(w.T - v / 2) / torch.linalg.vector_norm(v)) < 1e-15
+
+
+@pytest.mark.parametrize("kind,side,leaf,eps,nrhs", [
+    ("laplace", 48, 144, 1e-6, 32), ("laplace", 96, 144, 1e-9, 65), ("laplace", 64, 256, 1e-6, 33),
+    ("laplace", 128, 256, 1e-10, 40), ("laplace", 80, 100, 1e-11, 64), ("laplace", 192, 144, 1e-6, 17),
+    ("helmholtz", 48, 144, 1e-6, 16), ("helmholtz", 96, 144, 1e-9, 33), ("helmholtz", 64, 256, 1e-6, 17),
+    ("helmholtz", 80, 100, 1e-10, 40)])
+def test_boxes_of_more_than_one_row_tile(P, kind, side, leaf, eps, nrhs):
+    """Boxes of 129 to about 400 points: the row tiles of one box read what the others
+    write.  Against one-column solves, as in the panels of smaller boxes: at most four
+    products of 6000 2^-53 for each class, below 1e-12 of the solution; repeated solves
+    and any split into panels give the same bits."""
+    cplx = kind == "helmholtz"
+    f = P.rss_factor(P.rss_build_tree(W.grid_points(side), leaf), kind=P.HELMHOLTZ if cplx else P.LAPLACE, eps=eps,
+                     h=1.0 / side, kappa=25.0 if cplx else 0.0)
+    assert max(L["k_max"] for L in P.rss_info(f)["levels"]) * 4 > 128 or leaf > 128
+    b = torch.from_numpy(np.ascontiguousarray(W.gaussian_rhs(side * side, nrhs, cplx, 5).T)).cuda()
+    fly = b.clone()
+    if b.numel() * b.element_size() <= 8 << 20:
+        P.rss_solve_noalloc(f, fly.T)   # real: no digits kept yet, cut on the fly
+    else:
+        fly = None
+    x = P.rss_solve(f, b.clone().T).T
+    for _ in range(4):
+        assert torch.equal(x, P.rss_solve(f, b.clone().T).T)
+    for j in (0, 7, nrhs - 1):
+        one = P.rss_solve(f, b[j].clone())
+        assert float(torch.linalg.vector_norm(x[j] - one) / torch.linalg.vector_norm(one)) <= 1e-12, j
+    if fly is not None:
+        assert float(torch.linalg.vector_norm(fly - x) / torch.linalg.vector_norm(x)) <= 1e-12
