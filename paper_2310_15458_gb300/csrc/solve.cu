@@ -414,10 +414,11 @@ rss_status ensure_slices(rss_factorization* f, cudaStream_t st) {
     const unsigned tr = cdiv(b.max_r, TW_M), tc = std::max(1u, cdiv(b.max_c, TW_M)), tn = cdiv(b.max_n, TW_M);
     auto cut = [&](auto sx) {
       constexpr int SX = decltype(sx)::value;
-      k_tw_cache<TW_UPW, SX><<<dim3(tr, b.nrec), TW_NT, 0, st>>>(dr, recs[bi]);
-      k_tw_cache<TW_UPE, SX><<<dim3(tc, b.nrec), TW_NT, 0, st>>>(dr, recs[bi]);
-      k_tw_cache<TW_DNF, SX><<<dim3(tr, b.nrec), TW_NT, 0, st>>>(dr, recs[bi]);
-      k_tw_cache<TW_DNW, SX><<<dim3(tn, b.nrec), TW_NT, 0, st>>>(dr, recs[bi]);
+      auto z = [](int k) { return std::max(1u, cdiv(k, SX * TW_K)); };
+      k_tw_cache<TW_UPW, SX><<<dim3(tr, b.nrec, z(b.max_n)), TW_NT, 0, st>>>(dr, recs[bi]);
+      k_tw_cache<TW_UPE, SX><<<dim3(tc, b.nrec, z(b.max_r)), TW_NT, 0, st>>>(dr, recs[bi]);
+      k_tw_cache<TW_DNF, SX><<<dim3(tr, b.nrec, z(b.max_c)), TW_NT, 0, st>>>(dr, recs[bi]);
+      k_tw_cache<TW_DNW, SX><<<dim3(tn, b.nrec, z(b.max_r)), TW_NT, 0, st>>>(dr, recs[bi]);
     };
     if (tw_stages(true, b.max_n) == TW_SX) cut(std::integral_constant<int, TW_SX>{});
     else cut(std::integral_constant<int, TW_SX_LONG>{});

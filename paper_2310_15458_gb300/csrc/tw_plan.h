@@ -4,7 +4,7 @@
 #include <algorithm>
 
 constexpr int TW_MAXN = 1024;                 // rows of the products that write what they read: a cluster of 8 tiles
-constexpr int TW_MAXC = 6000;                 // entries of K whose exponents k_tw_cache holds
+constexpr int TW_MAXC = 6000;                 // (the plan's own limit lies below)
 constexpr int TW_SMEM = 222 * 1024;
 
 // NST stages of the rows' digits (rows8 rows of 8 slices x 32 entries) and of 2 gw real
