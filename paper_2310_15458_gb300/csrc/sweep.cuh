@@ -46,15 +46,35 @@ template <int W, typename T> __device__ __forceinline__ T part_sum(T v) {
   return v;
 }
 
+// The same for the sums of RC columns (RC a multiple of 4, four lanes, p = lane % 4): lane
+// p ends with the sums of columns own_column(p) .. + RC / 4 - 1 in acc[0 ..].  6 additions
+// for 8 columns instead of 16, which counts where a lane has about ten products a column:
+// 15 columns, Laplace 896^2, leaf 49 30.0 -> 26.5 ms, 1024^2 36.8 -> 32.9 ms.
+template <int RC> __device__ __forceinline__ int own_column(int p) { return (p & 1) * (RC / 2) + (p >> 1) * (RC / 4); }
+template <int RC, typename T> __device__ __forceinline__ void part_scatter(T (&acc)[RC], int p) {
+#pragma unroll
+  for (int q = 0; q < RC / 2; ++q) {
+    const T give = (p & 1) ? acc[q] : acc[q + RC / 2];
+    const T keep = (p & 1) ? acc[q + RC / 2] : acc[q];
+    acc[q] = keep + shfl_xor(give, 1);
+  }
+#pragma unroll
+  for (int q = 0; q < RC / 4; ++q) {
+    const T give = (p & 2) ? acc[q] : acc[q + RC / 4];
+    const T keep = (p & 2) ? acc[q + RC / 4] : acc[q];
+    acc[q] = keep + shfl_xor(give, 2);
+  }
+}
+
 // (entry (g, q) of the right-hand sides at x[g * ldx + q]: the columns of a point
 // side by side)
-// x_g(i) = [keep(i)] x_g(i) + sgn sum_j M(i, j) w_j for the rows i < rows of M (ld
+// x_g(i) = [keep(i)] x_g(i) +- sum_j M(i, j) w_j (+: add) for the rows i < rows of M (ld
 // scalars between columns) and the columns j >= lo(i) (M is zero before), w in shared
 // memory (RC scalars per j): four lanes per row, or, for one column when the rows fill
 // half the CTA, one thread per row (no shuffles); the same sums either way.
 template <typename T, int RC, typename LO, typename GI, typename KP>
 __device__ __forceinline__ void row_products(int rows, int r, int nq, int tid, int nt, const T* w, const T* M, size_t ld,
-                                             LO lo, GI gidx, KP keep, double sgn, T* xq, int64_t ldx) {
+                                             LO lo, GI gidx, KP keep, bool add, T* xq, int64_t ldx) {
   const int L4 = (r + SW_PE - 1) / SW_PE;
   if constexpr (RC == 1) {
     if (rows * 2 >= nt) {
@@ -72,15 +92,18 @@ __device__ __forceinline__ void row_products(int rows, int r, int nq, int tid, i
             const int j = p * L4 + t;
             if (j >= a && j < r) acc[p] = mad(acc[p], m[(size_t)j * ld], w[j]);
           }
-        const T s = scl(sgn, (acc[0] + acc[1]) + (acc[2] + acc[3]));
-        *g = keep(i) ? ld_l2(g) + s : s;
+        const T s = (acc[0] + acc[1]) + (acc[2] + acc[3]);
+        *g = !keep(i) ? s : add ? ld_l2(g) + s : ld_l2(g) - s;
       }
       return;
     }
   }
   for (int e = tid; e < ((rows * SW_PE + 31) & ~31); e += nt) {
     const int p = e % SW_PE, i = e / SW_PE;
-    T acc[RC], old[(RC + SW_PE - 1) / SW_PE];
+    constexpr int OW = (RC + SW_PE - 1) / SW_PE;   // columns that a lane stores: c0 ..
+    const int c0 = RC == 1 ? 0 : own_column<RC>(p);
+    const bool own = RC > 1 || p == 0;
+    T acc[RC], old[OW];
 #pragma unroll
     for (int q = 0; q < RC; ++q) acc[q] = zero<T>();
     int64_t gi = 0;
@@ -88,8 +111,8 @@ __device__ __forceinline__ void row_products(int rows, int r, int nq, int tid, i
       gi = gidx(i);
       const bool kp = keep(i);
 #pragma unroll
-      for (int q = 0; q < RC; q += SW_PE)
-        if (p + q < nq) old[q / SW_PE] = kp ? ld_l2(xq + gi * ldx + p + q) : zero<T>();
+      for (int q = 0; q < OW; ++q)
+        if (own && c0 + q < nq) old[q] = kp ? ld_l2(xq + gi * ldx + c0 + q) : zero<T>();
       const int j1 = min(r, (p + 1) * L4);
       const T* m = M + i;
 #pragma unroll 4
@@ -99,12 +122,12 @@ __device__ __forceinline__ void row_products(int rows, int r, int nq, int tid, i
         for (int q = 0; q < RC; ++q) acc[q] = mad(acc[q], mv, w[j * RC + q]);
       }
     }
-#pragma unroll
-    for (int q = 0; q < RC; ++q) acc[q] = part_sum<SW_PE>(acc[q]);
+    if constexpr (RC == 1) acc[0] = part_sum<SW_PE>(acc[0]);
+    else part_scatter<RC>(acc, p);
     if (i < rows) {
 #pragma unroll
-      for (int q = 0; q < RC; ++q)
-        if (q % SW_PE == p && q < nq) xq[gi * ldx + q] = old[q / SW_PE] + scl(sgn, acc[q]);
+      for (int q = 0; q < OW; ++q)
+        if (own && c0 + q < nq) xq[gi * ldx + c0 + q] = add ? old[q] + acc[q] : old[q] - acc[q];
     }
   }
 }
@@ -171,14 +194,19 @@ __device__ void up_box(const BoxRec<T>& R, T* xq, int64_t ldx, int nq, T* sm, si
         for (int q = 0; q < RC; ++q) acc[q] = mad(acc[q], wv, v[l * RC + q]);
       }
     }
+    if constexpr (RC == 1) {
+      acc[0] = part_sum<SW_PF>(acc[0]);
+      if (j < j1)
+        for (int t = p; t < Q; t += SW_PF) *cl.peer(y + j, t) = acc[0];
+    } else {
+      part_scatter<RC>(acc, p);
+      if (j < j1)
+        for (int t = 0; t < Q; ++t) {
+          T* d = cl.peer(y + (size_t)j * RC + own_column<RC>(p), t);
 #pragma unroll
-    for (int q = 0; q < RC; ++q) acc[q] = part_sum<SW_PF>(acc[q]);
-    if (j < j1)
-      for (int t = p; t < Q; t += SW_PF) {
-        T* d = cl.peer(y + (size_t)j * RC, t);
-#pragma unroll
-        for (int q = 0; q < RC; ++q) d[q] = acc[q];
-      }
+          for (int q = 0; q < RC / 4; ++q) d[q] = acc[q];
+        }
+    }
   }
   cp_async_wait_group<0>();
   __syncthreads();
@@ -189,7 +217,7 @@ __device__ void up_box(const BoxRec<T>& R, T* xq, int64_t ldx, int nq, T* sm, si
     if (q < nq) xq[R.idxR[j] * ldx + q] = y[j * RC + q];
   }
   row_products<T, RC>(rows, r, nq, tid, nt, y, ste ? Es : R.E + i0, ste ? lde : c, [](int) { return 0; },
-                      [&](int i) { return (int64_t)R.idxC[i0 + i]; }, [](int) { return true; }, -1.0, xq, ldx);
+                      [&](int i) { return (int64_t)R.idxC[i0 + i]; }, [](int) { return true; }, false, xq, ldx);
 }
 
 template <typename T, int RC, typename CL>
@@ -244,12 +272,15 @@ __device__ void down_box(const BoxRec<T>& R, T* xq, int64_t ldx, int nq, T* sm, 
         for (int q = 0; q < RC; ++q) acc[q] = mad(acc[q], fv, yc[i * RC + q]);
       }
     }
+    if constexpr (RC == 1) {
+      acc[0] = part_sum<SW_PC>(acc[0]);
+      if (s < sl && p == 0) gp[(size_t)s * r + j] = acc[0];
+    } else {
+      part_scatter<RC>(acc, p);
+      if (s < sl) {
 #pragma unroll
-    for (int q = 0; q < RC; ++q) acc[q] = part_sum<SW_PC>(acc[q]);
-    if (s < sl) {
-#pragma unroll
-      for (int q = 0; q < RC; ++q)
-        if (q % SW_PC == p) gp[((size_t)s * r + j) * RC + q] = acc[q];
+        for (int q = 0; q < RC / 4; ++q) gp[((size_t)s * r + j) * RC + own_column<RC>(p) + q] = acc[q];
+      }
     }
   }
   cp_async_wait_group<0>();
@@ -274,7 +305,7 @@ __device__ void down_box(const BoxRec<T>& R, T* xq, int64_t ldx, int nq, T* sm, 
   row_products<T, RC>(lw, r, nq, tid, nt, z, stw ? Ws : R.We + l0, stw ? ldw : n,
                       [&](int l) { return max(0, l0 + l - k); },   // rows of U^{-1} are zero left of the diagonal
                       [&](int l) { return (int64_t)(l0 + l < k ? R.idxC[l0 + l] : R.idxR[l0 + l - k]); },
-                      [&](int l) { return l0 + l < k; }, 1.0, xq, ldx);
+                      [&](int l) { return l0 + l < k; }, true, xq, ldx);
   cl.wait();   // no CTA ends while its sums are read
 }
 
