@@ -274,21 +274,35 @@ template <typename T, int RC> int sweep_persistent_start(const rss_factorization
 
 // One colour class of the FP64 sweeps: Q CTAs per box, at most as many as the class
 // has slices.  Fewer boxes (times column chunks) than SMs: a cluster per box, at most
-// two CTAs to an SM, every matrix staged.  More: 128-thread CTAs that stage nothing,
-// up to twelve to an SM, since the memory latency is then hidden by their number (one
-// column at 1024^2: 4.0 ms so, 4.9 with the same classes staged; at 64^2, where every
-// class is small, 0.26 ms staged and 0.40 not).  The columns are taken in smaller
-// chunks where a box's vectors would not fit (the sums do not depend on it).
+// two CTAs to an SM, its matrices staged.  More: CTAs that stage nothing, many to an SM,
+// since the memory latency is then hidden by their number (one column at 1024^2: 4.0 ms so,
+// 4.9 with the same classes staged; at 64^2, where every class is small, 0.26 ms staged and
+// 0.40 not).  Boxes too large for either matrix to be staged count as many: alone on their
+// SMs for nothing, such CTAs took 5.5 instead of 3.0 ms (one column, 512^2, leaf 256).
+// Unstaged CTAs of 256 threads, so that a box is shared by fewer, but of 128 where boxes
+// hold at most 40 points (128 threads everywhere, then this, ms: 15 columns, 512^2, leaf 256
+// 24.8, 23.1; 1024^2 32.9, 31.7; one column, 1024^2 4.0, 3.7; 256 threads everywhere, 15
+// columns, 512^2, leaf 4: 8.2 instead of 7.9).  The columns are taken in smaller chunks
+// where a box's vectors would not fit (the sums do not depend on any of this).
 template <typename T, int RC, bool UP>
 rss_status sweep_class(const Batch& b, T* x, int64_t ldx, int nrhs, cudaStream_t st) {
+  constexpr size_t MOST = 220 * 1024 / sizeof(T);   // scalars
   const long long nz = cdiv(nrhs, RC);
   const int qc = sweep_slices(b.nrec);
+  const bool large = b.max_n > 40;
+  bool staged = b.nrec * nz <= 152;
   int Q = 1;
-  const bool fills = b.nrec * nz > 152;
-  while (Q < qc && b.nrec * nz * Q * 2 <= (fills ? 12 : 2) * 152) Q *= 2;
-  const SweepSm s = UP ? sweep_sm_up<T, RC>(b.max_n, b.max_r, b.max_c, Q)
-                       : sweep_sm_down<T, RC>(b.max_n, b.max_r, b.max_c, Q, qc);
-  if (s.need * sizeof(T) > 220 * 1024) {
+  auto split = [&](int per_sm) {
+    while (Q < qc && b.nrec * nz * Q * 2 <= per_sm * 152) Q *= 2;
+    return UP ? sweep_sm_up<T, RC>(b.max_n, b.max_r, b.max_c, Q) : sweep_sm_down<T, RC>(b.max_n, b.max_r, b.max_c, Q, qc);
+  };
+  SweepSm s = {};
+  if (staged) {
+    s = split(2);
+    staged = s.one <= MOST;
+  }
+  if (!staged) s = split(!large ? 12 : RC == 1 ? 4 : 8);
+  if (s.need > MOST) {
     if constexpr (RC > 1) {
       return sweep_class<T, RC == 8 ? 4 : 1, UP>(b, x, ldx, nrhs, st);
     } else {
@@ -296,9 +310,9 @@ rss_status sweep_class(const Batch& b, T* x, int64_t ldx, int nrhs, cudaStream_t
       return RSS_EINVAL;
     }
   }
-  const size_t smem = fills ? s.need * sizeof(T) : std::min<size_t>(s.full * sizeof(T), 220 * 1024);
+  const size_t smem = (staged ? std::min(s.full, MOST) : s.need) * sizeof(T);
   RSS_CUDA(allow_smem(k_sweep_cl<T, RC, UP>));
-  RSS_CUDA(launch_pdl(k_sweep_cl<T, RC, UP>, dim3(b.nrec * Q, (unsigned)nz), fills ? 128 : SW_NT, smem, st, Q,
+  RSS_CUDA(launch_pdl(k_sweep_cl<T, RC, UP>, dim3(b.nrec * Q, (unsigned)nz), staged || large ? SW_NT : 128, smem, st, Q,
                       static_cast<const BoxRec<T>*>(b.d_recs), x, ldx, nrhs, Q, qc, (int)(smem / sizeof(T))));
   return RSS_OK;
 }

@@ -24,19 +24,21 @@ constexpr int SW_PF = 4, SW_PE = 4, SW_PC = 4;
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
-// scalars of shared memory: always, and with both matrices staged
+// scalars of shared memory: always, with the smaller and with both matrices staged
 struct SweepSm {
-  size_t need, full;
+  size_t need, one, full;
 };
 template <typename T, int RC> inline SweepSm sweep_sm_up(int n, int r, int c, int Q) {
   const size_t rows = (c + Q - 1) / Q, js = (r + Q - 1) / Q;
   const size_t need = ((size_t)n + r) * RC;
-  return SweepSm{need, need + js * (n | 1) + (rows | 1) * r};
+  const size_t w = js * (n | 1), e = (rows | 1) * r;
+  return SweepSm{need, need + std::min(w, e), need + w + e};
 }
 template <typename T, int RC> inline SweepSm sweep_sm_down(int n, int r, int c, int Q, int qc) {
   const size_t rows = (c + Q - 1) / Q, ls = (n + Q - 1) / Q, sl = qc / Q;
   const size_t need = (rows + r + sl * r) * RC;
-  return SweepSm{need, need + (rows | 1) * r + (ls | 1) * r};
+  const size_t f = (rows | 1) * r, w = (ls | 1) * r;
+  return SweepSm{need, need + std::min(f, w), need + f + w};
 }
 
 // W lanes that hold the parts of one sum: their tree sum, in every lane
