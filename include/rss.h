@@ -198,9 +198,11 @@ rss_status rss_solve_noalloc(const rss_factorization* f, void* b, int64_t nrhs, 
  *    coarse levels, where per-class launches are bound by latency).
  * The persistent part has a knob, "ctas_per_sm" (0: as many as fit); "spread" is
  * read and written for tables from earlier builds and has no effect.  rss_tune_solve
- * times the solve of nrhs zero right-hand sides under eleven candidates (the
- * per-class form, four persistent and six hybrid schedules; median of three
- * after one untimed run, CUDA events on stream), keeps the fastest for the
+ * times the solve of nrhs zero right-hand sides under six launch forms (per
+ * class, persistent with two settings of "ctas_per_sm", hybrid with three of
+ * "tail_boxes"; median of three after one untimed run, CUDA events on stream),
+ * lists them as eleven candidates (all but the first with two values of "spread",
+ * which share one time), keeps the fastest for the
  * later solves of f, and writes the table to json (may be NULL) as {"nrhs": ..,
  * "path": .., "candidates": [..], "launch": .., "spread": .., "ctas_per_sm":
  * .., "tail_boxes": .., "ms": ..}; passing that text back as
