@@ -2723,7 +2723,6 @@ rss_status factor_impl(const rss_tree* tree, const rss_params* prm, cudaStream_t
         R.Tm = static_cast<T*>(f->arena.get(sizeof(T) * (size_t)k * r));
         R.LU = static_cast<T*>(f->arena.get(sizeof(T) * (size_t)r * r));
         R.piv = static_cast<int*>(f->arena.get(sizeof(int) * r));
-        R.pos = static_cast<int*>(f->arena.get(sizeof(int) * r));
         R.We = static_cast<T*>(f->arena.get(sizeof(T) * (size_t)n * r));
         R.Wf = static_cast<T*>(f->arena.get(sizeof(T) * (size_t)n * r));
         R.E = static_cast<T*>(f->arena.get(sizeof(T) * (size_t)c * r));
@@ -2731,7 +2730,7 @@ rss_status factor_impl(const rss_tree* tree, const rss_params* prm, cudaStream_t
         R.idxR = static_cast<int*>(f->arena.get(sizeof(int) * r));
         R.idxC = static_cast<int*>(f->arena.get(sizeof(int) * c));
         R.cmap = static_cast<int*>(f->arena.get(sizeof(int) * c));
-        if (!R.Tm || !R.LU || !R.piv || !R.pos || !R.We || !R.Wf || !R.E || !R.Ft || !R.idxR || !R.idxC ||
+        if (!R.Tm || !R.LU || !R.piv || !R.We || !R.Wf || !R.E || !R.Ft || !R.idxR || !R.idxC ||
             !R.cmap) {
           rss_set_error("rss_factor: device arena allocation failed");
           return RSS_ENOMEM;
@@ -2852,9 +2851,9 @@ rss_status factor_impl(const rss_tree* tree, const rss_params* prm, cudaStream_t
           ef_later && std::max(elim_x_bytes<T>(8, max_k, max_n), elim_inv_bytes<T>(16, max_r)) <= 200 * 1024;
       {
         auto rr = [](const BoxRec<T>& R) { return ((size_t)R.r * R.r * sizeof(T) + 255) & ~size_t(255); };
+        auto rp = [](const BoxRec<T>& R) { return ((size_t)R.r * sizeof(int) + 255) & ~size_t(255); };
         size_t bytes = 0;
-        for (const BoxRec<T>& R : recs)
-          if (!elim_cols || !R.ozp) bytes += 3 * rr(R);
+        for (const BoxRec<T>& R : recs) bytes += rp(R) + (!elim_cols || !R.ozp ? 3 * rr(R) : 0);
         if (!gb_inv.ensure(bytes)) {
           rss_set_error("rss_factor: device workspace allocation failed");
           return RSS_ENOMEM;
@@ -2862,6 +2861,8 @@ rss_status factor_impl(const rss_tree* tree, const rss_params* prm, cudaStream_t
         f->peak_transient = std::max(f->peak_transient, transient + bytes);
         char* p = static_cast<char*>(gb_inv.p);
         for (BoxRec<T>& R : recs) {
+          R.pos = reinterpret_cast<int*>(p);
+          p += rp(R);
           if (elim_cols && R.ozp) continue;
           R.Ui = reinterpret_cast<T*>(p);
           R.Li = reinterpret_cast<T*>(p + rr(R));
@@ -3000,7 +3001,7 @@ rss_status factor_impl(const rss_tree* tree, const rss_params* prm, cudaStream_t
       }
       RSS_LAUNCHED();
       evs.back().second->stop(st);
-      for (BoxRec<T>& R : recs) R.Esl = R.Fsl = nullptr, R.Eexp = R.Fexp = nullptr, R.Ui = R.Li = R.LiP = nullptr;
+      for (BoxRec<T>& R : recs) R.Esl = R.Fsl = nullptr, R.Eexp = R.Fexp = nullptr, R.Ui = R.Li = R.LiP = nullptr, R.pos = nullptr;
       f->launches += 2;
       f->n_elim += 1;
       f->n_schur += 1;
