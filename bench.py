@@ -35,20 +35,14 @@ import workloads as W  # noqa: E402
 
 WORKLOAD = "laplace_1024x1024_eps1e-6"
 METRIC = "RS-S factor s and solve RHS/s at N=1M, rel.res<=1e-5; serve p50/p99 latency"
-# FP64 roof of the FP64-bound phases: the nominal FP64 rate of a GB300, 1.25
-# TFLOP/s (152 SMs x 2.07 GHz x 2 FP64 FMA per clock and SM x 2 flop = 1.26).  The
-# bench also measures it with the library's DFMA probe (rss_probe_fp64) and
-# reports both; FP64 tensor-core MMAs (mma.sync f64) are no faster than DFMA here.
+# Rates that the phases are held against.  An FP64-accurate product on the tensor cores is 36
+# bf16 products of 7-bit digits, so the measured bf16 rate (8192^3 cuBLAS GEMM, 1894
+# TFLOP/s) allows 52.6 TFLOP/s of them; the small factorizations of the boxes run on the
+# FP64 pipe, nominally 1.25 TFLOP/s (152 SMs x 2.07 GHz x 2 FMA per clock and SM x 2 flop =
+# 1.26), which the library's DFMA probe (rss_probe_fp64) measures.  FP64 tensor-core MMAs
+# (mma.sync f64) are no faster than DFMA here.
+DIGIT_PEAK_TFLOPS = 1893.8 / 36
 FP64_PEAK_TFLOPS = 1.25
-# DRAM bytes (read + write) of the dominant phase's kernels per factorization of
-# the 1024 x 1024 Laplace workload, from an ncu capture of the same kernels on a
-# smaller grid scaled by the boxes processed (source in the dict); None when the
-# kernels have changed since the capture.
-TRAFFIC = {"id": {"bytes_per_factor": 31.22e9 * (78.52 / 19.18),
-                  "source": "ncu dram__bytes_read.sum + dram__bytes_write.sum over every k_id and k_id_cl "
-                            "launch of one 512 x 512 Laplace factorization (31.2 GB), scaled to 1024 x 1024 "
-                            "by the ratio of the phase's algorithmic flops (78.5 / 19.2 GFLOP), then divided "
-                            "by the launches of one factorization"}}
 CPU_SAMPLE_SIDES = (128, 256)   # oracle samples: the same workload on these grids
 
 
@@ -656,21 +650,21 @@ def native_arm(args, w):
     launches = info["phase_launches"][dom]
     flops = info["flops"][dom]
     achieved = flops / (gms[dom] * 1e-3) / 1e12
-    kern = {"id": "k_id", "elim": "k_elim", "schur": "k_schur"}[dom]
-    tr = TRAFFIC.get(dom) if args.workload == WORKLOAD else None
-    traffic = tr["bytes_per_factor"] / max(launches, 1) if tr else None
+    kern = {"id": "k_idg_split, k_idg_gram, k_idg_chol, k_idg_tsolve",
+            "elim": "k_elim_x, k_elim_lu2, k_elim_inv, k_ep_cut_w, k_ep", "schur": "k_schur_*"}[dom]
     if args.no_probe:
         probe_tflops = probe_ms = dmma_tflops = None
     else:
         probe_tflops, probe_ms = P.rss_probe_fp64(stream=stream)
         dmma_tflops, dmma_ms = P.rss_probe_dmma(stream=stream)
     # kernels of one 1-RHS solve: the user-order permutations, the top block's gather and
-    # product, and per colour class k_up_r, k_up_c and k_down (per-class form) or the two
-    # persistent sweeps (persistent form)
-    if info.get("solve_launch") == "persistent":
+    # product, and the upward and the downward sweep, of each colour class (per-class form)
+    # or of all of them (persistent form; of the hybrid one only these are counted, not the
+    # launches of its finer classes)
+    if info.get("solve_launch") in ("persistent", "hybrid"):
         solve_launches = 2 + 2 + 2
     else:
-        solve_launches = 2 + 2 + 3 * info["batches"]
+        solve_launches = 2 + 2 + 2 * info["batches"]
     line = {
         "metric": METRIC, "value": ms / 1e3, "unit": "s", "n_gpus": world, "steps": args.steps,
         "warmup": args.warmup, "ms_per_step": ms, "higher_is_better": False, "scaling": "weak",
@@ -699,16 +693,18 @@ def native_arm(args, w):
         "e2e": {"value": e2e_s, "unit": "s", "h2d_bytes_per_step": pts_h.nbytes + bh.nbytes,
                 "d2h_bytes_per_step": bh.nbytes},
         "gpu_launches": args.steps * (info["launches"] + solve_launches),
-        "roofline": {"kernel": kern, "bound": "alu", "achieved": achieved, "peak": FP64_PEAK_TFLOPS,
-                     "unit": "TFLOP/s", "frac": achieved / FP64_PEAK_TFLOPS, "traffic": traffic,
+        # the dominant phase's FP64-equivalent rate against the digit products' roof; the part
+        # of it that runs on the FP64 pipe (LU and inverses of the boxes) has the lower roof
+        "roofline": {"kernel": kern, "bound": "tensor", "achieved": achieved, "peak": DIGIT_PEAK_TFLOPS,
+                     "unit": "TFLOP/s", "frac": achieved / DIGIT_PEAK_TFLOPS, "traffic": None,
                      "launches": launches, "avg_launch_ms": gms[dom] / max(launches, 1),
-                     "peak_source": "nominal FP64 rate (152 SMs x 2.07 GHz x 2 FMA/clk x 2); no FP64 "
-                                    "figure in MEASURED_PEAKS.json",
-                     "peak_probe": probe_tflops, "frac_of_probe": achieved / probe_tflops if probe_tflops else None,
+                     "peak_source": "36 bf16 digit products per FP64-accurate product, measured bf16 rate "
+                                    "1894 TFLOP/s",
+                     "fp64_pipe_peak": FP64_PEAK_TFLOPS, "fp64_pipe_probe": probe_tflops,
                      "probe": ("rss_probe_fp64: independent DFMA chains, 8 CTAs x 256 threads per SM, "
                                "best of 5 launches of %.1f ms" % probe_ms) if probe_ms else None,
                      "fp64_mma_probe": dmma_tflops,
-                     "traffic_source": tr["source"] if tr else "none for the kernels as built"},
+                     "traffic_source": "none for the kernels as built"},
     }
     if not args.no_serve:
         line["serve"] = serve_run(P, torch, args)
