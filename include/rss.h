@@ -221,7 +221,8 @@ rss_status rss_tune_solve(rss_factorization* f, int64_t nrhs, void* stream, char
  * with one rss_solve; requests arriving meanwhile join the next panel, and
  * panels of different factorizations run concurrently on their own streams.
  * A panel takes the tensor-core sweeps when all of its requests would by
- * themselves (16 or more columns), and with a real factor from 32 columns on; the
+ * themselves (16 or more columns), and from 32 columns on (with a complex factor in
+ * the colour classes of at least 152 boxes times groups of 32 columns); the
  * others take the FP64 sweeps, where every column goes through the same
  * operations whatever it is batched with, so a result equals the one rss_solve
  * gives for the request alone (between the two kinds of sweeps: to rounding).  This is

@@ -169,12 +169,13 @@ struct rss_factorization {
 
 template <typename T> rss_status factor_impl(const rss_tree* tree, const rss_params* p,
                                              cudaStream_t st, rss_factorization* f);
+// Which sweeps a solve takes: by its number of columns; FP64 ones; or, of a complex panel
+// packed from smaller requests, the products in its large classes alone
+enum class Sweeps { by_columns, fp64, large_classes };
 template <typename T> rss_status solve_impl(const rss_factorization* f, T* b_dev, int64_t nrhs,
-                                            int64_t ldb, cudaStream_t st, bool fp64 = false);
-// whether a panel of `cols` columns, packed from requests of at least `smallest`
-// columns, takes the FP64 sweeps whatever its width, so that each request's result is
-// the one of its own solve
-bool panel_in_fp64(const rss_factorization* f, int64_t cols, int64_t smallest);
+                                            int64_t ldb, cudaStream_t st, Sweeps how = Sweeps::by_columns);
+// the sweeps of a panel of `cols` columns, packed from requests of at least `smallest`
+Sweeps panel_sweeps(const rss_factorization* f, int64_t cols, int64_t smallest);
 // device bytes one solve of nrhs columns allocates (working copy plus sweep
 // workspace), beside the caller's b
 size_t solve_device_bytes(const rss_factorization* f, int64_t nrhs);

@@ -147,10 +147,10 @@ bool launch_panel(rss_server* S, Slot& s) {
   }
   cudaError_t e = cudaMemcpyAsync(s.d_panel, s.h_panel, bytes, cudaMemcpyHostToDevice, s.stream);
   rss_status st = RSS_OK;
-  const bool fp64 = panel_in_fp64(s.f, cols, smallest);
+  const Sweeps how = panel_sweeps(s.f, cols, smallest);
   if (e == cudaSuccess)
-    st = s.f->is_complex ? solve_impl<zd>(s.f, static_cast<zd*>(s.d_panel), cols, n, s.stream, fp64)
-                         : solve_impl<double>(s.f, static_cast<double*>(s.d_panel), cols, n, s.stream, fp64);
+    st = s.f->is_complex ? solve_impl<zd>(s.f, static_cast<zd*>(s.d_panel), cols, n, s.stream, how)
+                         : solve_impl<double>(s.f, static_cast<double*>(s.d_panel), cols, n, s.stream, how);
   if (e == cudaSuccess && st == RSS_OK)
     e = cudaMemcpyAsync(s.h_panel, s.d_panel, bytes, cudaMemcpyDeviceToHost, s.stream);
   if (e == cudaSuccess && st == RSS_OK) e = cudaEventRecord(s.done, s.stream);

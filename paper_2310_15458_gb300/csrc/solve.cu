@@ -496,8 +496,10 @@ cudaError_t launch_tw(const Batch& b, const SliceRec* sl, T* x, int64_t ldx, int
 // others.  may_build: the
 // caller allows the one-time allocation of a real factor's digits (rss_solve_noalloc
 // does not; it uses them only when they already exist, and cuts them per call else).
+// large: the products in classes of many boxes only.
 template <typename T>
-rss_status sweeps_tc(const rss_factorization* f, T* x, int64_t ldx, int nrhs, cudaStream_t st, void* ws, bool may_build) {
+rss_status sweeps_tc(const rss_factorization* f, T* x, int64_t ldx, int nrhs, cudaStream_t st, void* ws, bool may_build,
+                     bool large) {
   constexpr int RC = 8;
   constexpr bool real = sizeof(T) == sizeof(double);
   bool sl = real && nrhs >= TCB;
@@ -512,6 +514,9 @@ rss_status sweeps_tc(const rss_factorization* f, T* x, int64_t ldx, int nrhs, cu
   T* topz = reinterpret_cast<T*>(static_cast<char*>(ws) + w.topz_off);
   int* err = reinterpret_cast<int*>(static_cast<char*>(ws) + w.bar_off + 2 * sizeof(unsigned));
   const int polls = wait_limit(f->params.wait_polls, TW_POLLS);
+  auto takes = [&](const Batch& b) {
+    return tw_takes(b, nrhs, real) && (!large || (long long)b.nrec * cdiv(nrhs, TCB) >= 152);
+  };
   auto product = [&](size_t bi, auto op) -> cudaError_t {
     constexpr int OP = decltype(op)::value;
     const Batch& b = f->batches[bi];
@@ -520,7 +525,7 @@ rss_status sweeps_tc(const rss_factorization* f, T* x, int64_t ldx, int nrhs, cu
     return launch_tw<T, OP, false>(b, nullptr, x, ldx, nrhs, err, polls, st);
   };
   for (size_t bi = 0; bi < f->batches.size(); ++bi) {
-    if (!tw_takes(f->batches[bi], nrhs, real)) {
+    if (!takes(f->batches[bi])) {
       const rss_status s = sweep_class<T, RC, true>(f->batches[bi], x, ldx, nrhs, st);
       if (s != RSS_OK) return s;
       continue;
@@ -531,7 +536,7 @@ rss_status sweeps_tc(const rss_factorization* f, T* x, int64_t ldx, int nrhs, cu
   const rss_status stp = top_apply<T, RC>(f, x, ldx, nrhs, st, topz);
   if (stp != RSS_OK) return stp;
   for (size_t bi = f->batches.size(); bi-- > 0;) {
-    if (!tw_takes(f->batches[bi], nrhs, real)) {
+    if (!takes(f->batches[bi])) {
       const rss_status s = sweep_class<T, RC, false>(f->batches[bi], x, ldx, nrhs, st);
       if (s != RSS_OK) return s;
       continue;
@@ -548,8 +553,9 @@ bool use_tc(const rss_factorization* f, int64_t nrhs) {
 
 template <typename T>
 rss_status run_sweeps(const rss_factorization* f, T* x, int64_t ldx, int64_t nrhs, cudaStream_t st, void* ws,
-                      bool may_build = true, bool fp64 = false) {
-  if (!fp64 && use_tc(f, nrhs)) return sweeps_tc<T>(f, x, ldx, (int)nrhs, st, ws, may_build);
+                      bool may_build = true, Sweeps how = Sweeps::by_columns) {
+  if (how != Sweeps::fp64 && use_tc(f, nrhs))
+    return sweeps_tc<T>(f, x, ldx, (int)nrhs, st, ws, may_build, how == Sweeps::large_classes);
   const int rc = rhs_chunk(nrhs);
   return rc == 1 ? sweeps<T, 1>(f, x, ldx, (int)nrhs, st, ws)
          : rc == 4 ? sweeps<T, 4>(f, x, ldx, (int)nrhs, st, ws)
@@ -559,7 +565,7 @@ rss_status run_sweeps(const rss_factorization* f, T* x, int64_t ldx, int64_t nrh
 }  // namespace
 
 template <typename T>
-rss_status solve_impl(const rss_factorization* f, T* b, int64_t nrhs, int64_t ldb, cudaStream_t st, bool fp64) {
+rss_status solve_impl(const rss_factorization* f, T* b, int64_t nrhs, int64_t ldb, cudaStream_t st, Sweeps how) {
   const int64_t N = f->n;
   const SweepWs w = sweep_ws<T>(f, nrhs, rhs_chunk(nrhs));
   const size_t xb = (sizeof(T) * (size_t)N * nrhs + 255) & ~size_t(255);
@@ -575,7 +581,7 @@ rss_status solve_impl(const rss_factorization* f, T* b, int64_t nrhs, int64_t ld
     rss_set_error("rss_solve: launch failed");
     s = RSS_ECUDA;
   }
-  if (s == RSS_OK) s = run_sweeps<T>(f, x, nrhs, nrhs, st, mem + xb, true, fp64);
+  if (s == RSS_OK) s = run_sweeps<T>(f, x, nrhs, nrhs, st, mem + xb, true, how);
   if (s == RSS_OK) {
     if (launch_pdl(k_perm_out<T>, dim3(grid), NT, 0, st, 1, b, ldb, x, N, (int)nrhs, f->d_user_to_tree, err) !=
         cudaSuccess) {
@@ -588,7 +594,7 @@ rss_status solve_impl(const rss_factorization* f, T* b, int64_t nrhs, int64_t ld
   return s;
 }
 
-template rss_status solve_impl<double>(const rss_factorization*, double*, int64_t, int64_t, cudaStream_t, bool);
+template rss_status solve_impl<double>(const rss_factorization*, double*, int64_t, int64_t, cudaStream_t, Sweeps);
 
 template <typename T> rss_status build_sweep_classes(rss_factorization* f, cudaStream_t st) {
   if (f->batches.empty()) return RSS_OK;
@@ -618,8 +624,14 @@ size_t solve_device_bytes(const rss_factorization* f, int64_t nrhs) {
                              : sweep_ws<double>(f, nrhs, rhs_chunk(nrhs)).bytes);
 }
 
-bool panel_in_fp64(const rss_factorization* f, int64_t cols, int64_t smallest) {
-  return smallest < TCN && (f->is_complex || cols < TCB);
+// Requests of TCN columns take the products alone, so also in a panel; smaller ones, whose
+// solves take the FP64 sweeps, do so in panels of TCB columns: on real factors in every
+// class, on complex ones in the classes whose products fill the GPU.  (Requests of one
+// column in panels of 64, Helmholtz 2048^2: 45 RHS/s, with FP64 sweeps in all classes 21;
+// 256^2: 1868 and 1329.)
+Sweeps panel_sweeps(const rss_factorization* f, int64_t cols, int64_t smallest) {
+  if (smallest >= TCN) return Sweeps::by_columns;
+  return cols < TCB ? Sweeps::fp64 : f->is_complex ? Sweeps::large_classes : Sweeps::by_columns;
 }
 
 size_t solve_cache_bytes(const rss_factorization* f, int64_t max_nrhs) {
@@ -630,7 +642,7 @@ rss_status prepare_solve_caches(const rss_factorization* f, int64_t max_nrhs, cu
   if (f->is_complex || max_nrhs < TCB || !use_tc(f, max_nrhs)) return RSS_OK;
   return ensure_slices(const_cast<rss_factorization*>(f), st);
 }
-template rss_status solve_impl<zd>(const rss_factorization*, zd*, int64_t, int64_t, cudaStream_t, bool);
+template rss_status solve_impl<zd>(const rss_factorization*, zd*, int64_t, int64_t, cudaStream_t, Sweeps);
 
 // ---------------------------------------------------------------------------
 // rss_solve_noalloc: the same sweeps as rss_solve, with the working copy of
@@ -782,8 +794,8 @@ extern "C" rss_status rss_tune_solve(rss_factorization* f, int64_t nrhs, void* s
         float t[3];
         for (int rep = -1; rep < 3 && s == RSS_OK; ++rep) {   // one untimed run first
           cudaEventRecord(e0, st);
-          s = f->is_complex ? solve_impl<zd>(f, static_cast<zd*>(b), nrhs, f->n, st, true)
-                            : solve_impl<double>(f, static_cast<double*>(b), nrhs, f->n, st, true);
+          s = f->is_complex ? solve_impl<zd>(f, static_cast<zd*>(b), nrhs, f->n, st, Sweeps::fp64)
+                            : solve_impl<double>(f, static_cast<double*>(b), nrhs, f->n, st, Sweeps::fp64);
           cudaEventRecord(e1, st);
           if (cudaEventSynchronize(e1) != cudaSuccess) s = RSS_ECUDA;
           if (rep >= 0 && s == RSS_OK) cudaEventElapsedTime(&t[rep], e0, e1);
