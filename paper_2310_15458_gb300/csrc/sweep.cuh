@@ -331,11 +331,14 @@ __global__ void __launch_bounds__(SW_NT) k_sweep_cl(const BoxRec<T>* __restrict_
 }
 
 // ------------------------------------------------------------------ one persistent launch per sweep
-// The sweeps as two cooperative launches: the CTAs walk the colour classes in
-// factor order (upward) or reverse order (downward), one box and RC columns per
-// CTA, and meet at a grid barrier between classes.  The same sums in the same
-// order as the launches per class.
-constexpr int SWP_NT = 128;
+// The sweeps as two cooperative launches of clusters of SW_QMAX CTAs: they walk the
+// colour classes in factor order (upward) or reverse order (downward) and meet at a grid
+// barrier between classes.  A class whose boxes have SW_QMAX slices of C, one too small to
+// fill the GPU, takes a cluster per box (and RC columns), the others a CTA per box.  The
+// same sums in the same order as the launches per class.  (One column, one CTA per box in
+// every class, then this: Laplace 64^2 1.20, 0.42 ms, 1024^2 11.7, 4.5; Helmholtz 256^2 13.3,
+// 2.3.)
+constexpr int SWP_NT = 256;
 
 // One colour class as the persistent sweeps see it (device array in factor order).
 template <typename T> struct SwpClass {
@@ -355,20 +358,39 @@ template <typename T> struct SwpArgs {
   int sm_cap;               // scalars of dynamic shared memory
 };
 
+// whether v holds in every CTA of the cluster: its CTAs leave the sweep together (one that
+// left alone would take the shared memory along that its peers write)
+__device__ inline bool cluster_all(bool v) {
+  __shared__ int s_v;
+  namespace cg = cooperative_groups;
+  if (threadIdx.x == 0) s_v = v;
+  cg::this_cluster().sync();
+  int all = 1;
+  for (int q = 0; q < SW_QMAX; ++q) all &= *cg::this_cluster().map_shared_rank(&s_v, q);
+  cg::this_cluster().sync();
+  return all != 0;
+}
+
 template <typename T, int RC, bool UP> __global__ void __launch_bounds__(SWP_NT) k_sweep(SwpArgs<T> a) {
   extern __shared__ __align__(16) unsigned char smraw[];
   T* sm = reinterpret_cast<T*>(smraw);
   const int nz = (a.nrhs + RC - 1) / RC;
   for (int step = 0; step < a.ncls; ++step) {
     const SwpClass<T> C = a.cls[UP ? step : a.ncls - 1 - step];
-    for (int it = blockIdx.x; it < C.nrec * nz; it += gridDim.x) {
-      const int q0 = (it / C.nrec) * RC;
+    const int Q = C.qc == SW_QMAX ? SW_QMAX : 1, rank = blockIdx.x % Q;
+    for (int it = blockIdx.x / Q; it < C.nrec * nz; it += gridDim.x / Q) {
+      const int q0 = (it / C.nrec) * RC, nq = min(RC, a.nrhs - q0);
       const BoxRec<T> R = C.recs[it % C.nrec];
       T* xq = a.x + q0;
-      if (UP) up_box<T, RC>(R, xq, a.ldx, min(RC, a.nrhs - q0), sm, a.sm_cap, 0, 1, false, SoloCta{});
-      else down_box<T, RC>(R, xq, a.ldx, min(RC, a.nrhs - q0), sm, a.sm_cap, 0, 1, C.qc, false, SoloCta{});
+      if (Q == 1) {
+        if (UP) up_box<T, RC>(R, xq, a.ldx, nq, sm, a.sm_cap, 0, 1, false, SoloCta{});
+        else down_box<T, RC>(R, xq, a.ldx, nq, sm, a.sm_cap, 0, 1, C.qc, false, SoloCta{});
+      } else {
+        if (UP) up_box<T, RC>(R, xq, a.ldx, nq, sm, a.sm_cap, rank, Q, false, ClusterCta{});
+        else down_box<T, RC>(R, xq, a.ldx, nq, sm, a.sm_cap, rank, Q, C.qc, false, ClusterCta{});
+      }
       __syncthreads();
     }
-    if (step + 1 < a.ncls && !grid_barrier(a.bar, a.polls, a.err)) return;
+    if (step + 1 < a.ncls && !cluster_all(grid_barrier(a.bar, a.polls, a.err))) return;
   }
 }
