@@ -369,7 +369,8 @@ rss_status sweeps(const rss_factorization* f, T* x, int64_t ldx, int nrhs, cudaS
 
 // The digits of a real factor's matrices for the tensor-core sweeps: built once per
 // factor by the first solve that needs them (on its stream, which it then waits for),
-// kept until the factor is freed.
+// kept until the factor is freed.  They take more than twice the matrices' bytes; where the
+// device has not that much left (RSS_ENOMEM), a solve cuts them per call.
 bool tw_fits(const Batch& b, bool real) { return tw_shape_fits(b.max_n, b.max_r, b.max_c, real); }
 // whether a class takes the tensor-core products in a call with nrhs right-hand sides
 // (real classes of at most four boxes of 129 to 192 points: FP64 below TCL; 128^2, eps
@@ -416,7 +417,13 @@ rss_status ensure_slices(rss_factorization* f, cudaStream_t st) {
   auto al = [](size_t b) { return (b + 255) & ~size_t(255); };
   const size_t total = slice_total(f);
   char* base = nullptr;
-  RSS_CUDA(pool_malloc(reinterpret_cast<void**>(&base), total, st));
+  const cudaError_t em = pool_malloc(reinterpret_cast<void**>(&base), total, st);
+  if (em == cudaErrorMemoryAllocation) {
+    cudaGetLastError();
+    rss_set_error("rss_solve: no device memory for the digits of the factor");
+    return RSS_ENOMEM;
+  }
+  RSS_CUDA(em);
   char* p = base;
   auto take = [&](size_t b) {
     char* q = p;
@@ -522,7 +529,8 @@ rss_status sweeps_tc(const rss_factorization* f, T* x, int64_t ldx, int nrhs, cu
   bool sl = real && nrhs >= TCB;
   if (sl && may_build) {
     const rss_status s = ensure_slices(const_cast<rss_factorization*>(f), st);
-    if (s != RSS_OK) return s;
+    if (s != RSS_OK && s != RSS_ENOMEM) return s;
+    sl = s == RSS_OK;   // (no memory for the digits: cut per call)
   } else if (sl) {
     std::lock_guard<std::mutex> lk(const_cast<rss_factorization*>(f)->slice_mu);
     sl = f->slices_ready;

@@ -60,3 +60,32 @@ def test_boxes_of_more_than_one_row_tile(P, kind, side, leaf, eps, nrhs):
         assert float(torch.linalg.vector_norm(x[j] - one) / torch.linalg.vector_norm(one)) <= 1e-12, j
     if fly is not None:
         assert float(torch.linalg.vector_norm(fly - x) / torch.linalg.vector_norm(x)) <= 1e-12
+
+
+def test_panel_without_memory_for_the_digits(P):
+    """A real panel of 64 columns on a device whose memory is nearly all taken: the digits
+    that the factor would keep do not fit, so they are cut per call (under the scales of a
+    CTA's share of a long sum, so not to the same bits); with memory again, the same solve
+    keeps them.  Both against one-column solves, as above."""
+    side = 256
+    f = P.rss_factor(P.rss_build_tree(W.grid_points(side), 64), eps=1e-6, h=1.0 / side)
+    b = torch.from_numpy(np.ascontiguousarray(W.gaussian_rhs(side * side, 64, False, 4).T)).cuda()
+    P.rss_solve(f, b[:15].clone().T)
+    torch.cuda.synchronize()
+    torch.cuda.empty_cache()
+    P.rss_trim_memory(0)
+    free = torch.cuda.mem_get_info()[0]
+    hold = torch.empty(max(0, free - (600 << 20)), dtype=torch.uint8, device="cuda")
+    x = P.rss_solve(f, b.clone().T).clone()
+    torch.cuda.synchronize()
+    del hold
+    torch.cuda.empty_cache()
+    P.rss_trim_memory(0)
+    free = torch.cuda.mem_get_info()[0]
+    y = P.rss_solve(f, b.clone().T)
+    torch.cuda.synchronize()
+    assert free - torch.cuda.mem_get_info()[0] > 600 << 20   # (the digits, now)
+    for j in (0, 31, 63):
+        one = P.rss_solve(f, b[j].clone())
+        for z in (x.T, y.T):
+            assert float(torch.linalg.vector_norm(z[j] - one) / torch.linalg.vector_norm(one)) <= 1e-12, j
