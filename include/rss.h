@@ -161,8 +161,15 @@ rss_status rss_factor(const rss_tree* tree, const rss_params* params, void* stre
  * (Section 2.5).  b may be device memory (the call is then asynchronous on
  * stream) or host memory (the library stages it through the device and
  * returns after the result is back).  Real factors take double, complex
- * factors interleaved complex double.  Calls on distinct streams may run
- * concurrently on the same factor (the factor is read only). */
+ * factors interleaved complex double.  Calls on distinct streams, and from several
+ * host threads, may run concurrently on the same factor (the factor is read only).
+ * With fewer than 16 columns (and always with schur_path 1) every column goes through
+ * the same FP64 sums whatever it is solved with.  With 16 or more, colour classes that
+ * fit take tensor-core products: rows and columns as 56-bit fixed point under
+ * power-of-two scales per stretch of 48 to 384 entries of a sum, multiplied and added
+ * exactly.  In norm the error is that of the FP64 sums; an entry below 2^-56 of the
+ * largest of its stretch counts as zero, and a column's result differs from that of its
+ * own solve by rounding. */
 rss_status rss_solve(const rss_factorization* f, void* b, int64_t nrhs, int64_t ldb, void* stream);
 
 /* rss_solve without any device allocation.  The paper has no counterpart:

@@ -11,7 +11,7 @@
 // issues the products.  Real boxes (n <= 128) keep the tile's digits in shared memory
 // over all columns, and the group sums of one pass of 32 columns are joined from one
 // half of tensor memory while the products of the next fill the other.  Complex rows
-// are cut again for each pass, hidden behind the products, which take twice as long.
+// are cut again for each pass.
 // A class of few boxes splits the passes over CTAs.
 //
 // Real: the same integers, so the same E and F^T, as the digits of whole rows and
@@ -20,8 +20,9 @@
 // of 16 to 256 points an error of 0.47 to 0.9 times that of 32 entries at a time
 // joined at 53 bits, and 0.3 to 0.9 times that of FP64.
 //
-// Bound by the products (about 80 clocks each, near the tensor peak) and the join of the
-// group sums (integer instructions).
+// Bound by latency: one CTA of 17 warps on an SM gathers rows of A, cuts and joins; in the
+// first leaf class (512^2 real, 256^2 complex) the schedulers issue in 28 to 29 % of their
+// cycles, the tensor pipe is busy for 9 to 10 % (70 clocks a product), ALU 26 to 29 %.
 // Panels of a factorization against products on mma.sync with the rows and columns cut
 // per 64-row CTA: Laplace 1024^2 34.3 -> 24.8 ms, Helmholtz 256^2 22.1 -> 9.3 ms (of which
 // cutting W 2.0 and 0.6); a coarse complex class of one or two boxes 530 -> 100 us.

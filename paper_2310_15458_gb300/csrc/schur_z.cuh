@@ -11,8 +11,9 @@
 // entries j >= i are formed, and stored to A_CC(j, i) as well; the row blocks with the
 // most tiles of every box start first (60.2 -> 59.5 ms at Helmholtz 256^2).
 //
-// Bound by the products (96 per tile at r = 48, 80 clocks each) and the join of the sums,
-// which cannot overlap (a tile's sums fill tensor memory); the FP64 arithmetic (a
+// Bound by the entries of A_CC (DRAM 39 % of its peak, warps waiting for global loads) and
+// the products (tensor pipe 32 %: 96 a tile at r = 48, about 70 clocks each); the join of
+// the sums cannot overlap them (a tile's sums fill tensor memory), the FP64 arithmetic (a
 // conversion and a subtraction take 32 clocks a warp) runs beside the next products.
 // One tile per CTA, staged by cp.async and never overlapped, took 10.9 ms a
 // factorization at Helmholtz 256^2 and 32 ms at Lippmann-Schwinger 512^2; now 7.6 ms and

@@ -83,10 +83,11 @@ __global__ void __launch_bounds__(NT) k_perm_out(T* __restrict__ b, int64_t ldb,
 #include "sweep_tc.cuh"
 
 // Right-hand sides from which a call takes the tensor-core sweeps.  16 complex columns at
-// 256^2: 7 ms against 15.8 in FP64; 16 real ones: 3.4 ms against 4.6 (with the classes
+// 256^2: 6.9 ms against 14.7 in FP64; 16 real ones: 3.2 ms against 4.1 (with the classes
 // of fewer than TCMIN boxes, where four launches of the products take longer than one of
 // the FP64 sweep, left to the latter; at 64^2 every class).  From TCB on a real factor
-// keeps its digits, which a first call builds, and all classes that fit take the products.
+// keeps its digits, which a first call builds, and the classes that fit take the products,
+// below TCL columns but the smallest (tw_takes).
 constexpr int TCN = 16, TCB = 32, TCL = 64, TCMIN = 16;
 
 // Top block: x_top <- A_top^{-1} x_top with the inverse formed at factor time.

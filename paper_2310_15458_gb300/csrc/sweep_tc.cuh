@@ -2,16 +2,18 @@
 // colour class two products up, y = W_F^T [b_S; b_R] into b_R and b_C -= E b_R, and
 // two down, z = y_R - F y_C into y_R and [y_S; y_R] = [y_S; 0] + W_E y_R (see
 // sweep.cuh), each a launch of one CTA per box, 128 rows of the matrix and TW_NC real
-// columns.  The products with W_F and W_E write what they read: of a box of more than 128
-// points the row tiles form a cluster and meet between the two (64 columns, FP64 sweeps
-// before, this after: Laplace 384^2, leaf 144 36.5 -> 6.5 ms, 512^2, leaf 256 112 -> 13.1;
-// Helmholtz 192^2, leaf 144 31.6 -> 9.1).  Rows of the matrix and columns of the right-hand sides are scaled by
-// powers of two over stretches of K (SX) and cut into eight signed 7-bit
-// digits; the slice products of equal weight u = p + q <= 7 are summed exactly in
-// FP32 in tensor memory over a stretch, gathered into one int64 per
-// output and added in FP64: the accuracy of an FP64 product.  A complex product is
-// the real one with K doubled, [A_re A_im] times [B_re; -B_im] and [B_im; B_re]: the
-// two column groups of a CTA are then the real and imaginary parts of 32 columns.
+// columns.  Rows of the matrix and columns of the right-hand sides are scaled by powers of
+// two over stretches of K (SX) and cut into eight signed 7-bit digits; the slice products
+// of equal weight u = p + q <= 7 are summed exactly in FP32 in tensor memory over a
+// stretch, gathered into one int64 per output and added in FP64: the accuracy of an FP64
+// product.  A complex product is the real one with K doubled, [A_re A_im] times
+// [B_re; -B_im] and [B_im; B_re]: the two column groups of a CTA are then the real and
+// imaginary parts of 32 columns.
+//
+// The products with W_F and W_E write what they read: of a box of more than 128 points the
+// row tiles form a cluster and meet between the two (64 columns, FP64 sweeps before, this
+// after: Laplace 384^2, leaf 144 36.5 -> 6.5 ms, 512^2, leaf 256 112 -> 13.1; Helmholtz
+// 192^2, leaf 144 31.6 -> 9.1).
 //
 // K is staged 32 at a time in two to four buffers, so the digits of one stage are cut
 // while the products of the others run; the down sweep's F y_C (K = c, up to thousands)
@@ -21,12 +23,13 @@
 // by the first call of 32 and more columns), which then come by bulk copies; with fewer
 // columns and for complex factors they are cut on the fly.
 //
-// Bound by the products (36 slice pairs for 54 bits: about 80 clocks an instruction,
-// close to the tensor peak) and the gathering of x in the large classes, by latency
-// (about 20 us a launch) in the coarse ones.  64 columns, against mma.sync products of
-// one CTA per box (real) and the FP64 sweeps (complex): Laplace 512^2 23.3 -> 9.2 ms,
-// Helmholtz 256^2 30.3 -> 11.9 ms; 16 columns, against the FP64 sweeps: 4.6 -> 3.4 ms
-// (Laplace 256^2).
+// Bound by latency: one CTA of 16 warps on an SM gathers x, cuts, meets at a block barrier
+// a stage and joins; in the leaf classes the tensor pipe is busy for 9 to 10 % of the time
+// (about 70 clocks a product), no other unit for more than 25 %; in the coarse classes a
+// launch takes about 20 us.  64 columns, against mma.sync products of one CTA per box
+// (real) and the FP64 sweeps (complex): Laplace 512^2 23.3 -> 9.2 ms, Helmholtz 256^2
+// 30.3 -> 11.9 ms; 16 columns, against the FP64 sweeps: 4.1 -> 3.2 ms (Laplace
+// 256^2).
 // Stages of K that share scales and sums (SX below; tw_stages).  Shorter stretches follow
 // the entries' range more closely and cost a gather each.  Errors of a panel against the
 // records applied in quadruple precision, and 64 columns' times:
